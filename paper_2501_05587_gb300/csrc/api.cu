@@ -209,9 +209,10 @@ popcorn_status check_kernel(const popcorn_kernel& kern, KernParams* kp) {
     }
 }
 
-// K = kappa(P P^T) on stream s.  FP32: CUDA-core tiles.  BF16 / BF16X3: tcgen05
-// tiles; their operand copies come from `ws`, and *err (device) reports a
-// timed-out wait inside the kernel.
+// K = kappa(P P^T) on stream s.  FP32: CUDA-core tiles, or tcgen05 tiles of the points split
+// into two FP16 parts where that is as exact (decided on the device).  BF16 / BF16X3: tcgen05
+// tiles.  Operand copies come from `ws`, and *err (device) reports a timed-out wait inside a
+// kernel.
 // packed: the build writes the block-packed upper triangle (symmetric pass only).
 popcorn_status build_kernel_matrix(const float* P, int n, int d, int64_t ldp, const KernParams& kp,
                                    int precision, void* K, int64_t ldk, int k_storage, float* kdiag, Workspace* ws,
@@ -224,8 +225,17 @@ popcorn_status build_kernel_matrix(const float* P, int n, int d, int64_t ldp, co
             POPCORN_TRY(ws->alloc(&rn, (size_t)n, "row norms"));
             POPCORN_TRY(ws->alloc(&maxr, 1, "largest row norm"));
         }
+        // The tensor-core split build's operands (kbuild_tc.cu).  Without room for them the
+        // CUDA-core build runs alone.
+        unsigned char* split = nullptr;
+        if (ws && err && k_storage == POPCORN_K_FP32 && kbuild_split_applies(n, d, kp.kind != POPCORN_GAUSSIAN) &&
+            ws->alloc(&split, kbuild_split_workspace(n, d), "split operands") != POPCORN_OK) {
+            split = nullptr;
+            g_err.clear();
+        }
         POPCORN_CUDA(launch_kbuild_simt(P, n, d, ldp, kp, K, ldk, k_storage, kdiag, s, launches, packed, full, rn,
-                                        maxr));
+                                        maxr, split, err, num_sms));
+        if (split) ws->release(split);
         return POPCORN_OK;
     }
     if (k_storage != POPCORN_K_FP32 && packed != kPackedSw128H)

@@ -423,30 +423,34 @@ __global__ void __launch_bounds__(256) kbuild_simt_kernel(const float* __restric
                                                           KernParams kp, TK* __restrict__ K, int64_t ldk,
                                                           float* __restrict__ kdiag, int T, int full,
                                                           const float* __restrict__ rn, const unsigned* maxr,
-                                                          float expand_coef, int dot_expands) {
+                                                          float expand_coef, int dot_expands, long long tiles) {
     __shared__ __align__(16) TileSmem sm;
     const bool expand = KIND == POPCORN_GAUSSIAN && expansion_applies(rn, maxr, expand_coef);
     if (expand && dot_expands) return;
-    if (expand)
-        kbuild_tile<kGaussExpand, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, (long long)blockIdx.x, sm,
-                                                     full, rn);
-    else
-        kbuild_tile<KIND, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, (long long)blockIdx.x, sm, full);
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        if (expand)
+            kbuild_tile<kGaussExpand, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full, rn);
+        else
+            kbuild_tile<KIND, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full);
+    }
 }
 
 // The dot-product kinds (linear, polynomial, the Gaussian by the norm expansion) on FP32 K:
 // 16 x 8 outputs a thread, 128 threads.  The Gaussian instance returns at once when the
-// expansion does not apply (the 256-thread kernel then forms coordinate differences).
+// expansion does not apply (the 256-thread kernel then forms coordinate differences), and
+// every instance when the tensor-core split build (kbuild_tc.cu) has taken the matrix.
 template <int KIND, int PACKED>
 __global__ void __launch_bounds__(128, 2) kbuild_dot_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
                                                             KernParams kp, float* __restrict__ K, int64_t ldk,
                                                             float* __restrict__ kdiag, int T, int full,
                                                             const float* __restrict__ rn, const unsigned* maxr,
-                                                            float expand_coef) {
+                                                            float expand_coef, const SplitState* __restrict__ split,
+                                                            long long tiles) {
     __shared__ __align__(16) TileSmem sm;
+    if (split && split->use) return;   // the tensor-core build has written K
     if (KIND == kGaussExpand && !expansion_applies(rn, maxr, expand_coef)) return;
-    kbuild_tile<KIND, float, false, PACKED, 16>(P, n, d, ldp, kp, K, ldk, kdiag, T, (long long)blockIdx.x, sm, full,
-                                                rn);
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x)
+        kbuild_tile<KIND, float, false, PACKED, 16>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full, rn);
 }
 
 // d <= KC: the depth loop is one slice, so no next slice is held in registers;
@@ -468,7 +472,8 @@ __global__ void __launch_bounds__(256, 2) kbuild_simt_small_kernel(const float* 
 
 template <typename TK, int PACKED>
 cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernParams kp, TK* K, int64_t ldk,
-                              float* kdiag, cudaStream_t s, int full, float* rn, unsigned* maxr, int* launches) {
+                              float* kdiag, cudaStream_t s, int full, float* rn, unsigned* maxr, int* launches,
+                              void* split_ws = nullptr, int* err = nullptr, int num_sms = 0) {
     const int T = (n + TILE - 1) / TILE;
     // Gaussian: row norms and their maximum first (the build then picks the distance form);
     // 4 sqrt(d) u gamma / sigma^2 bounds the expansion's error per unit of max_i r_i
@@ -486,6 +491,10 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
     const long long tiles = full ? (long long)T * T : (long long)T * (T + 1) / 2;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     dim3 grid((unsigned)tiles), block(256);
+    // d > KC: blocks walk the tiles in strides of a grid of at most 8 blocks an SM, so that a
+    // launch whose work another kernel took costs one short wave (images: 150,000 empty blocks
+    // took 0.23 ms) and tiles of equal cost still spread evenly
+    const dim3 wgrid((unsigned)(num_sms > 0 && tiles > 8ll * num_sms ? 8ll * num_sms : tiles));
     if (d <= KC) {
         switch (kp.kind) {
             case POPCORN_LINEAR:
@@ -507,40 +516,46 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
         // FP32 K, d > KC: the dot-product kinds on the 16 x 8 kernel; the Gaussian launches both
         // forms, and the one whose distance form does not apply returns at once
         dim3 dblock(128);
+        const SplitState* split = nullptr;
+        if (split_ws && (rn || kp.kind != POPCORN_GAUSSIAN)) {
+            const cudaError_t e = launch_kbuild_split(P, n, d, ldp, kp, K, ldk, kdiag, split_ws, rn, maxr, expand_coef,
+                                                      err, num_sms, s, launches, PACKED, full, &split);
+            if (e != cudaSuccess) return e;
+        }
         switch (kp.kind) {
             case POPCORN_LINEAR:
-                kbuild_dot_kernel<POPCORN_LINEAR, PACKED>
-                    <<<grid, dblock, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef);
+                kbuild_dot_kernel<POPCORN_LINEAR, PACKED><<<wgrid, dblock, 0, s>>>(
+                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles);
                 return cudaGetLastError();
             case POPCORN_POLYNOMIAL:
-                kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED>
-                    <<<grid, dblock, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef);
+                kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED><<<wgrid, dblock, 0, s>>>(
+                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles);
                 return cudaGetLastError();
             default:
                 if (rn) {
-                    kbuild_dot_kernel<kGaussExpand, PACKED>
-                        <<<grid, dblock, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef);
+                    kbuild_dot_kernel<kGaussExpand, PACKED><<<wgrid, dblock, 0, s>>>(
+                        P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles);
                     cudaError_t e = cudaGetLastError();
                     if (e != cudaSuccess) return e;
                     if (launches) ++*launches;
                 }
-                kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED>
-                    <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 1);
+                kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED><<<wgrid, block, 0, s>>>(
+                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 1, tiles);
                 return cudaGetLastError();
         }
     }
     switch (kp.kind) {
         case POPCORN_LINEAR:
             kbuild_simt_kernel<POPCORN_LINEAR, TK, PACKED>
-                <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0);
+                <<<wgrid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0, tiles);
             break;
         case POPCORN_POLYNOMIAL:
             kbuild_simt_kernel<POPCORN_POLYNOMIAL, TK, PACKED>
-                <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0);
+                <<<wgrid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0, tiles);
             break;
         default:
             kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED>
-                <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0);
+                <<<wgrid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0, tiles);
             break;
     }
     return cudaGetLastError();
@@ -592,15 +607,15 @@ cudaError_t launch_batched_kbuild_simt(const BatchInst* dI, const BatchPlan& bp,
 
 cudaError_t launch_kbuild_simt(const float* P, int n, int d, int64_t ldp, KernParams kp, void* K, int64_t ldk,
                                int k_storage, float* kdiag, cudaStream_t s, int* launches, int packed, int full,
-                               float* rn, unsigned* maxr) {
+                               float* rn, unsigned* maxr, void* split_ws, int* err, int num_sms) {
     if (launches) ++*launches;
     if (packed) {
         if (k_storage != POPCORN_K_FP32) return cudaErrorInvalidValue;
         if (packed == kPackedSw4)
             return launch_simt_typed<float, kPackedSw4>(P, n, d, ldp, kp, static_cast<float*>(K), ldk, kdiag, s, 0,
-                                                        rn, maxr, launches);
+                                                        rn, maxr, launches, split_ws, err, num_sms);
         return launch_simt_typed<float, kPackedSw16>(P, n, d, ldp, kp, static_cast<float*>(K), ldk, kdiag, s, 0, rn,
-                                                     maxr, launches);
+                                                     maxr, launches, split_ws, err, num_sms);
     }
     if (k_storage == POPCORN_K_FP16)
         return launch_simt_typed<__half, 0>(P, n, d, ldp, kp, static_cast<__half*>(K), ldk, kdiag, s, 0, rn, maxr,
@@ -609,7 +624,7 @@ cudaError_t launch_kbuild_simt(const float* P, int n, int d, int64_t ldp, KernPa
         return launch_simt_typed<__nv_bfloat16, 0>(P, n, d, ldp, kp, static_cast<__nv_bfloat16*>(K), ldk, kdiag, s, 0,
                                                    rn, maxr, launches);
     return launch_simt_typed<float, 0>(P, n, d, ldp, kp, static_cast<float*>(K), ldk, kdiag, s, full, rn, maxr,
-                                       launches);
+                                       launches, split_ws, err, num_sms);
 }
 
 }  // namespace popcorn

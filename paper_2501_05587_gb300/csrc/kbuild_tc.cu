@@ -2,28 +2,30 @@
 //
 // Sec. 3.2 forms B = P P^T with GEMM or SYRK and then applies the kernel
 // function elementwise (Gaussian through Eq. 12 from B and the row norms).
-// Here one persistent kernel walks the tiles (p, j) of the upper triangle,
-// where a tile is a pair of 128-row blocks (2p, 2p + 1) against one
-// 128-column block j >= 2p:
+// Here one persistent kernel walks the tiles (i, q) of the upper triangle,
+// where a tile is a 128-row block i against a pair of 128-column blocks
+// (2q, 2q + 1), 2q + 1 >= i:
 //
-//   warp 0  (one lane)  TMA loads, per 64-deep k-block, of the 256 rows of the
-//                       row pair and the 128 rows of the column block (128-byte
-//                       swizzle) into a ring of stages;
-//   warp 1  (one lane)  tcgen05.mma kind::f16 (BF16 x BF16 -> FP32, M = N = 128)
-//                       into the two 128-column TMEM accumulators of the tile
-//                       (double-buffered: 512 columns);
-//   warps 2-5           epilogue: tcgen05.ld the accumulators, apply kappa with
-//                       FP32 row norms, stage each 128 x 32 chunk and its
-//                       transpose in shared memory and TMA-store both into K --
-//                       or, for the block-packed upper triangle the symmetric
-//                       pass reads, bulk-copy the swizzled chunk alone to its
-//                       place in the packed tile (each value stored once).
+//   warp 0  (one lane)  TMA loads, per k-block, of the 128 rows of the row block
+//                       and the 256 rows of the column pair (swizzled) into a ring
+//                       of stages;
+//   warp 1  (one lane)  tcgen05.mma kind::f16 (M = 128, N = 256, FP32 accumulator
+//                       in TMEM), double-buffered (512 columns);
+//   warps 2-9           epilogue, one warpgroup a column block: tcgen05.ld the
+//                       accumulator, apply kappa with FP32 row norms, stage a chunk
+//                       and its transpose in shared memory and TMA-store both into
+//                       K -- or, for the block-packed upper triangle the symmetric
+//                       pass reads, bulk-copy the swizzled chunk alone to its place
+//                       in the packed tile (each value stored once).
 //
-// Why row pairs: an SM takes in about 36 bytes per clock from L2 whichever path
+// Why column pairs: an SM takes in about 36 bytes per clock from L2 whichever path
 // it uses (TMA, bulk copy, cp.async or vector loads), and a 128 x 128 tile moves
 // 32 KB per k-block for 4 MMAs -- three times what that allows at the MMA rate.
-// Sharing each column block between two row blocks cuts the bytes per MMA by a
-// quarter; block (2p + 1, 2p), below the diagonal, is computed and not stored.
+// Sharing each row block between two column blocks cuts the bytes per MMA by a
+// quarter, and one N = 256 MMA reads 12 KB of shared memory where two of N = 128
+// read 16 (at 128 bytes a clock those alone take 64 of an N = 128 MMA's 68 clocks,
+// before the operand ring's own writes): the images FP32 build 13.3 -> 11.8 ms.
+// Block (2q + 1, 2q), below the diagonal, is computed and not stored.
 //
 // Precision modes (operand matrix W, one row per point):
 //   BF16    W = bf16(P);  norms of the rounded rows, so the Gaussian distance
@@ -33,6 +35,25 @@
 //           hi.hi + hi.lo + lo.hi (~16 significant bits of the cross term that
 //           the Gaussian's cancellation needs) -- 2 d loaded instead of the 3 d
 //           a [hi|hi|lo] x [hi|lo|hi] GEMM would stream.
+//   FP32    (SPLIT) W = [hi | lo] in FP16 of the points times a power of two s:
+//           hi = fp16(s p), lo = fp16(s p - hi), which represent p to 2^-24 of itself
+//           (hi and lo carry 11 bits each and lo's sign one more; column-wise the
+//           error is below 2^-26 of the column's largest value, see split_decide_kernel).
+//           The products are exact in FP32, but the tensor core adds them with
+//           truncation: left in TMEM over a long row the sum drifts low by half an ulp an
+//           MMA (measured at d = 784 on uniform points: relative error 6.1e-6 against
+//           4.2e-7 for FP32 FMAs).  So a TMEM accumulator holds only 32 columns of the
+//           rows: the small products lo.lo, hi.lo, lo.hi first, then the two hi.hi MMAs, and
+//           the epilogue warps add each such chunk into FP32 registers (round to nearest, the
+//           last two away from zero: the truncations of a chunk pull it low by about 1.5 half
+//           ulps on average, which J = trace K - ... of tight clusters sees as a bias).
+//           lo.lo is below an ulp, but on the diagonal it is a sum of squares: left out, J =
+//           trace K - ... of tight clusters is off by ten times that.
+//           Images, n = 70,000, d = 784: 10.9 ms (64.7 on CUDA cores); the operand loads allow
+//           8.4 (36 bytes a clock an SM), the MMAs 6.7, and the epilogue's stores (about 2 ms)
+//           are not overlapped: the next tile's MMAs run two chunks ahead.  n = 20,001,
+//           d = 1,000: 6.87 -> 1.43 ms a call.
+//           Measured on those points: 7.8e-8 (and 5.0e-8 at d = 128, where FMAs give 1.6e-7).
 //
 // Every mbarrier wait is bounded (about 2 s by %globaltimer).  A wait that
 // runs out sets *err, raises a shared abort flag that ends every role's loop,
@@ -54,63 +75,93 @@ namespace {
 
 using namespace tc;
 
-__device__ __forceinline__ void epi_bar() { named_bar<128>(1); }   // the 4 epilogue warps
-constexpr uint32_t kIdesc = idesc_bf16(128, 128);
+constexpr uint32_t kIdescBf16 = idesc_bf16(128, 256);
+constexpr uint32_t kIdescF16 = idesc_f16(128, 256);
 
-constexpr int BM = 128, BK = 64;             // block rows / columns, bf16 depth per k-block
-constexpr int ROWS_BYTES = 2 * BM * BK * 2;  // 32 KB: 256 rows of one part (hi or lo)
-constexpr int COLS_BYTES = BM * BK * 2;      // 16 KB: 128 rows of one part
-constexpr int STG_BYTES = 128 * 32 * 4;      // one 128 x 32 FP32 staging chunk
-constexpr int NTHREADS = 192;                // 6 warps
-constexpr int MAX_STAGES = 4;
-constexpr int RING_BYTES = 192 * 1024;       // operand ring
-constexpr uint32_t kTmemCols = 512;          // 2 buffers x 2 row blocks x 128 columns
+constexpr int kModeBf16 = 0, kModeX3 = 1, kModeSplit = 2;
+constexpr int BM = 128;                      // block rows / columns
+// depth of a k-block, in 16-bit elements: a stage is 48 KB in every mode (SPLIT: also what a TMEM
+// accumulator holds before it is drained)
+constexpr int kbuild_dk(int mode) { return mode == kModeBf16 ? 64 : 32; }
+constexpr int STG_BYTES = 16 * 1024;         // staging of one epilogue warpgroup: a 128 x 32 FP32 chunk, a
+                                             // 128 x 64 half box, or a 128 x 16 chunk and its transpose
+constexpr int NTHREADS = 320;                // 10 warps
+constexpr int kStageBytes = 48 * 1024;       // a k-block of the row block and the column pair
+constexpr int kStages = 3;                   // operand ring
+constexpr int kStg = 2;                      // staging buffers per warpgroup
+constexpr int NBARS = 2 * kStages + 5;
+// shared memory: ring, staging of both warpgroups, their copies of the column norms, barriers
+constexpr int kOffStg = kStages * kStageBytes, kOffRj = kOffStg + 2 * kStg * STG_BYTES, kOffBar = kOffRj + 2 * BM * 4,
+              kOffMisc = kOffBar + NBARS * 8, kSmemBytes = kOffMisc + 16 + 1024;   // (slack: 1024-byte alignment)
+constexpr uint32_t kTmemCols = 512;          // 2 buffers x 256 columns
 
 struct TcArgs {
-    int n, T, T2, nkb;        // rows, 128-blocks, row pairs, 64-deep k-blocks per part
-    int dpad;                 // elements per part (W row = [hi | lo] for BF16X3)
-    int x3;                   // 1: BF16X3 (three products per k-step)
-    int stages, stage_bytes;  // ring: 48 KB (BF16) or 96 KB (BF16X3) stages
-    int nstg;                 // staging buffers per kind (2, or 1 when the ring needs the room)
-    int off_sd, off_st, off_rj, off_bar, off_misc;
-    long long tiles;          // sum_p (T - 2 p)
+    int n, T, T2, nkb;        // rows, 128-blocks, column pairs, k-blocks per part
+    int dpad;                 // elements per part (W row = [hi | lo] for BF16X3 and SPLIT)
+    long long tiles;          // places of the walk over the tiles (tile_coords)
+    float* K;                 // row-major square (SPLIT: the diagonal blocks are stored with plain stores)
+    int64_t ldk;
     float* Kp;                // block-packed K (tile (I, J), I <= J, at its row-by-row triangle index
                               // times 16384 floats, four 128 x 32 boxes; FP16 / BF16: times 32 KB,
                               // two 128 x 64 boxes), or null
     int full;                 // 1: every tile of the square (the GEMM form), each stored once; 0: the
                               // tiles on and above the diagonal (the SYRK form), stored with their
                               // transposes unless K is packed
-    int sw4;                  // packed layout kPackedSw4 (element c of row r at c ^ (r mod 32)): the
-                              // kernel's SW4 instance; else kPackedSw16 (the 128-byte swizzle)
     KernParams kp;
     const float* norms;       // row norms of the represented rows (Gaussian)
     float* kdiag;
+    const SplitState* split;  // SPLIT: the device's decision and scale
     int* err;
 };
 
-// tile t -> (row pair p, column block j): row pair p holds tiles j = 2p .. T-1 and
-// starts at off(p) = p T - p (p - 1); a binary search over p (no floating point).
-// The full schedule (every column block, the GEMM form) has row pair p at p T.
-__device__ __forceinline__ void pair_coords(long long t, int T, int T2, int full, int* p, int* j) {
+// tile t -> (row block i, column pair q); false for a place of the walk that holds no tile.  The
+// walk goes through bands of kBand row blocks, and in a band column pair by column pair, so that
+// the tiles in flight at a time (152) touch kBand row blocks and about 19 column pairs (20 MB of
+// W at d = 784): W is read from HBM once a band.  Row block by row block, it was read once a row
+// block: 64 GB at n = 70,000, as much HBM time as the whole build takes now (11.8 -> 10.9 ms;
+// BF16 4.96 -> 4.17).  Band b of the upper
+// triangle is the rectangle of its row blocks and the pairs from its first diagonal block on
+// (12 places of it lie below the diagonal), and starts at kBand (b T2 - (kBand / 4) b (b - 1)):
+// a binary search over b, no floating point.  The full schedule takes every pair.
+constexpr int kBand = 8;
+__device__ __forceinline__ bool tile_coords(long long t, int T, int T2, int full, int* i, int* q) {
+    int lo = 0;
+    long long off = 0;
     if (full) {
-        *p = (int)(t / T);
-        *j = (int)(t % T);
-        return;
+        lo = (int)(t / ((long long)kBand * T2));
+        off = (long long)lo * kBand * T2;
+    } else {
+        int hi = (T - 1) / kBand;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            const long long o = (long long)kBand * ((long long)mid * T2 - (long long)(kBand / 4) * mid * (mid - 1));
+            if (o <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        off = (long long)kBand * ((long long)lo * T2 - (long long)(kBand / 4) * lo * (lo - 1));
     }
-    int lo = 0, hi = T2 - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        const long long off = (long long)mid * T - (long long)mid * (mid - 1);
-        if (off <= t) lo = mid;
-        else hi = mid - 1;
-    }
-    *p = lo;
-    *j = 2 * lo + (int)(t - ((long long)lo * T - (long long)lo * (lo - 1)));
+    const int rows = min(kBand, T - kBand * lo);
+    const int r = (int)(t - off);
+    *i = kBand * lo + r % rows;
+    *q = (full ? 0 : kBand / 2 * lo) + r / rows;
+    return full || 2 * *q + 1 >= *i;
+}
+// The number of places of the walk.
+long long tile_count(int T, int T2, int full) {
+    if (full) return (long long)T * T2;
+    const long long b = (T - 1) / kBand;
+    return kBand * (b * T2 - (kBand / 4) * b * (b - 1)) + (T - kBand * b) * (T2 - kBand / 2 * b);
 }
 
+// The kernel kind is a template parameter: with a runtime branch an element, the epilogue's
+// 128 elements a thread ran one after the other (about 300 clocks each, no overlap between
+// their chains), and it, not the MMAs, bounded every Gaussian build (images: 18.2 ms for
+// BF16 and BF16X3 alike; 4.9 and 7.9 ms with the kind a parameter and two epilogue
+// warpgroups, 4.2 and 7.8 now).
+template <int KIND>
 __device__ __forceinline__ float kappa(float b, float ri, float rj, const KernParams& kp) {
-    if (kp.kind == POPCORN_LINEAR) return b;
-    if (kp.kind == POPCORN_POLYNOMIAL) {
+    if constexpr (KIND == POPCORN_LINEAR) return b;
+    if constexpr (KIND == POPCORN_POLYNOMIAL) {
         const float base = fmaf(kp.gamma, b, kp.coef0);
         float r = base;
         for (int e = 1; e < kp.degree; ++e) r *= base;
@@ -119,13 +170,36 @@ __device__ __forceinline__ float kappa(float b, float ri, float rj, const KernPa
     const float d2 = fmaxf(fmaf(-2.f, b, ri + rj), 0.f);
     return expf(kp.neg_gamma_over_sigma2 * d2);
 }
+// kappa over a 32-element chunk: the polynomial's degree loop outside the elements, for the
+// same reason.
+template <int KIND>
+__device__ __forceinline__ void kappa32(float (&v)[32], float ri, const float* rj, const KernParams& kp) {
+    if constexpr (KIND == POPCORN_POLYNOMIAL) {
+        float base[32];
+#pragma unroll
+        for (int x = 0; x < 32; ++x) v[x] = base[x] = fmaf(kp.gamma, v[x], kp.coef0);
+        for (int e = 1; e < kp.degree; ++e) {
+#pragma unroll
+            for (int x = 0; x < 32; ++x) v[x] *= base[x];
+        }
+    } else if constexpr (KIND == POPCORN_GAUSSIAN) {
+#pragma unroll
+        for (int x = 0; x < 32; x += 4) {
+            const float4 r = *reinterpret_cast<const float4*>(rj + x);
+            v[x] = kappa<KIND>(v[x], ri, r.x, kp);
+            v[x + 1] = kappa<KIND>(v[x + 1], ri, r.y, kp);
+            v[x + 2] = kappa<KIND>(v[x + 2], ri, r.z, kp);
+            v[x + 3] = kappa<KIND>(v[x + 3], ri, r.w, kp);
+        }
+    }
+}
 
 // Output of the epilogue, one instance each, since a runtime choice between staging stores
-// slowed the epilogue about 2.8x: kOutSw16 (full square through tensor maps, or the packed
-// triangle in the 128-byte swizzle), kOutSw4 (packed XOR-32, kPackedSw4), kOutHalf16 /
-// kOutHalfB16 (packed FP16 / BF16 triangle, kPackedSw128H: each 64-column box is staged
-// whole -- two 32-column chunks -- and stored with one bulk copy; entries past n are zeros).
-constexpr int kOutSw16 = 0, kOutSw4 = 1, kOutHalf16 = 2, kOutHalfB16 = 3;
+// slowed the epilogue about 2.8x: kOutFull (full square through tensor maps), kOutSw16 /
+// kOutSw4 (the packed triangle in that layout), kOutHalf16 / kOutHalfB16 (packed FP16 / BF16
+// triangle, kPackedSw128H: each 64-column box is staged whole -- two 32-column chunks -- and
+// stored with one bulk copy; entries past n are zeros).
+constexpr int kOutFull = 0, kOutSw16 = 1, kOutSw4 = 2, kOutHalf16 = 3, kOutHalfB16 = 4;
 
 __device__ __forceinline__ uint32_t pack_half2(float x, float y, bool bf16) {
     if (bf16) {
@@ -139,25 +213,168 @@ __device__ __forceinline__ float round_half(float x, bool bf16) {
     return bf16 ? __bfloat162float(__float2bfloat16_rn(x)) : __half2float(__float2half_rn(x));
 }
 
+// What the epilogue of one 128 x 128 block knows.
+struct BlockCtx {
+    int rb, j;                 // row block, column block
+    int row_local, row;        // this thread's row
+    int et;                    // thread within the warpgroup
+    int bar;                   // the warpgroup's named barrier
+    unsigned char* stg;        // the warpgroup's staging
+    bool diag;
+};
+
+// Elements [32 c, 32 c + 32) of this thread's row of a block, kappa applied: staged and stored.
+// ctr counts the staging fills of the warpgroup.
 template <int OUT>
+__device__ __forceinline__ void store_chunk(const TcArgs& a, const BlockCtx& b, const CUtensorMap* map_kd,
+                                            const CUtensorMap* map_kt, int c, float (&v)[32], int& ctr) {
+    auto begin = [&]() -> unsigned char* {   // the store that last used this buffer has read it
+        unsigned char* sb = b.stg + (ctr & 1) * STG_BYTES;
+        ++ctr;
+        if (b.et == 0) bulk_wait_read<kStg - 1>();
+        named_bar<128>(b.bar);
+        return sb;
+    };
+    const long long tri = (long long)b.rb * a.T - (long long)b.rb * (b.rb - 1) / 2 + (b.j - b.rb);
+    if constexpr (OUT == kOutHalf16 || OUT == kOutHalfB16) {
+        constexpr bool HB16 = OUT == kOutHalfB16;
+        // box c / 2 of the half tile: staged over two chunks, stored after the second
+        unsigned char* sb;
+        if ((c & 1) == 0) sb = begin();
+        else sb = b.stg + ((ctr - 1) & 1) * STG_BYTES;
+        const int col0 = b.j * BM + 32 * c;
+        const bool rv = b.row < a.n;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            // logical 16-byte chunk 4 (c mod 2) + i of the row, at its swizzled place
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int x = 8 * i + 2 * e;
+                const float x0 = (rv && col0 + x < a.n) ? v[x] : 0.f;
+                const float x1 = (rv && col0 + x + 1 < a.n) ? v[x + 1] : 0.f;
+                w[e] = pack_half2(x0, x1, HB16);
+            }
+            const int pc = (4 * (c & 1) + i) ^ (b.row_local & 7);
+            *reinterpret_cast<uint4*>(sb + b.row_local * 128 + 16 * pc) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        if (c & 1) {
+            fence_proxy_async();
+            named_bar<128>(b.bar);
+            if (b.et == 0) {
+                bulk_store_1d(reinterpret_cast<unsigned char*>(a.Kp) + tri * 32768 + (c >> 1) * 16384, smem_u32(sb),
+                              (uint32_t)STG_BYTES);
+                bulk_commit();
+            }
+        }
+    } else if constexpr (OUT == kOutSw4 || OUT == kOutSw16) {
+        // the staged chunk is box c of packed tile (rb, j), byte for byte
+        float* sd = reinterpret_cast<float*>(begin());
+        if constexpr (OUT == kOutSw4) {
+            // element x of row row_local at x ^ (row_local mod 32) (the 32 lanes hold 32
+            // consecutive rows: 32 different banks per store)
+#pragma unroll
+            for (int x = 0; x < 32; ++x) sd[b.row_local * 32 + (x ^ (b.row_local & 31))] = v[x];
+        } else {
+            // 16-byte piece i of the row at i ^ (row % 8)
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<float4*>(sd + b.row_local * 32 + ((i ^ (b.row_local & 7)) * 4)) =
+                    make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+        fence_proxy_async();
+        named_bar<128>(b.bar);
+        if (b.et == 0) {
+            bulk_store_1d(a.Kp + tri * (BM * BM) + c * (BM * 32), smem_u32(sd), (uint32_t)STG_BYTES);
+            bulk_commit();
+        }
+    } else {
+        const bool transpose = !b.diag && !a.full;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            // 16 columns: the direct chunk in the 64-byte swizzle (16-byte piece i of a row at
+            // i ^ ((row / 2) mod 4)), then the transpose, 16 rows of 128
+            float* sd = reinterpret_cast<float*>(begin());
+            float* sx = sd + BM * 16;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                *reinterpret_cast<float4*>(sd + b.row_local * 16 + ((i ^ ((b.row_local >> 1) & 3)) * 4)) =
+                    make_float4(v[16 * half + 4 * i], v[16 * half + 4 * i + 1], v[16 * half + 4 * i + 2],
+                                v[16 * half + 4 * i + 3]);
+            if (transpose) {
+#pragma unroll
+                for (int x = 0; x < 16; ++x) sx[x * BM + b.row_local] = v[16 * half + x];
+            }
+            fence_proxy_async();
+            named_bar<128>(b.bar);
+            if (b.et == 0) {
+                const int col = b.j * BM + 32 * c + 16 * half;
+                if (col < a.n) {
+                    tma_store_2d(map_kd, col, b.rb * BM, smem_u32(sd));
+                    if (transpose) tma_store_2d(map_kt, b.rb * BM, col, smem_u32(sx));
+                }
+                bulk_commit();
+            }
+        }
+    }
+}
+
+// SPLIT, a diagonal block: hi.lo and lo.hi reach element (r, c) in the opposite order of
+// (c, r), so the elements on and above the diagonal are stored to both places (`below`: those
+// on and below it, in a tile whose MMAs ran in the order of the blocks below the diagonal).
+template <int OUT>
+__device__ __forceinline__ void store_diag_chunk(const TcArgs& a, const BlockCtx& b, bool below, int c,
+                                                 const float (&v)[32]) {
+    const int r = b.row_local;
+    float* tile = nullptr;
+    if constexpr (OUT != kOutFull)
+        tile = a.Kp + ((long long)b.rb * a.T - (long long)b.rb * (b.rb - 1) / 2) * (BM * BM);
+    auto put = [&](int i, int l, float x) {
+        if constexpr (OUT == kOutFull) {
+            const int gi = b.rb * BM + i, gl = b.rb * BM + l;
+            if (gi < a.n && gl < a.n) a.K[(int64_t)gi * a.ldk + gl] = x;
+        } else if constexpr (OUT == kOutSw4) {
+            tile[(l >> 5) * (BM * 32) + i * 32 + ((l & 31) ^ (i & 31))] = x;
+        } else {
+            tile[(l >> 5) * (BM * 32) + i * 32 + ((((l & 31) >> 2) ^ (i & 7)) << 2) + (l & 3)] = x;
+        }
+    };
+#pragma unroll
+    for (int x = 0; x < 32; ++x) {
+        const int l = 32 * c + x;
+        if (l == r || (l > r) != below) {
+            put(r, l, v[x]);
+            if (l != r) put(l, r, v[x]);
+        }
+    }
+}
+
+// a + b rounded away from zero (an exact sum stays exact).
+__device__ __forceinline__ float add_away(float a, float b) {
+    const float up = __fadd_ru(a, b), dn = __fadd_rd(a, b);
+    return fabsf(up) >= fabsf(dn) ? up : dn;
+}
+
+template <int MODE, int OUT, int KIND>
 __global__ void __launch_bounds__(NTHREADS, 1)
     kbuild_tc_kernel(const __grid_constant__ CUtensorMap map_r, const __grid_constant__ CUtensorMap map_c,
                      const __grid_constant__ CUtensorMap map_kd, const __grid_constant__ CUtensorMap map_kt,
                      TcArgs a) {
+    constexpr bool SPLIT = MODE == kModeSplit, X3 = MODE != kModeBf16;
+    if (SPLIT && !a.split->use) return;   // the CUDA-core build takes this matrix
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar0 = sbase + a.off_bar;
-    const int S = a.stages;
+    const uint32_t bar0 = sbase + kOffBar;
+    constexpr int S = kStages;
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
-    auto accf_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + b); };
-    auto acce_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + 2 + b); };
-    const uint32_t down_bar = bar0 + 8u * (2 * MAX_STAGES + 4);
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + a.off_misc);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + a.off_misc + 4);
-    float* rj_s = reinterpret_cast<float*>(smem + a.off_rj);
+    auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
+    auto accf_bar = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
+    auto acce_bar = [&](int b) { return bar0 + 8u * (2 * kStages + 2 + b); };
+    const uint32_t down_bar = bar0 + 8u * (2 * kStages + 4);
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 4);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -166,7 +383,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(accf_bar(b), 1);
-            mbar_init(acce_bar(b), 4);
+            mbar_init(acce_bar(b), 8);
         }
         mbar_init(down_bar, 1);
         *abort_flag = 0;
@@ -184,34 +401,35 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // stage layout: rows-hi (32 KB) | cols-hi (16 KB) [| rows-lo (32 KB) | cols-lo (16 KB)]
-    constexpr uint32_t kRowsHi = 0, kColsHi = ROWS_BYTES, kRowsLo = ROWS_BYTES + COLS_BYTES,
-                       kColsLo = 2 * ROWS_BYTES + COLS_BYTES;
+    // stage layout: cols-hi (256 rows of W) | rows-hi (128 rows) [| cols-lo | rows-lo], rows of DK elements
+    constexpr int DK = kbuild_dk(MODE);
+    constexpr uint32_t kBlock = BM * DK * 2;   // 128 rows of one part
+    constexpr uint32_t kColsHi = 0, kRowsHi = 2 * kBlock, kColsLo = 3 * kBlock, kRowsLo = 5 * kBlock;
     const long long G = gridDim.x;
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- TMA producer ----------------
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t issued_parity[MAX_STAGES];
-            bool issued[MAX_STAGES];
-            for (int s = 0; s < MAX_STAGES; ++s) issued[s] = false;
+            uint32_t issued_parity[kStages];
+            bool issued[kStages];
+            for (int s = 0; s < kStages; ++s) issued[s] = false;
             bool ok = true;
             for (long long t = blockIdx.x; t < a.tiles && ok; t += G) {
-                int p, j;
-                pair_coords(t, a.T, a.T2, a.full, &p, &j);
+                int i, q;
+                if (!tile_coords(t, a.T, a.T2, a.full, &i, &q)) continue;
                 for (int kb = 0; kb < a.nkb; ++kb) {
                     if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, a.err)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t st = sbase + (uint32_t)(stage * a.stage_bytes);
-                    mbar_arrive_expect_tx(full_bar(stage), (uint32_t)a.stage_bytes);
-                    tma_load_2d(st + kRowsHi, &map_r, kb * BK, p * 2 * BM, full_bar(stage));
-                    tma_load_2d(st + kColsHi, &map_c, kb * BK, j * BM, full_bar(stage));
-                    if (a.x3) {
-                        tma_load_2d(st + kRowsLo, &map_r, a.dpad + kb * BK, p * 2 * BM, full_bar(stage));
-                        tma_load_2d(st + kColsLo, &map_c, a.dpad + kb * BK, j * BM, full_bar(stage));
+                    const uint32_t st = sbase + (uint32_t)(stage * kStageBytes);
+                    mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kStageBytes);
+                    tma_load_2d(st + kColsHi, &map_c, kb * DK, q * 2 * BM, full_bar(stage));
+                    tma_load_2d(st + kRowsHi, &map_r, kb * DK, i * BM, full_bar(stage));
+                    if constexpr (X3) {
+                        tma_load_2d(st + kColsLo, &map_c, a.dpad + kb * DK, q * 2 * BM, full_bar(stage));
+                        tma_load_2d(st + kRowsLo, &map_r, a.dpad + kb * DK, i * BM, full_bar(stage));
                     }
                     issued[stage] = true;
                     issued_parity[stage] = phase;
@@ -236,35 +454,65 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // ---------------- MMA issuer ----------------
             int stage = 0;
             uint32_t phase = 0;
-            int lt = 0;
+            int fill = 0;   // accumulator fills: a tile, or (SPLIT) a 32-deep chunk
             bool ok = true;
-            for (long long t = blockIdx.x; t < a.tiles && ok; t += G, ++lt) {
-                const int ab = lt & 1;
-                const uint32_t use = (uint32_t)(lt >> 1);
-                if (!mbar_wait(acce_bar(ab), (use & 1u) ^ 1u, abort_flag, a.err)) {
-                    ok = false;
-                    break;
-                }
+            const uint64_t desc0 = DK == 32 ? sw64_desc(sbase) : sw128_desc(sbase);
+            // both halves of the next buffer have been read by the epilogue
+            auto take_buffer = [&](int ab, uint32_t use) {
+                if (!mbar_wait(acce_bar(ab), (use & 1u) ^ 1u, abort_flag, a.err)) return false;
                 tc_fence_after();
-                for (int kb = 0; kb < a.nkb; ++kb) {
+                return true;
+            };
+            for (long long t = blockIdx.x; t < a.tiles && ok; t += G) {
+                bool below = false;   // SPLIT: the tile holds a block below the diagonal
+                int i, q;
+                if (!tile_coords(t, a.T, a.T2, a.full, &i, &q)) continue;
+                if (SPLIT && a.full) below = 2 * q < i;
+                if (!SPLIT && !take_buffer(fill & 1, (uint32_t)(fill >> 1))) break;
+                for (int kb = 0; kb < a.nkb && ok; ++kb) {
                     if (!mbar_wait(full_bar(stage), phase, abort_flag, a.err)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t st = sbase + (uint32_t)(stage * a.stage_bytes);
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t d_tmem = tmem + (uint32_t)(ab * 2 * BM + h * BM);
-                        const uint32_t rh = st + kRowsHi + h * (BM * BK * 2);   // row block h of the pair
-                        const uint32_t rl = st + kRowsLo + h * (BM * BK * 2);
+                    const uint32_t st = sbase + (uint32_t)(stage * kStageBytes);
+                    // 16 elements = 32 bytes further along K inside the swizzled row.  Descriptors are
+                    // advanced by adds: the 14-bit address field never carries.
+                    if constexpr (SPLIT) {
+                        const int ab = fill & 1;
+                        if (!take_buffer(ab, (uint32_t)(fill >> 1))) {
+                            ok = false;
+                            break;
+                        }
+                        ++fill;
+                        const uint64_t sd = desc0 + (uint64_t)(uint32_t)(stage * (kStageBytes >> 4));
+                        const uint64_t rh = sd + (kRowsHi >> 4), rl = sd + (kRowsLo >> 4);
+                        const uint64_t ch = sd + (kColsHi >> 4), cl = sd + (kColsLo >> 4);
+                        const uint32_t d_tmem = tmem + (uint32_t)(ab * 2 * BM);
+                        // the small products first; hi.lo and lo.hi in the order of the
+                        // transposed block below the diagonal (full schedule): K stays symmetric
+                        const uint64_t r1 = below ? rl : rh, c1 = below ? ch : cl;
+                        const uint64_t r2 = below ? rh : rl, c2 = below ? cl : ch;
+                        mma_bf16(d_tmem, rl, cl, kIdescF16, 0u);
+                        mma_bf16(d_tmem, rl + 2, cl + 2, kIdescF16, 1u);
+                        mma_bf16(d_tmem, r1, c1, kIdescF16, 1u);
+                        mma_bf16(d_tmem, r2, c2, kIdescF16, 1u);
+                        mma_bf16(d_tmem, r1 + 2, c1 + 2, kIdescF16, 1u);
+                        mma_bf16(d_tmem, r2 + 2, c2 + 2, kIdescF16, 1u);
+                        mma_bf16(d_tmem, rh, ch, kIdescF16, 1u);
+                        mma_bf16(d_tmem, rh + 2, ch + 2, kIdescF16, 1u);
+                        mma_commit(accf_bar(ab));
+                    } else {
+                        const uint64_t sd = desc0 + (uint64_t)(uint32_t)(stage * (kStageBytes >> 4));
+                        const uint64_t rh = sd + (kRowsHi >> 4), rl = sd + (kRowsLo >> 4);
+                        const uint64_t ch = sd + (kColsHi >> 4), cl = sd + (kColsLo >> 4);
+                        const uint32_t d_tmem = tmem + (uint32_t)((fill & 1) * 2 * BM);
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            // 16 bf16 = 32 bytes further along K inside the 128-byte swizzled row
-                            mma_bf16(d_tmem, sw128_desc(rh + kk * 32), sw128_desc(st + kColsHi + kk * 32), kIdesc,
-                                     (kb | kk) ? 1u : 0u);
-                            if (a.x3) {
-                                mma_bf16(d_tmem, sw128_desc(rh + kk * 32), sw128_desc(st + kColsLo + kk * 32), kIdesc, 1u);
-                                mma_bf16(d_tmem, sw128_desc(rl + kk * 32), sw128_desc(st + kColsHi + kk * 32), kIdesc, 1u);
+                        for (int kk = 0; kk < DK / 16; ++kk) {
+                            mma_bf16(d_tmem, rh + 2 * kk, ch + 2 * kk, kIdescBf16, (kb | kk) ? 1u : 0u);
+                            if constexpr (X3) {
+                                mma_bf16(d_tmem, rh + 2 * kk, cl + 2 * kk, kIdescBf16, 1u);
+                                mma_bf16(d_tmem, rl + 2 * kk, ch + 2 * kk, kIdescBf16, 1u);
                             }
                         }
                     }
@@ -275,7 +523,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     }
                 }
                 if (!ok) break;
-                mma_commit(accf_bar(ab));           // both accumulators ready for the epilogue
+                if (!SPLIT) {
+                    mma_commit(accf_bar(fill & 1));   // ready for the epilogue
+                    ++fill;
+                }
             }
             // all MMAs issued by this thread complete before TMEM is released
             mma_commit(down_bar);
@@ -284,145 +535,120 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
         }
     } else {
-        // ---------------- epilogue: warps 2..5, TMEM lanes 32 * (warp % 4) ----------------
+        // ---------------- epilogue: warpgroup h takes column block h, TMEM lanes 32 * (warp % 4) ----------------
+        const int h = (warp - 2) >> 2;
         const int q = warp & 3;
-        const int et = threadIdx.x - 64;          // 0..127 within the epilogue group
-        int lt = 0;
-        int chunk_ctr = 0;
-        bool ok = true;
-        for (long long t = blockIdx.x; t < a.tiles; t += G, ++lt) {
-            int p, j;
-            pair_coords(t, a.T, a.T2, a.full, &p, &j);
-            const int ab = lt & 1;
-            const uint32_t use = (uint32_t)(lt >> 1);
-            // column norms of this tile's column block j
-            if (a.kp.kind == POPCORN_GAUSSIAN) {
-                const int col = j * BM + et;
-                epi_bar();   // previous tile finished reading rj_s
-                rj_s[et] = col < a.n ? a.norms[col] : 0.f;
+        BlockCtx b;
+        b.et = threadIdx.x - 64 - 128 * h;
+        b.bar = 1 + h;
+        b.stg = smem + kOffStg + h * kStg * STG_BYTES;
+        b.row_local = 32 * q + lane;
+        float* rj_s = reinterpret_cast<float*>(smem + kOffRj) + h * BM;
+        const uint32_t tlane = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(h * BM);
+        const float unscale = SPLIT ? a.split->unscale : 1.f;
+        int fill = 0, ctr = 0;
+        for (long long t = blockIdx.x; t < a.tiles; t += G) {
+            int pair;
+            if (!tile_coords(t, a.T, a.T2, a.full, &b.rb, &pair)) continue;
+            b.j = 2 * pair + h;           // 128-column block of K
+            b.row = b.rb * BM + b.row_local;
+            b.diag = b.rb == b.j;
+            // blocks past the matrix and block (2q + 1, 2q) below the diagonal are not stored
+            const bool store = b.rb < a.T && b.j < a.T && (a.full || b.rb <= b.j);
+            const float ri = (KIND == POPCORN_GAUSSIAN && b.row < a.n) ? a.norms[b.row] : 0.f;
+            if (KIND == POPCORN_GAUSSIAN) {   // column norms of this tile's column block j
+                const int col = b.j * BM + b.et;
+                named_bar<128>(b.bar);   // the warpgroup finished reading the previous tile's
+                rj_s[b.et] = col < a.n ? a.norms[col] : 0.f;
+                named_bar<128>(b.bar);
             }
-            if (!mbar_wait(accf_bar(ab), use & 1u, abort_flag, a.err)) ok = false;
-            // all epilogue threads agree (one barrier, one AND) before touching TMEM or staging
-            if (!named_bar_all(1, 128, ok && !*abort_flag)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const int row_local = 32 * q + lane;
-            for (int h = 0; h < 2; ++h) {
-                const int rb = 2 * p + h;             // 128-row block of K
-                const int row = rb * BM + row_local;
-                const float ri = (a.kp.kind == POPCORN_GAUSSIAN && row < a.n) ? a.norms[row] : 0.f;
-                // blocks past the matrix and block (2p + 1, 2p) below the diagonal are not stored
-                const bool store = rb < a.T && (a.full || rb <= j);
-                const bool diag = (rb == j);
+            constexpr bool HALF = OUT == kOutHalf16 || OUT == kOutHalfB16;
+            auto finish = [&](int c, float (&v)[32]) {
+                kappa32<KIND>(v, ri, rj_s + 32 * c, a.kp);
+                if (b.diag && (b.row_local >> 5) == c) {
+#pragma unroll
+                    for (int x = 0; x < 32; ++x)
+                        if (x == (b.row_local & 31)) {
+                            if (KIND == POPCORN_GAUSSIAN) v[x] = 1.f;
+                            if (b.row < a.n) a.kdiag[b.row] = HALF ? round_half(v[x], OUT == kOutHalfB16) : v[x];
+                        }
+                }
+                if (SPLIT && b.diag) store_diag_chunk<OUT>(a, b, a.full && 2 * pair < b.rb, c, v);
+                else store_chunk<OUT>(a, b, &map_kd, &map_kt, c, v, ctr);
+            };
+            bool ok = true;
+            if constexpr (SPLIT) {
+                // the row's 128 sums, as f32x2 pairs: one chunk of 32 columns of P at a time
+                unsigned long long acc[BM / 2];
+#pragma unroll
+                for (int x = 0; x < BM / 2; ++x) acc[x] = 0ull;
+                for (int kb = 0; kb < a.nkb; ++kb, ++fill) {
+                    const int ab = fill & 1;
+                    const bool got = mbar_wait(accf_bar(ab), (uint32_t)(fill >> 1) & 1u, abort_flag, a.err);
+                    if (__any_sync(0xffffffffu, !got)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t tacc = tlane + (uint32_t)(ab * 2 * BM);
+                    const bool last = kb + 2 >= a.nkb;   // the last two are rounded away from zero
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        uint32_t r[16];
+                        tmem_ld16(tacc + 16 * c, r);
+                        if (!last) {
+#pragma unroll
+                            for (int x = 0; x < 8; ++x)
+                                acc[8 * c + x] = f2add(acc[8 * c + x], f2pack(__uint_as_float(r[2 * x]),
+                                                                              __uint_as_float(r[2 * x + 1])));
+                        } else {
+#pragma unroll
+                            for (int x = 0; x < 8; ++x) {
+                                float a0, a1;
+                                f2unpack(acc[8 * c + x], a0, a1);
+                                acc[8 * c + x] = f2pack(add_away(a0, __uint_as_float(r[2 * x])),
+                                                        add_away(a1, __uint_as_float(r[2 * x + 1])));
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(acce_bar(ab));
+                }
+                // the warpgroup agrees (one barrier, one AND) before touching staging
+                if (!named_bar_all(b.bar, 128, ok && !*abort_flag)) break;
+                if (!store) continue;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float v[32];
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) {
+                        f2unpack(acc[16 * c + x], v[2 * x], v[2 * x + 1]);
+                        v[2 * x] *= unscale;
+                        v[2 * x + 1] *= unscale;
+                    }
+                    finish(c, v);
+                }
+            } else {
+                const int ab = fill & 1;
+                ok = mbar_wait(accf_bar(ab), (uint32_t)(fill >> 1) & 1u, abort_flag, a.err);
+                ++fill;
+                if (!named_bar_all(b.bar, 128, ok && !*abort_flag)) break;
+                tc_fence_after();
                 for (int c = 0; c < BM / 32; ++c) {
                     float v[32];
-                    tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(ab * 2 * BM + h * BM + 32 * c), v);
-                    if (h == 1 && c == BM / 32 - 1) {
-                        // both accumulators fully read: hand the buffer back to the MMA warp
+                    tmem_ld32(tlane + (uint32_t)(ab * 2 * BM + 32 * c), v);
+                    if (c == BM / 32 - 1) {
+                        // accumulator fully read: hand it back to the MMA warp
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(acce_bar(ab));
                     }
-                    if (!store) continue;
-                    constexpr bool HALF = OUT == kOutHalf16 || OUT == kOutHalfB16;
-                    constexpr bool HB16 = OUT == kOutHalfB16;
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) {
-                        v[x] = kappa(v[x], ri, rj_s[32 * c + x], a.kp);
-                        if (diag && 32 * c + x == row_local) {
-                            if (a.kp.kind == POPCORN_GAUSSIAN) v[x] = 1.f;
-                            if (row < a.n) a.kdiag[row] = HALF ? round_half(v[x], HB16) : v[x];
-                        }
-                    }
-                    if constexpr (HALF) {
-                        // box c / 2 of the half tile: staged over two chunks, stored after the second
-                        const int sbuf = a.nstg == 2 ? ((chunk_ctr >> 1) & 1) : 0;
-                        ++chunk_ctr;
-                        if ((c & 1) == 0) {
-                            // the store that last used this staging buffer has read it
-                            if (et == 0) {
-                                if (a.nstg == 2) bulk_wait_read<1>();
-                                else bulk_wait_read<0>();
-                            }
-                            epi_bar();
-                        }
-                        unsigned char* sb = smem + a.off_sd + sbuf * STG_BYTES;
-                        const int col0 = j * BM + 32 * c;
-                        const bool rv = row < a.n;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            // logical 16-byte chunk 4 (c mod 2) + i of the row, at its swizzled place
-                            uint32_t w[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int x = 8 * i + 2 * e;
-                                const float x0 = (rv && col0 + x < a.n) ? v[x] : 0.f;
-                                const float x1 = (rv && col0 + x + 1 < a.n) ? v[x + 1] : 0.f;
-                                w[e] = pack_half2(x0, x1, HB16);
-                            }
-                            const int pc = (4 * (c & 1) + i) ^ (row_local & 7);
-                            *reinterpret_cast<uint4*>(sb + row_local * 128 + 16 * pc) = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                        if (c & 1) {
-                            fence_proxy_async();
-                            epi_bar();
-                            if (et == 0) {
-                                const long long tri = (long long)rb * a.T - (long long)rb * (rb - 1) / 2 + (j - rb);
-                                bulk_store_1d(reinterpret_cast<unsigned char*>(a.Kp) + tri * 32768 + (c >> 1) * 16384,
-                                              smem_u32(sb), (uint32_t)STG_BYTES);
-                                bulk_commit();
-                            }
-                        }
-                        continue;
-                    }
-                    const int sbuf = a.nstg == 2 ? (chunk_ctr & 1) : 0;
-                    ++chunk_ctr;
-                    // the store that last used this staging buffer has read it
-                    if (et == 0) {
-                        if (a.nstg == 2) bulk_wait_read<1>();
-                        else bulk_wait_read<0>();
-                    }
-                    epi_bar();
-                    float* sd = reinterpret_cast<float*>(smem + a.off_sd + sbuf * STG_BYTES);
-                    float* sx = reinterpret_cast<float*>(smem + a.off_st + sbuf * STG_BYTES);
-                    if constexpr (OUT == kOutSw4) {
-                        // packed XOR-32 layout: element x of row row_local at x ^ (row_local mod 32)
-                        // (the 32 lanes hold 32 consecutive rows: 32 different banks per store)
-#pragma unroll
-                        for (int x = 0; x < 32; ++x) sd[row_local * 32 + (x ^ lane)] = v[x];
-                    } else {
-                        // direct chunk: row row_local, 8 x 16-byte pieces, piece i at i ^ (row % 8)
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            float4 w = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                            *reinterpret_cast<float4*>(sd + row_local * 32 + ((i ^ (row_local & 7)) * 4)) = w;
-                        }
-                    }
-                    const bool transpose = !diag && !a.Kp && !a.full;
-                    if (transpose) {
-#pragma unroll
-                        for (int x = 0; x < 32; ++x) sx[x * 128 + row_local] = v[x];
-                    }
-                    fence_proxy_async();
-                    epi_bar();
-                    if (et == 0) {
-                        if (a.Kp) {
-                            // the staged chunk is box c of packed tile (rb, j), byte for byte
-                            const long long tri = (long long)rb * a.T - (long long)rb * (rb - 1) / 2 + (j - rb);
-                            bulk_store_1d(a.Kp + tri * (BM * BM) + c * (BM * 32), smem_u32(sd), (uint32_t)STG_BYTES);
-                        } else {
-                            tma_store_2d(&map_kd, j * BM + 32 * c, rb * BM, smem_u32(sd));
-                            if (transpose) tma_store_2d(&map_kt, rb * BM, j * BM + 32 * c, smem_u32(sx));
-                        }
-                        bulk_commit();
-                    }
+                    if (store) finish(c, v);
                 }
             }
         }
-        if (et == 0) bulk_wait_all();
-        (void)ok;
+        if (b.et == 0) bulk_wait_all();
     }
 
     tc_fence_before();
@@ -463,6 +689,118 @@ __global__ void __launch_bounds__(256) prep_operands_kernel(const float* __restr
     if (lane == 0) norms[warp] = nrm;
 }
 
+// ---- FP32 operands as two FP16 parts (SPLIT) ----------------------------------------------
+
+// Largest |p| of every column (bit patterns: non-negative floats order like them, and NaN and
+// infinity lie above every finite value), and the number of nonzero entries.  A block takes
+// `rows` rows, a thread columns.
+__global__ void __launch_bounds__(256) split_colmax_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
+                                                           int rows, unsigned* __restrict__ colmax,
+                                                           unsigned long long* __restrict__ nonzero) {
+    const int64_t r0 = (int64_t)blockIdx.x * rows;
+    const int64_t r1 = r0 + rows < n ? r0 + rows : n;
+    unsigned nz = 0u;
+    for (int l = blockIdx.y * blockDim.x + threadIdx.x; l < d; l += gridDim.y * blockDim.x) {
+        unsigned m = 0u;
+#pragma unroll 8
+        for (int64_t r = r0; r < r1; ++r) {
+            const unsigned v = __float_as_uint(P[r * ldp + l]) & 0x7fffffffu;
+            m = max(m, v);
+            nz += v != 0u;
+        }
+        if (m) atomicMax(colmax + l, m);
+    }
+    nz = __reduce_add_sync(0xffffffffu, nz);
+    if ((threadIdx.x & 31) == 0 && nz) atomicAdd(nonzero, (unsigned long long)nz);
+}
+
+// The scale, and whether the split build takes the matrix.  s is the power of two that puts
+// the largest |p| into [2^14, 2^15).  hi = fp16(s p) keeps 11 bits, lo = fp16(s p - hi) the
+// next 11 and a sign while |s p| >= 2^-2; below that lo is subnormal and the error at most
+// 2^-25.  Every column's largest value must be at least 2^2 (after the scale): an element's
+// error is then at most 2^-24 of itself or 2^-27 of its column's largest value.  Columns
+// further apart than that (a factor of 4096), values outside 2^+-40 (whose products could
+// leave FP32) and non-finite points stay on CUDA cores.  So do dot products of few nonzero
+// terms, where FP32 FMAs round less than the truncated chunks: with a fraction f of nonzero
+// entries a pair adds about d f^2 of them, and the two errors cross near 20 (measured, linear
+// kernel, 80% zeros: d = 256 5.6e-8 in FMAs against 6.8e-8, d = 512 7.4e-8 in both).  The line
+// is at 128 terms, four chunks a row: from there the objective of a fit, J = trace K - ..., is
+// no further off either (2,000-point clusters, polynomial: d = 100 -3e-7 against -9e-8, d = 128
+// -1.0e-7 against -1.3e-7, d = 256 -4e-8 against 1.4e-7).  The Gaussian has no such line: its error is that of the last rounding (3.6e-8
+// either way), and the split takes it where the norm expansion applies (kbuild_simt.cu).
+constexpr float kSplitMinTerms = 128.f;
+constexpr int kSplitMinD = 48;   // the Gaussian's line
+__global__ void __launch_bounds__(256) split_decide_kernel(const unsigned* __restrict__ colmax,
+                                                           const unsigned long long* __restrict__ nonzero, int n, int d,
+                                                           int gaussian, const unsigned* maxr, float expand_coef,
+                                                           SplitState* __restrict__ st) {
+    __shared__ unsigned mx_s, mn_s;
+    if (threadIdx.x == 0) {
+        mx_s = 0u;
+        mn_s = 0xffffffffu;
+    }
+    __syncthreads();
+    unsigned mx = 0u, mn = 0xffffffffu;
+    for (int l = threadIdx.x; l < d; l += blockDim.x) {
+        const unsigned v = colmax[l];
+        mx = max(mx, v);
+        if (v) mn = min(mn, v);
+    }
+    atomicMax(&mx_s, mx);
+    atomicMin(&mn_s, mn);
+    __syncthreads();
+    if (threadIdx.x) return;
+    mx = mx_s;
+    mn = mn_s;
+    const float fill = (float)*nonzero / ((float)n * (float)d);
+    bool use = gaussian ? __uint_as_float(*maxr) * expand_coef <= 1e-6f : (float)d * fill * fill >= kSplitMinTerms;
+    int e = 0;   // s = 2^e
+    if (mx) {
+        e = 14 + 127 - (int)(mx >> 23);
+        use = use && mx >= __float_as_uint(0x1p-40f) && mx < __float_as_uint(0x1p40f) &&
+              ldexpf(__uint_as_float(mn), e) >= 4.f;
+    }
+    st->use = use ? 1 : 0;
+    st->scale = use ? ldexpf(1.f, e) : 0.f;
+    st->unscale = use ? ldexpf(1.f, -2 * e) : 0.f;
+}
+
+// FP32 rows -> W = [hi | lo] in FP16, zero padding.  A thread takes four columns of a row
+// (float4 loads when rows are 16-byte aligned), 8-byte stores.
+__global__ void __launch_bounds__(256) split_operands_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
+                                                             int dpad, const SplitState* __restrict__ st,
+                                                             __half* __restrict__ W) {
+    if (!st->use) return;
+    const float s = st->scale;
+    const bool vec = (ldp & 3) == 0 && ((uintptr_t)P & 15) == 0;
+    const int q4 = dpad / 4;
+    const int64_t total = (int64_t)n * q4, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += step) {
+        const int64_t r = t / q4;
+        const int l = 4 * (int)(t - r * q4);
+        const float* p = P + r * ldp + l;
+        float v[4];
+        if (vec && l + 3 < d) {
+            const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+            v[0] = f.x, v[1] = f.y, v[2] = f.z, v[3] = f.w;
+        } else {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) v[x] = l + x < d ? __ldg(p + x) : 0.f;
+        }
+        __half2 hi[2], lo[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const float f0 = v[2 * x] * s, f1 = v[2 * x + 1] * s;
+            hi[x] = __floats2half2_rn(f0, f1);
+            const float2 h = __half22float2(hi[x]);
+            lo[x] = __floats2half2_rn(f0 - h.x, f1 - h.y);
+        }
+        __half* w = W + r * (2 * (int64_t)dpad) + l;
+        *reinterpret_cast<uint2*>(w) = *reinterpret_cast<const uint2*>(hi);
+        *reinterpret_cast<uint2*>(w + dpad) = *reinterpret_cast<const uint2*>(lo);
+    }
+}
+
 }  // namespace
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -493,101 +831,175 @@ bool make_tensor_map_2d(CUtensorMap* m, CUtensorMapDataType dt, void* base, uint
 
 
 size_t kbuild_tc_workspace(int n, int d, int precision) {
-    const size_t dpad = ((size_t)d + BK - 1) / BK * BK;
+    const size_t dpad = ((size_t)d + 63) / 64 * 64;
     const size_t ldw = (precision == POPCORN_BF16X3 ? 2 : 1) * dpad;
     const size_t ops = (size_t)n * ldw * 2;
     return ((ops + 255) & ~(size_t)255) + (size_t)n * 4 + 256;
 }
 
-// shared memory the kernel is configured for: the largest layout below (BF16X3:
-// a full 192 KB ring and one staging buffer of each kind), the column norms,
-// barriers and slack for the 1024-byte alignment
-constexpr int kSmemBytes = RING_BYTES + 2 * STG_BYTES + BM * 4 + 16 * 8 + 16 + 1024;
+namespace {
+
+using TcFn = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, TcArgs);
+
+template <int MODE, int OUT>
+TcFn tc_fn_kind(int kind) {
+    switch (kind) {
+        case POPCORN_LINEAR: return kbuild_tc_kernel<MODE, OUT, POPCORN_LINEAR>;
+        case POPCORN_POLYNOMIAL: return kbuild_tc_kernel<MODE, OUT, POPCORN_POLYNOMIAL>;
+        default: return kbuild_tc_kernel<MODE, OUT, POPCORN_GAUSSIAN>;
+    }
+}
+template <int MODE>
+TcFn tc_fn_out(int out, int kind) {
+    if constexpr (MODE != kModeSplit) {   // (SPLIT: FP32 K only)
+        if (out == kOutHalf16) return tc_fn_kind<MODE, kOutHalf16>(kind);
+        if (out == kOutHalfB16) return tc_fn_kind<MODE, kOutHalfB16>(kind);
+    }
+    if (out == kOutSw16) return tc_fn_kind<MODE, kOutSw16>(kind);
+    if (out == kOutSw4) return tc_fn_kind<MODE, kOutSw4>(kind);
+    return tc_fn_kind<MODE, kOutFull>(kind);
+}
+TcFn tc_fn(int mode, int out, int kind) {
+    if (mode == kModeSplit) return tc_fn_out<kModeSplit>(out, kind);
+    return mode == kModeX3 ? tc_fn_out<kModeX3>(out, kind) : tc_fn_out<kModeBf16>(out, kind);
+}
+
+}  // namespace
 
 cudaError_t configure_kbuild_tc() {
     encode_fn();
-    decltype(&kbuild_tc_kernel<kOutSw16>) fs[4] = {kbuild_tc_kernel<kOutSw16>, kbuild_tc_kernel<kOutSw4>,
-                                                   kbuild_tc_kernel<kOutHalf16>, kbuild_tc_kernel<kOutHalfB16>};
-    for (auto f : fs) {
-        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-    }
+    for (int mode = kModeBf16; mode <= kModeSplit; ++mode)
+        for (int out = kOutFull; out <= (mode == kModeSplit ? kOutSw4 : kOutHalfB16); ++out)
+            for (int kind = POPCORN_LINEAR; kind <= POPCORN_GAUSSIAN; ++kind) {
+                const cudaError_t e = cudaFuncSetAttribute(tc_fn(mode, out, kind),
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+                if (e != cudaSuccess) return e;
+            }
     return cudaSuccess;
 }
 
-cudaError_t launch_kbuild_tc(const float* P, int n, int d, int64_t ldp, KernParams kp, int precision, float* K,
-                             int64_t ldk, float* kdiag, void* workspace, int* err, int num_sms, cudaStream_t s,
-                             int* launches, int packed, int full, int k_storage) {
-    // packed kPackedSw128H: K is the FP16 / BF16 packed triangle (k_storage)
-    const int half = packed == kPackedSw128H ? (k_storage == POPCORN_K_BF16 ? 2 : 1) : 0;
-    if (packed == kPackedSw128H && k_storage != POPCORN_K_FP16 && k_storage != POPCORN_K_BF16)
-        return cudaErrorInvalidValue;
-    const int dpad = (d + BK - 1) / BK * BK;
-    const int x3 = precision == POPCORN_BF16X3 ? 1 : 0;
-    const int64_t ldw = (int64_t)(x3 ? 2 : 1) * dpad;
-    __nv_bfloat16* W = static_cast<__nv_bfloat16*>(workspace);
-    const size_t ops = (size_t)n * ldw * 2;
-    float* norms = reinterpret_cast<float*>(static_cast<char*>(workspace) + ((ops + 255) & ~(size_t)255));
+namespace {
 
-    prep_operands_kernel<<<(n * 32 + 255) / 256, 256, 0, s>>>(P, n, d, ldp, dpad, x3, W, norms);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (launches) ++*launches;
-
+// The tile kernel on operand rows W (n x ldw 16-bit elements).
+cudaError_t launch_tiles(int mode, const void* W, int n, int64_t ldw, int dpad, const SplitState* split,
+                         const KernParams& kp, const float* norms, float* K, int64_t ldk, float* kdiag, int* err,
+                         int num_sms, cudaStream_t s, int out, int full) {
     CUtensorMap mr, mc, mkd, mkt;
     memset(&mkd, 0, sizeof mkd);
     memset(&mkt, 0, sizeof mkt);
-    if (!make_tensor_map_2d(&mr, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, BK,
-                            2 * BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_tensor_map_2d(&mc, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, W, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, BK,
-                            BM, CU_TENSOR_MAP_SWIZZLE_128B))
+    const CUtensorMapDataType dt = split ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    void* w = const_cast<void*>(W);
+    const int dk = kbuild_dk(mode);
+    const CUtensorMapSwizzle sw = dk == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;   // rows of dk elements
+    if (!make_tensor_map_2d(&mr, dt, w, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, dk, BM, sw) ||
+        !make_tensor_map_2d(&mc, dt, w, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, dk, 2 * BM, sw))
         return cudaErrorInvalidValue;
     // the full-square stores go through tensor maps; the packed stores are plain bulk copies
-    if (!packed && (!make_tensor_map_2d(&mkd, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, K, (uint64_t)n, (uint64_t)n,
-                                        (uint64_t)ldk * 4, 32, BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-                    !make_tensor_map_2d(&mkt, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, K, (uint64_t)n, (uint64_t)n,
-                                        (uint64_t)ldk * 4, BM, 32, CU_TENSOR_MAP_SWIZZLE_NONE)))
+    if (out == kOutFull && (!make_tensor_map_2d(&mkd, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, K, (uint64_t)n, (uint64_t)n,
+                                                (uint64_t)ldk * 4, 16, BM, CU_TENSOR_MAP_SWIZZLE_64B) ||
+                            !make_tensor_map_2d(&mkt, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, K, (uint64_t)n, (uint64_t)n,
+                                                (uint64_t)ldk * 4, BM, 16, CU_TENSOR_MAP_SWIZZLE_NONE)))
         return cudaErrorInvalidValue;
-
     TcArgs a;
     a.n = n;
     a.T = (n + BM - 1) / BM;
     a.T2 = (a.T + 1) / 2;
     a.dpad = dpad;
-    a.nkb = dpad / BK;
-    a.x3 = x3;
-    // BF16: 3 stages of 48 KB; BF16X3: 2 stages of 96 KB (hi and lo of both operands)
-    a.stage_bytes = x3 ? 2 * (ROWS_BYTES + COLS_BYTES) : ROWS_BYTES + COLS_BYTES;
-    a.stages = x3 ? 2 : 3;
-    // staging: two buffers of each kind when the ring leaves room, else one
-    const int ring = a.stages * a.stage_bytes;
-    a.nstg = ring + 4 * STG_BYTES <= RING_BYTES + 2 * STG_BYTES ? 2 : 1;
-    a.off_sd = ring;
-    a.off_st = a.off_sd + a.nstg * STG_BYTES;
-    a.off_rj = a.off_st + a.nstg * STG_BYTES;
-    a.off_bar = a.off_rj + BM * 4;
-    a.off_misc = a.off_bar + 16 * 8;
-    a.full = full && !packed ? 1 : 0;
-    a.tiles = a.full ? (long long)a.T2 * a.T : (long long)a.T2 * a.T - (long long)a.T2 * (a.T2 - 1);
-    a.Kp = packed ? K : nullptr;
-    a.sw4 = packed == kPackedSw4 ? 1 : 0;
+    a.nkb = dpad / dk;
+    a.full = full;
+    a.tiles = tile_count(a.T, a.T2, a.full);
+    a.K = K;
+    a.ldk = ldk;
+    a.Kp = out == kOutFull ? nullptr : K;
     a.kp = kp;
     a.norms = norms;
     a.kdiag = kdiag;
+    a.split = split;
     a.err = err;
-    const int smem = a.off_misc + 16 + 1024;
-    if (smem > kSmemBytes) return cudaErrorInvalidConfiguration;
     const int grid = (int)(a.tiles < num_sms ? a.tiles : num_sms);
-    if (half == 1)
-        kbuild_tc_kernel<kOutHalf16><<<grid, NTHREADS, smem, s>>>(mr, mc, mkd, mkt, a);
-    else if (half == 2)
-        kbuild_tc_kernel<kOutHalfB16><<<grid, NTHREADS, smem, s>>>(mr, mc, mkd, mkt, a);
-    else if (a.sw4)
-        kbuild_tc_kernel<kOutSw4><<<grid, NTHREADS, smem, s>>>(mr, mc, mkd, mkt, a);
-    else
-        kbuild_tc_kernel<kOutSw16><<<grid, NTHREADS, smem, s>>>(mr, mc, mkd, mkt, a);
-    if (launches) ++*launches;
+    tc_fn(mode, out, kp.kind)<<<grid, NTHREADS, kSmemBytes, s>>>(mr, mc, mkd, mkt, a);
     return cudaGetLastError();
+}
+
+int packed_out(int packed) { return packed == kPackedSw4 ? kOutSw4 : packed == kPackedSw16 ? kOutSw16 : kOutFull; }
+
+}  // namespace
+
+cudaError_t launch_kbuild_tc(const float* P, int n, int d, int64_t ldp, KernParams kp, int precision, float* K,
+                             int64_t ldk, float* kdiag, void* workspace, int* err, int num_sms, cudaStream_t s,
+                             int* launches, int packed, int full, int k_storage) {
+    // packed kPackedSw128H: K is the FP16 / BF16 packed triangle (k_storage)
+    int out = packed_out(packed);
+    if (packed == kPackedSw128H) {
+        if (k_storage != POPCORN_K_FP16 && k_storage != POPCORN_K_BF16) return cudaErrorInvalidValue;
+        out = k_storage == POPCORN_K_BF16 ? kOutHalfB16 : kOutHalf16;
+    }
+    const int x3 = precision == POPCORN_BF16X3 ? 1 : 0;
+    const int dk = kbuild_dk(x3 ? kModeX3 : kModeBf16), dpad = (d + dk - 1) / dk * dk;
+    const int64_t ldw = (int64_t)(x3 ? 2 : 1) * dpad;
+    __nv_bfloat16* W = static_cast<__nv_bfloat16*>(workspace);
+    const size_t ops = (size_t)n * ldw * 2;
+    float* norms = reinterpret_cast<float*>(static_cast<char*>(workspace) + ((ops + 255) & ~(size_t)255));
+
+    prep_operands_kernel<<<(unsigned)(((int64_t)n * 32 + 255) / 256), 256, 0, s>>>(P, n, d, ldp, dpad, x3, W, norms);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = launch_tiles(x3 ? kModeX3 : kModeBf16, W, n, ldw, dpad, nullptr, kp, norms, K, ldk, kdiag, err, num_sms, s, out,
+                     full && !packed ? 1 : 0);
+    if (launches) *launches += 2;
+    return e;
+}
+
+// Where the split build is the faster one.  The CUDA-core build takes its tiles in waves, each
+// as long as d; the split build costs five more launches (about 25 us) and then a small
+// fraction of that.  Measured (a whole call, us, CUDA cores / split): n = 2,000: d = 400 78 / 77,
+// 512 89 / 78, 784 109 / 91; n = 4,000: d = 128 91 / 88, 256 140 / 95; n = 6,000: d = 48 90 / 101,
+// 96 127 / 103; n = 8,000: d = 64 154 / 134, 784 953 / 266; n = 20,000: d = 48 609 / 441,
+// 784 5397 / 1163.  Below 128 columns the device's rule on the number of terms refuses dot
+// products (linear, polynomial) anyway.
+bool kbuild_split_applies(int n, int d, bool dot) {
+    const long long T = (n + BM - 1) / BM, tiles = T * (T + 1) / 2;
+    return d >= (dot ? (int)kSplitMinTerms : kSplitMinD) && (tiles < 136 ? 136 : tiles) * d >= 65000;
+}
+
+size_t kbuild_split_workspace(int n, int d) {
+    const size_t dpad = ((size_t)d + 31) / 32 * 32;
+    return (((size_t)n * 2 * dpad * 2 + 255) & ~(size_t)255) + (((size_t)d * 4 + 255) & ~(size_t)255) + 512;
+}
+
+cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernParams kp, float* K, int64_t ldk,
+                                float* kdiag, void* workspace, const float* rn, const unsigned* maxr,
+                                float expand_coef, int* err, int num_sms, cudaStream_t s, int* launches, int packed,
+                                int full, const SplitState** state) {
+    const int dpad = (d + 31) / 32 * 32;
+    unsigned char* w = static_cast<unsigned char*>(workspace);
+    const size_t ops = ((size_t)n * 2 * dpad * 2 + 255) & ~(size_t)255;
+    const size_t cols = ((size_t)d * 4 + 255) & ~(size_t)255;
+    __half* W = reinterpret_cast<__half*>(w);
+    unsigned long long* nonzero = reinterpret_cast<unsigned long long*>(w + ops);
+    unsigned* colmax = reinterpret_cast<unsigned*>(w + ops + 256);
+    SplitState* st = reinterpret_cast<SplitState*>(w + ops + 256 + cols);
+    cudaError_t e = cudaMemsetAsync(w + ops, 0, 256 + cols, s);
+    if (e != cudaSuccess) return e;
+    // about eight blocks an SM over (row chunk, 256 columns), at least 32 rows a block
+    const int cy = (d + 255) / 256;
+    int rows = (int)(((int64_t)n * cy + 8 * num_sms - 1) / (8 * num_sms));
+    if (rows < 32) rows = 32;
+    split_colmax_kernel<<<dim3((unsigned)((n + rows - 1) / rows), (unsigned)(cy < 65535 ? cy : 65535)), 256, 0, s>>>(
+        P, n, d, ldp, rows, colmax, nonzero);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    split_decide_kernel<<<1, 256, 0, s>>>(colmax, nonzero, n, d, kp.kind == POPCORN_GAUSSIAN ? 1 : 0, maxr, expand_coef, st);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const int64_t work = (int64_t)n * (dpad / 4);
+    const int64_t blocks = (work + 255) / 256;
+    split_operands_kernel<<<(unsigned)(blocks < 16 * num_sms ? blocks : 16 * num_sms), 256, 0, s>>>(P, n, d, ldp, dpad,
+                                                                                                st, W);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_tiles(kModeSplit, W, n, 2 * (int64_t)dpad, dpad, st, kp, rn, K, ldk, kdiag, err, num_sms, s,
+                     packed_out(packed), full && !packed ? 1 : 0);
+    if (launches) *launches += 4;
+    *state = st;
+    return e;
 }
 
 }  // namespace popcorn

@@ -193,10 +193,13 @@ cudaError_t launch_pack_half(const float* Kf, void* Kh, int k_storage, int n, fl
 // GEMM form) instead of the upper-triangle tiles stored with their transposes (SYRK form).
 // rn (n floats) and maxr (one word), both device workspace: for a Gaussian kernel the row
 // norms, from which the build decides on the device whether the norm expansion is accurate
-// enough; null keeps the coordinate-difference form.
+// enough; null keeps the coordinate-difference form.  split_ws (kbuild_split_workspace bytes; FP32
+// K and d > 16 only) with err and num_sms: the tensor-core split build is launched first, and the
+// CUDA-core kernels return at once where it applies.
 cudaError_t launch_kbuild_simt(const float* P, int n, int d, int64_t ldp, KernParams kp,
                                void* K, int64_t ldk, int k_storage, float* kdiag, cudaStream_t s, int* launches,
-                               int packed = 0, int full = 0, float* rn = nullptr, unsigned* maxr = nullptr);
+                               int packed = 0, int full = 0, float* rn = nullptr, unsigned* maxr = nullptr,
+                               void* split_ws = nullptr, int* err = nullptr, int num_sms = 0);
 
 // ---- K build on tensor cores (kbuild_tc.cu) ---------------------------------
 // Workspace bytes for the BF16 operand copies and row norms.
@@ -213,6 +216,26 @@ cudaError_t configure_kbuild_tc();
 cudaError_t launch_kbuild_tc(const float* P, int n, int d, int64_t ldp, KernParams kp, int precision, float* K,
                              int64_t ldk, float* kdiag, void* workspace, int* err, int num_sms, cudaStream_t s,
                              int* launches, int packed = 0, int full = 0, int k_storage = POPCORN_K_FP32);
+
+// ---- the FP32 K build on tensor cores: FP32 operands as two FP16 parts (kbuild_tc.cu) --------
+// Written on the device from the points: whether the split represents them as FP32 does (and,
+// for the Gaussian, the norm expansion applies), and the power-of-two scales.  Exactly one of
+// the split build and the CUDA-core build does the work of a launch pair.
+struct SplitState {
+    int use;
+    float scale;     // s: operands are s p
+    float unscale;   // s^-2
+};
+bool kbuild_split_applies(int n, int d, bool dot);   // dot: linear or polynomial kernel
+size_t kbuild_split_workspace(int n, int d);
+// FP32 K as launch_kbuild_simt writes it (packed 0, kPackedSw16 or kPackedSw4; full).  rn / maxr /
+// expand_coef: the Gaussian's row norms, their largest and the expansion's error bound (as in
+// launch_kbuild_simt).  *state (device, inside the workspace) tells the CUDA-core launch that
+// follows whether anything is left to do.
+cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernParams kp, float* K, int64_t ldk,
+                                float* kdiag, void* workspace, const float* rn, const unsigned* maxr,
+                                float expand_coef, int* err, int num_sms, cudaStream_t s, int* launches, int packed,
+                                int full, const SplitState** state);
 
 // 2-D tiled TMA descriptor over a row-major matrix (inner = contiguous extent
 // in elements, row_bytes = pitch); false if the driver entry point is missing
