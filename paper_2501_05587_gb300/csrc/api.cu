@@ -1225,18 +1225,19 @@ popcorn_status popcorn_kmeanspp(const float* P, int64_t n, int32_t d, int64_t ld
     if (!lab_dev) POPCORN_TRY(ws.alloc(&labd, (size_t)ni, "labels"));
     int32_t* cend = cen_dev ? centers_out : nullptr;
     if (!cend) POPCORN_TRY(ws.alloc(&cend, (size_t)k, "centers"));
-    double* part;
-    int* small;   // [0] the chosen point, [1] the error word
+    double *part, *Dg;
+    int* err;
     unsigned* bar;
-    POPCORN_TRY(ws.alloc(&part, (size_t)dev->sms, "seeding partial sums"));
-    POPCORN_TRY(ws.alloc(&small, 2, "seeding words"));
+    POPCORN_TRY(ws.alloc(&part, 2 * (size_t)dev->sms, "seeding partial sums"));
+    POPCORN_TRY(ws.alloc(&Dg, 2 * (size_t)ni, "seeding distances"));
+    POPCORN_TRY(ws.alloc(&err, 1, "error word"));
     POPCORN_TRY(ws.alloc(&bar, 32, "grid barrier"));
-    POPCORN_CUDA(cudaMemsetAsync(small, 0, 2 * sizeof(int), s));
-    POPCORN_CUDA(launch_kmeanspp(Pd, ni, d, ldpd, k, kern, ud, labd, cend, part, small, bar, small + 1, dev->sms, s));
+    POPCORN_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+    POPCORN_CUDA(launch_kmeanspp(Pd, ni, d, ldpd, k, kern, ud, labd, cend, part, Dg, bar, err, dev->sms, s));
     void* hpin;
     POPCORN_TRY(pinned(sizeof(int), &hpin));
     int* herr = static_cast<int*>(hpin);
-    POPCORN_CUDA(cudaMemcpyAsync(herr, small + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+    POPCORN_CUDA(cudaMemcpyAsync(herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     if (!lab_dev)
         POPCORN_CUDA(cudaMemcpyAsync(labels_out, labd, (size_t)ni * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (centers_out && !cen_dev)

@@ -274,13 +274,13 @@ cudaError_t launch_fused_fit(const struct PassBuffers& b, double* zpart, unsigne
 
 // ---- K-means++ seeding (seeding.cu) --------------------------------------------
 // One cooperative launch (one CTA per SM) for all k steps; kappa in FP64 from the points.
-// u: k draws (device); labels: n, centers: k (device); part: num_sms doubles, chosen: one
-// int, bar: 32 words of workspace; *err (device) set when a grid-barrier wait runs out.
+// u: k draws (device); labels: n, centers: k (device); part: 2 num_sms doubles, Dg: 2 n doubles,
+// bar: 32 words of workspace; *err (device) set when a grid-barrier wait runs out.
 bool kmeanspp_fits(int n, int d, int num_sms, int smem_optin);
 size_t kmeanspp_smem(int n, int d, int num_sms);
 cudaError_t configure_kmeanspp(int smem_optin);
 cudaError_t launch_kmeanspp(const float* P, int n, int d, int64_t ldp, int k, const popcorn_kernel& kern,
-                            const double* u, int32_t* labels, int32_t* centers, double* part, int* chosen,
+                            const double* u, int32_t* labels, int32_t* centers, double* part, double* Dg,
                             unsigned* bar, int* err, int num_sms, cudaStream_t s);
 
 // ---- recompute path (recompute.cu): K never stored ---------------------------

@@ -14,12 +14,20 @@
 //
 // kmeanspp_kernel: one cooperative launch, one CTA of 512 threads per SM.  CTA b owns the
 // points [b n / G, (b + 1) n / G) and keeps their D, labels and K_ii in shared memory.  A step:
-// the CTA's sum of D (its threads' contiguous chunks, each summed in order, then the chunk
-// sums in order) -> grid barrier -> every CTA adds the G sums in order and locates the CTA
-// whose range holds the target; that CTA finds the point and publishes it -> grid barrier ->
-// every warp evaluates kappa against the new point for its rows (lanes split the coordinates,
-// a butterfly adds them) and lowers D.  All orders are fixed: runs are bit-identical.  Every
-// wait is bounded (grid_sync.cuh).
+// the CTA's sum of D and a copy of its D go to global memory -> grid barrier -> every CTA adds
+// the G sums, locates the CTA whose range holds the target and, from that CTA's D, the point
+// (all alike, in one order) -> the threads evaluate kappa against the new point for their rows
+// and lower D.  D and the sums alternate between two buffers, so a CTA that is ahead never
+// overwrites what another still reads, and one barrier a step is enough.  All orders are fixed:
+// runs are bit-identical.  Every wait is bounded (grid_sync.cuh).
+//
+// What bounds a step is FP64 (2 multiply-adds a clock an SM on GB300), so no FP64 instruction
+// runs on a lane whose result is not used: a point has as many lanes as leave the CTA's threads
+// busy (one from 512 rows a CTA on), so that the inner product, kappa and the distance are not
+// computed 32 times over, as they were with a warp a point (its butterfly, the exponential and
+// the last three operations on every lane: about 1,400 FP64 lane operations a point at d = 64
+// where 230 are needed), and the sums of D are scans, not one thread's chain of 512 additions.
+// n = 50,000, d = 64, k = 32, Gaussian: 5.57 -> 1.35 ms a call.
 #include <cmath>
 
 #include "grid_sync.cuh"
@@ -41,27 +49,26 @@ struct SeedArgs {
     const double* u;           // k draws in [0, 1)
     int32_t* labels;           // n
     int32_t* centers;          // k
-    double* part;              // [G] the CTAs' sums of D
-    int* chosen;               // the point chosen in the running step
+    double* part;              // [2][G] the CTAs' sums of D, by step parity
+    double* Dg;                // [2][n] D, by step parity
     unsigned* bar;             // grid barrier words
     int* err;
     int rows_max;              // ceil(n / G)
 };
 
 // Dynamic shared memory: the center's coordinates [d], then per owned row D, K_ii (doubles)
-// and the label (int), then the threads' chunk sums and their prefix [kSeedThreads] and the
-// CTAs' sums [G] (doubles).
+// and the label (int), then the threads' running sums [kSeedThreads] and the CTAs' sums [G]
+// (doubles).
 struct SeedLayout {
-    size_t cs, D, kii, lab, tsum, tpre, part, bytes;
+    size_t cs, D, kii, lab, inc, part, bytes;
 };
 __host__ __device__ inline SeedLayout seed_layout(int d, int rows_max, int G) {
     SeedLayout L;
     L.cs = 0;
     L.D = L.cs + (size_t)d * 8;
     L.kii = L.D + (size_t)rows_max * 8;
-    L.tsum = L.kii + (size_t)rows_max * 8;
-    L.tpre = L.tsum + (size_t)kSeedThreads * 8;
-    L.part = L.tpre + (size_t)kSeedThreads * 8;
+    L.inc = L.kii + (size_t)rows_max * 8;
+    L.part = L.inc + 2 * (size_t)kSeedThreads * 8;   // (half of it spare: the largest n stays where it was)
     L.lab = L.part + (size_t)G * 8;
     L.bytes = L.lab + (size_t)rows_max * 4;
     return L;
@@ -80,22 +87,47 @@ __device__ __forceinline__ double kappa_of(const SeedArgs& a, double s) {
     return s;
 }
 
-// The warp's FP64 inner product (or squared distance, Gaussian) of point i with the center
-// in shared memory: lane l takes coordinates l, l + 32, ... in order, then a butterfly.
-__device__ __forceinline__ double warp_pair(const SeedArgs& a, int i, const double* __restrict__ cs, int lane) {
-    const float* p = a.P + (int64_t)i * a.ldp;
-    double s = 0.0;
+// The FP64 inner product (or squared distance, Gaussian) of a point with the center in shared
+// memory, by a group of `lanes` (a power of two) neighbouring lanes: lane s takes coordinates s,
+// s + lanes, ... in order, then a butterfly.
+__device__ __forceinline__ double group_pair(const SeedArgs& a, const float* __restrict__ p, const double* __restrict__ cs,
+                                             int s, int lanes) {
+    double t = 0.0;
     if (a.kind == POPCORN_GAUSSIAN) {
-        for (int l = lane; l < a.d; l += 32) {
-            const double t = (double)__ldg(p + l) - cs[l];
-            s = fma(t, t, s);
+#pragma unroll 4
+        for (int l = s; l < a.d; l += lanes) {
+            const double x = (double)__ldg(p + l) - cs[l];
+            t = fma(x, x, t);
         }
     } else {
-        for (int l = lane; l < a.d; l += 32) s = fma((double)__ldg(p + l), cs[l], s);
+#pragma unroll 4
+        for (int l = s; l < a.d; l += lanes) t = fma((double)__ldg(p + l), cs[l], t);
     }
+    for (int o = lanes >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+// Inclusive running sums over the warp's lanes.
+__device__ __forceinline__ double warp_scan(double v, int lane) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    return v;
+}
+
+// Running sums over the CTA: inc[t] = sum of s over threads 0 .. t (a fixed order); the total.
+__device__ double block_scan(double s, double* inc, double* wsum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v = warp_scan(s, lane);
+    if (lane == 31) wsum[warp] = v;
+    __syncthreads();
+    double before = 0.0;
+    for (int w = 0; w < warp; ++w) before += wsum[w];
+    inc[threadIdx.x] = warp ? before + v : v;
+    __syncthreads();
+    return inc[kSeedThreads - 1];
 }
 
 __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
@@ -105,36 +137,38 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
     double* cs = reinterpret_cast<double*>(smem + L.cs);
     double* D = reinterpret_cast<double*>(smem + L.D);
     double* kii = reinterpret_cast<double*>(smem + L.kii);
-    double* tsum = reinterpret_cast<double*>(smem + L.tsum);
-    double* tpre = reinterpret_cast<double*>(smem + L.tpre);
+    double* inc = reinterpret_cast<double*>(smem + L.inc);
     double* part_s = reinterpret_cast<double*>(smem + L.part);
     int* lab = reinterpret_cast<int*>(smem + L.lab);
-    __shared__ double kcc_s, tgt_s;
-    __shared__ int bstar_s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int lo = (int)((int64_t)blockIdx.x * n / G), hi = (int)((int64_t)(blockIdx.x + 1) * n / G);
-    const int rows = hi - lo;
-    const int ch = (rows + kSeedThreads - 1) / kSeedThreads;   // rows a thread sums, in order
-    const int r0 = min(rows, ch * (int)threadIdx.x), r1 = min(rows, r0 + ch);
+    __shared__ double kcc_s, tgt_s, wsum[kSeedWarps];
+    __shared__ int bstar_s, pick_s, pos_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto first_row = [&](int b) { return (int)((int64_t)b * n / G); };
+    const int lo = first_row(blockIdx.x), hi = first_row(blockIdx.x + 1), rows = hi - lo;
+    // lanes a point: as many (a power of two, up to a warp) as the CTA's threads give each row
+    int lanes = 32;
+    while (lanes > 1 && lanes * a.rows_max > kSeedThreads) lanes >>= 1;
+    const int sub = threadIdx.x & (lanes - 1), slot = threadIdx.x / lanes, slots = kSeedThreads / lanes;
 
     // K_ii of the owned points (the Gaussian's is 1)
-    for (int i = lo + warp; i < hi; i += kSeedWarps) {
+    for (int r0 = 0; r0 < rows; r0 += slots) {
+        const int r = r0 + slot;
         double v = 1.0;
         if (a.kind != POPCORN_GAUSSIAN) {
-            const float* p = a.P + (int64_t)i * a.ldp;
+            const float* p = a.P + (int64_t)(lo + min(r, rows - 1)) * a.ldp;
             double s = 0.0;
-            for (int l = lane; l < a.d; l += 32) {
+            for (int l = sub; l < a.d; l += lanes) {
                 const double x = (double)__ldg(p + l);
                 s = fma(x, x, s);
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            v = kappa_of(a, s);
+            for (int o = lanes >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (sub == 0) v = kappa_of(a, s);
         }
-        if (lane == 0) kii[i - lo] = v;
+        if (sub == 0 && r < rows) kii[r] = v;
     }
 
-    // point c joins the chosen set as number t: D and the labels of the owned points
+    // point c joins the chosen set as number t: D and the labels of the owned points, and (for
+    // the next step's choice) D to the buffer of that step
     auto add_center = [&](int t, int c) {
         const float* pc = a.P + (int64_t)c * a.ldp;
         for (int l = threadIdx.x; l < a.d; l += blockDim.x) cs[l] = (double)__ldg(pc + l);
@@ -150,12 +184,17 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
         }
         __syncthreads();
         const double kcc = kcc_s;
-        for (int i = lo + warp; i < hi; i += kSeedWarps) {
-            const double kic = kappa_of(a, warp_pair(a, i, cs, lane));
-            const double dc = fmax(kii[i - lo] - 2.0 * kic + kcc, 0.0);
-            if (lane == 0 && (t == 0 || dc < D[i - lo])) {
-                D[i - lo] = dc;
-                lab[i - lo] = t;
+        double* Dn = a.Dg + (size_t)((t + 1) & 1) * n + lo;
+        for (int r0 = 0; r0 < rows; r0 += slots) {   // (uniform trips: the groups shuffle)
+            const int r = r0 + slot;
+            const double s = group_pair(a, a.P + (int64_t)(lo + min(r, rows - 1)) * a.ldp, cs, sub, lanes);
+            if (sub == 0 && r < rows) {
+                const double dc = fmax(kii[r] - 2.0 * kappa_of(a, s) + kcc, 0.0);
+                if (t == 0 || dc < D[r]) {
+                    D[r] = dc;
+                    lab[r] = t;
+                }
+                Dn[r] = D[r];
             }
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) a.centers[t] = c;
@@ -165,82 +204,99 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
     __syncthreads();
     add_center(0, min((int)floor(a.u[0] * n), n - 1));
     for (int t = 1; t < k; ++t) {
-        // the CTA's sum of D: each thread's chunk in order, then the chunk sums in order
-        double s = 0.0;
-        for (int r = r0; r < r1; ++r) s += D[r];
-        tsum[threadIdx.x] = s;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double run = 0.0;
-            for (int j = 0; j < kSeedThreads; ++j) {
-                tpre[j] = run;
-                run += tsum[j];
-            }
-            a.part[blockIdx.x] = run;
+        double* part = a.part + (size_t)(t & 1) * G;
+        // the CTA's sum of D: each thread's contiguous rows in order, then the threads
+        {
+            const int ch = (rows + kSeedThreads - 1) / kSeedThreads;
+            const int r0 = min(rows, ch * (int)threadIdx.x), r1 = min(rows, r0 + ch);
+            double s = 0.0;
+            for (int r = r0; r < r1; ++r) s += D[r];
+            const double total = block_scan(s, inc, wsum);
+            if (threadIdx.x == 0) part[blockIdx.x] = total;
         }
         if (!gsync::grid_barrier(a.bar, a.err)) return;
-        for (int b = threadIdx.x; b < G; b += blockDim.x) part_s[b] = __ldcg(a.part + b);
-        __syncthreads();
-        // every CTA: the total in CTA order, the target, and the CTA whose range holds it
+        for (int b = threadIdx.x; b < G; b += blockDim.x) part_s[b] = __ldcg(part + b);
         if (threadIdx.x == 0) {
-            double W = 0.0;
-            for (int b = 0; b < G; ++b) W += part_s[b];
-            int bstar = -1;
-            double before = 0.0;
-            if (W > 0.0) {
-                const double target = a.u[t] * W;
-                double run = 0.0;
-                int lastpos = -1;
-                for (int b = 0; b < G && bstar < 0; ++b) {
-                    if (part_s[b] > 0.0) lastpos = b;
-                    if (run + part_s[b] > target) {
-                        bstar = b;
-                        before = run;
-                    }
-                    run += part_s[b];
-                }
-                if (bstar < 0) {   // u_t W rounded up to W: the last CTA with a positive sum
-                    bstar = lastpos;
-                    before = 0.0;
-                    for (int b = 0; b < bstar; ++b) before += part_s[b];
-                }
-                tgt_s = target - before;   // the target inside CTA bstar's range
+            pick_s = kSeedThreads;
+            pos_s = -1;
+        }
+        __syncthreads();
+        // every CTA alike: the running sums of the CTAs in order, the target, and the first CTA
+        // whose running sum exceeds it
+        if (warp == 0) {
+            const int per = (G + 31) / 32, b0 = min(G, lane * per), b1 = min(G, b0 + per);
+            double s = 0.0;
+            int lastpos = -1;
+            for (int b = b0; b < b1; ++b) {
+                s += part_s[b];
+                if (part_s[b] > 0.0) lastpos = b;
             }
-            bstar_s = bstar;
+            const double upto = warp_scan(s, lane);
+            double before = __shfl_up_sync(0xffffffffu, upto, 1);
+            if (lane == 0) before = 0.0;
+            const double W = __shfl_sync(0xffffffffu, upto, 31), target = a.u[t] * W;
+            int b = -1;
+            double run = before;
+            for (int x = b0; x < b1 && b < 0; ++x) {
+                const double next = run + part_s[x];
+                if (next > target) b = x;
+                else run = next;
+            }
+            const unsigned have = __ballot_sync(0xffffffffu, b >= 0);
+            lastpos = __reduce_max_sync(0xffffffffu, lastpos);
+            const int owner = have ? __ffs(have) - 1 : (lastpos >= 0 ? lastpos / per : 0);
+            if (!have && lane == owner) {   // u_t W rounded up to W: the last CTA with a positive sum
+                b = lastpos;
+                run = before;
+                for (int x = b0; x < lastpos; ++x) run += part_s[x];
+            }
+            if (lane == owner) {
+                bstar_s = W > 0.0 ? b : -1;
+                tgt_s = target - run;   // the target inside CTA bstar's range
+            }
         }
         __syncthreads();
         const int bstar = bstar_s;
-        if (bstar == (int)blockIdx.x) {
-            // the thread whose chunk holds the target walks it in order; the last point with
-            // a positive D of the CTA if rounding leaves the target past the end
+        int c;
+        if (bstar < 0) {
+            c = min((int)floor(a.u[t] * n), n - 1);
+        } else {
+            // the first of its rows whose running sum exceeds the target; its last row with a
+            // positive D if rounding leaves the target past the end
             const double tgt = tgt_s;
-            const double lo_run = tpre[threadIdx.x];
-            if (r0 < r1 && lo_run + tsum[threadIdx.x] > tgt && lo_run <= tgt) {
-                double run = lo_run;
-                int c = -1, lastpos = r0;
+            const int blo = first_row(bstar), brows = first_row(bstar + 1) - blo;
+            const double* Db = a.Dg + (size_t)(t & 1) * n + blo;
+            const int ch = (brows + kSeedThreads - 1) / kSeedThreads;
+            const int r0 = min(brows, ch * (int)threadIdx.x), r1 = min(brows, r0 + ch);
+            double s = 0.0;
+            int lastpos = -1;
+            for (int r = r0; r < r1; ++r) {
+                const double x = __ldcg(Db + r);
+                if (x > 0.0) lastpos = r;
+                s += x;
+            }
+            block_scan(s, inc, wsum);
+            if (inc[threadIdx.x] > tgt) atomicMin(&pick_s, (int)threadIdx.x);
+            if (lastpos >= 0) atomicMax(&pos_s, lastpos);
+            __syncthreads();
+            const int pick = pick_s;
+            __syncthreads();
+            if ((int)threadIdx.x == pick) {
+                double run = pick ? inc[pick - 1] : 0.0;
+                int found = -1;
                 for (int r = r0; r < r1; ++r) {
-                    if (D[r] > 0.0) lastpos = r;
-                    run += D[r];
+                    run += __ldcg(Db + r);
                     if (run > tgt) {
-                        c = r;
+                        found = r;
                         break;
                     }
                 }
-                *a.chosen = lo + (c >= 0 ? c : lastpos);   // rounding at the chunk's end
+                if (found < 0) found = lastpos >= 0 ? lastpos : max(r0, min(r1, brows) - 1);   // rounding at the chunk's end
+                pos_s = found;
             }
             __syncthreads();
-            if (threadIdx.x == 0) {
-                double total = 0.0;
-                for (int j = 0; j < kSeedThreads; ++j) total += tsum[j];
-                if (!(total > tgt)) {
-                    int c = rows - 1;
-                    while (c > 0 && !(D[c] > 0.0)) --c;
-                    *a.chosen = lo + c;
-                }
-            }
+            c = blo + max(0, pos_s);
         }
-        if (!gsync::grid_barrier(a.bar, a.err)) return;
-        const int c = bstar >= 0 ? __ldcg(a.chosen) : min((int)floor(a.u[t] * n), n - 1);
         add_center(t, c);
     }
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) a.labels[i] = lab[i - lo];
@@ -271,7 +327,7 @@ bool kmeanspp_fits(int n, int d, int num_sms, int smem_optin) {
 }
 
 cudaError_t launch_kmeanspp(const float* P, int n, int d, int64_t ldp, int k, const popcorn_kernel& kern,
-                            const double* u, int32_t* labels, int32_t* centers, double* part, int* chosen,
+                            const double* u, int32_t* labels, int32_t* centers, double* part, double* Dg,
                             unsigned* bar, int* err, int num_sms, cudaStream_t s) {
     SeedArgs a;
     a.P = P;
@@ -288,7 +344,7 @@ cudaError_t launch_kmeanspp(const float* P, int n, int d, int64_t ldp, int k, co
     a.labels = labels;
     a.centers = centers;
     a.part = part;
-    a.chosen = chosen;
+    a.Dg = Dg;
     a.bar = bar;
     a.err = err;
     a.rows_max = (n + num_sms - 1) / num_sms;
