@@ -55,7 +55,6 @@ struct DeviceInfo {
     int smem_optin = 0;
     int reduce_smem = 0;   // dynamic shared memory usable by the reduction kernel
     int recompute_smem = 0;
-    int batched_smem = 0;
     bool coop = false;   // cooperative launches (all CTAs of a grid resident at once)
     cudaMemPool_t pool = nullptr;
     bool ready = false;
@@ -86,8 +85,8 @@ popcorn_status device_info(DeviceInfo** out) {
         POPCORN_CUDA(configure_reduce_smem(d.smem_optin, &d.reduce_smem));
         POPCORN_CUDA(configure_kbuild_tc());
         POPCORN_CUDA(configure_recompute(d.smem_optin, &d.recompute_smem));
-        POPCORN_CUDA(configure_batched(d.smem_optin));
         POPCORN_CUDA(configure_batched_mma(d.smem_optin));
+        POPCORN_CUDA(configure_reduce_tiles(d.smem_optin));
         POPCORN_CUDA(configure_reduce_sym(d.smem_optin));
         POPCORN_CUDA(configure_pack_half());
         POPCORN_CUDA(configure_sym_mma(d.smem_optin));
@@ -96,7 +95,6 @@ popcorn_status device_info(DeviceInfo** out) {
         int coop = 0;
         POPCORN_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         d.coop = coop != 0;
-        d.batched_smem = d.smem_optin - 1024;
         d.ready = true;
     }
     *out = &d;
@@ -776,6 +774,12 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     if (opt.k_pass == 1 || (opt.k_pass == 0 && sym_auto))
         sym = plan_reduce_sym(ni, k, dev->sms, dev->smem_optin, opt.sym_tile, 0, (int)kelem);
     const bool use_sym = sym.ok;
+    // more clusters than the symmetric pass takes, FP32 K: the packed triangle all the same, read
+    // by block rows (each tile twice, the second time from L2).  k_pass = 2 keeps the row-by-row
+    // read of a row-major K.
+    const bool use_tiles = !use_sym && ks == POPCORN_K_FP32 && opt.k_pass != 2 && k > kSymMaxK && ni >= kTilesMinN &&
+                           plan_reduce_tiles(ni, k, dev->sms, &plan);
+    const int64_t tri_tiles = (int64_t)((ni + 127) / 128) * ((ni + 127) / 128 + 1) / 2;
     // A half K read as the full square (k > kSymMaxK, or k_pass = 2) goes through the tensor
     // cores, as batched mode's one-instance form: every tile of the square in the half tile
     // layout, each 128-row block's tiles MMA'd against the one-hot label operands with the
@@ -795,6 +799,7 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     // tensor-core builds alike.
     sym.packed = use_sym;
     const size_t k_bytes = sym.packed ? (size_t)sym.items * 128 * 128 * kelem
+                           : use_tiles ? (size_t)tri_tiles * 128 * 128 * kelem
                            : mma_full ? (size_t)Tf * Tf * 32768
                                       : (size_t)ni * (size_t)ldk * kelem;
     const int nslots = use_sym ? sym.nslots : mma_full ? 1 : plan.nseg;
@@ -860,6 +865,7 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     b.sym_meta = nullptr;
     b.sym_order = nullptr;
     if (use_sym && sym.meta_bytes) POPCORN_TRY(ws.alloc(&b.sym_meta, sym.meta_bytes, "block label metadata"));
+    if (use_tiles) POPCORN_TRY(ws.alloc(&b.sym_meta, tiles_record_bytes(ni), "label records"));
     std::vector<int> sym_order;
     if (use_sym && sym.units > 1 && !capturing) {   // (the natural order inside a caller's capture)
         sym_unit_order(sym, &sym_order);
@@ -872,7 +878,7 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     // one pass's reduction: the K stream (for the symmetric pass: stream, then fold with z)
     // kernels of one pass's reduction: the full-square stream; or the symmetric stream and its
     // fold (the sorted form first sorts every block's labels)
-    const int red_launches = use_sym ? (sym.sorted || sym.mma ? 3 : 2) : mma_full ? 3 : 1;
+    const int red_launches = use_sym ? (sym.sorted || sym.mma ? 3 : 2) : mma_full ? 3 : use_tiles ? 2 : 1;
     // Error-path test hook: with POPCORN_TEST_SYM_STALL_MS=<ms> in the environment, the
     // first symmetric stream launch of this fit (either form) leaves one block's copies out
     // and bounds its waits by <ms>, so the fit reports POPCORN_ERR_TIMEOUT (nothing faults
@@ -896,8 +902,9 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
             if (e == cudaSuccess && mid) e = cudaEventRecord(mid, st);
             return e != cudaSuccess ? e : launch_zreduce(b, 1, eval, st);
         }
-        if (!use_sym) return launch_reduce(b, plan, eval, st);
+        if (!use_sym && !use_tiles) return launch_reduce(b, plan, eval, st);
         stall_ms = 0;
+        if (use_tiles) return launch_reduce_tiles(b, plan, &b.st->wait_err, eval, st, stall);
         return launch_reduce_sym(b, sym, &b.st->wait_err, eval, st, mid, stall);
     };
     POPCORN_TRY(ws.alloc(&b.zsum, (size_t)k, "z sums"));
@@ -969,7 +976,8 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
         ws.release(kf);
     } else {
         POPCORN_TRY(build_kernel_matrix(Pd, ni, d, ldpd, kp, opt.precision, K, ldk, ks, kdiag, &ws,
-                                        &b.st->wait_err, dev->sms, s, &launches, sym.packed ? sym.layout : 0));
+                                        &b.st->wait_err, dev->sms, s, &launches,
+                                        sym.packed ? sym.layout : use_tiles ? kPackedSw4 : 0));
     }
     POPCORN_CUDA(launch_trace(kdiag, ni, b.st, s));
     POPCORN_CUDA(launch_init_labels(Ld, ni, k, b.lab32, b.lab8, b.counts, b.st, s));
@@ -1300,6 +1308,12 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     // K-stream unit lengths the autotuner may pick (Spart is sized for the shortest)
     static const int kSegCand[] = {2048, 4096, 8192, 16384};
     const int min_seglen = opt.autotune ? kSegCand[0] : kBatchSeg;
+    // FP32 K: column blocks a unit (and a sum) takes
+    auto set_segments = [](BatchInst* b, int seglen) {
+        const int blocks = std::min(seglen / 128, b->T);
+        b->seglen = 128 * blocks;
+        b->nseg = (b->T + blocks - 1) / blocks;
+    };
     for (int t = 0; t < count; ++t) {
         const popcorn_instance& x = inst[t];
         if (!x.P || !x.init_labels || !x.labels_out) return fail(POPCORN_ERR_INVALID, "instance %d: null pointer", t);
@@ -1325,12 +1339,15 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.ldk = (n + 3) / 4 * 4;
         b.n = n;
         b.k = k;
-        b.seglen = half ? n : min_seglen;
-        b.nseg = half ? 1 : (n + min_seglen - 1) / min_seglen;   // half K: S written once a row
+        if (half) {   // S written once a row
+            b.seglen = n;
+            b.nseg = 1;
+        } else {
+            set_segments(&b, min_seglen);
+        }
         b.init_labels = x.init_labels;
         b.labels_out = x.labels_out;
-        b.unit0 = bp.units;
-        bp.units += batch_units(n, b.nseg);
+        bp.units += b.T * b.nseg;
         b.zblock0 = bp.zblocks;
         bp.zblocks += (n + kZReduceRows - 1) / kZReduceRows;
         b.ablock0 = bp.ablocks;
@@ -1339,21 +1356,21 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         bp.lblocks += (n + kBatchLabelThreads - 1) / kBatchLabelThreads;
         if (k > bp.kmax) bp.kmax = k;
         const int zb = (n + kZReduceRows - 1) / kZReduceRows;
-        // the FP32 square: the K read by the FP32 passes, or the tensor-core builds' output that
-        // the pack rounds into half tiles (the FP32 build writes half tiles directly)
-        const bool fp32_square = !half || opt.precision != POPCORN_FP32;
-        o[t].K = fp32_square ? take((size_t)n * b.ldk * 4) : 0;
+        // FP32 K: the packed triangle the K stream reads.  Half K: the tensor-core builds write
+        // the FP32 square that the pack rounds into half tiles (the FP32 build writes those directly)
+        o[t].K = !half ? take((size_t)b.T * (b.T + 1) / 2 * 65536)
+                 : opt.precision != POPCORN_FP32 ? take((size_t)n * b.ldk * 4) : 0;
         if (half) {
             b.N = (k + 15) / 16 * 16;
             b.htile0 = bp.htiles;
             bp.htiles += (long long)b.T * b.T;
-            b.vblock0 = bp.vblocks;
-            bp.vblocks += b.T;
             bp.nunits += b.T;
             if (b.N > bp.Nmax) bp.Nmax = b.N;
             o_kh[t] = take((size_t)b.T * b.T * 32768);
-            o_v[t] = take((size_t)b.T * b.N * 256);
         }
+        b.vblock0 = bp.vblocks;
+        bp.vblocks += b.T;
+        o_v[t] = take(half ? (size_t)b.T * b.N * 256 : tiles_record_bytes(n));
         o[t].kdiag = take((size_t)n * 4);
         o[t].lab32 = take((size_t)n * 4);
         o[t].lab8 = take(((size_t)n + 15) & ~(size_t)15);
@@ -1372,21 +1389,23 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         }
     }
     if (bp.units <= 0 || bp.units >= (1 << 30)) return fail(POPCORN_ERR_UNSUPPORTED, "batch too large");
-    plan_batched_reduce(&bp, dev->sms, dev->batched_smem);
-    // half K: the units (instance, row block), the larger instances first (their units take
-    // longer), so that the static round-robin of the stream ends near balance
+    // the units of the K stream -- half K: (instance, row block); FP32 K: (instance, segment x T +
+    // row block) -- the larger instances first (their units take longer), so that the static
+    // round-robin of the stream ends near balance; an instance's units stay together (its block
+    // rows share tiles in L2)
     std::vector<int2> hunits;
-    if (half) {
-        if (!plan_batched_mma(&bp, dev->sms, dev->smem_optin))
-            return fail(POPCORN_ERR_UNSUPPORTED, "the batched tensor-core stream does not fit this device");
-        std::vector<int> order(count);
-        for (int t = 0; t < count; ++t) order[t] = t;
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h[x].T > h[y].T; });
-        hunits.reserve((size_t)bp.nunits);
+    std::vector<int> order(count);
+    for (int t = 0; t < count; ++t) order[t] = t;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h[x].T > h[y].T; });
+    auto list_units = [&]() {
+        hunits.clear();
         for (int t : order)
-            for (int r = 0; r < h[t].T; ++r) hunits.push_back(make_int2(t, r));
-    }
-    const size_t units_off = half ? take(sizeof(int2) * hunits.size()) : 0;
+            for (int r = 0; r < h[t].T * (half ? 1 : h[t].nseg); ++r) hunits.push_back(make_int2(t, r));
+    };
+    if (half ? !plan_batched_mma(&bp, dev->sms, dev->smem_optin) : !plan_batched_tiles(&bp, dev->sms))
+        return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
+    list_units();
+    const size_t units_off = take(sizeof(int2) * hunits.size());   // (the most units of any schedule)
     const size_t inst_off = take(sizeof(BatchInst) * (size_t)count);
     const size_t tc_off = tc_ws ? take(tc_ws) : 0;
     const size_t err_off = take(sizeof(int));
@@ -1409,29 +1428,27 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.st = reinterpret_cast<LoopState*>(base + o[t].st);
         b.J_hist = reinterpret_cast<double*>(base + o[t].J);
         b.changed_hist = reinterpret_cast<int32_t*>(base + o[t].ch);
-        if (half) {
-            b.Kh = base + o_kh[t];
-            b.V = base + o_v[t];
-        }
+        if (half) b.Kh = base + o_kh[t];
+        b.V = base + o_v[t];
     }
-    const int2* dunits = half ? reinterpret_cast<const int2*>(base + units_off) : nullptr;
-    if (half)
-        POPCORN_CUDA(cudaMemcpyAsync(base + units_off, hunits.data(), sizeof(int2) * hunits.size(),
-                                     cudaMemcpyHostToDevice, s));
+    const int2* dunits = reinterpret_cast<const int2*>(base + units_off);
+    auto upload_units = [&]() {
+        return cudaMemcpyAsync(base + units_off, hunits.data(), sizeof(int2) * hunits.size(), cudaMemcpyHostToDevice, s);
+    };
+    POPCORN_CUDA(upload_units());
     BatchInst* dI = reinterpret_cast<BatchInst*>(base + inst_off);
     POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count, cudaMemcpyHostToDevice, s));
     int* err = reinterpret_cast<int*>(base + err_off);
     POPCORN_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
 
-    // ---- schedule of the batched K stream: unit length, warps per block, blocks per SM
+    // ---- schedule of the batched K stream: unit length, blocks per SM (4 consumer warps a block)
     auto set_seglen = [&](int seglen) {
         bp.units = 0;
         for (int t = 0; t < count; ++t) {
-            h[t].seglen = seglen;
-            h[t].nseg = (h[t].n + seglen - 1) / seglen;
-            h[t].unit0 = bp.units;
-            bp.units += batch_units(h[t].n, h[t].nseg);
+            set_segments(&h[t], seglen);
+            bp.units += h[t].T * h[t].nseg;
         }
+        list_units();
     };
     int sched[3] = {kBatchSeg, 0, 0};
     int tune_hit = 0, tune_cands = 0;
@@ -1457,45 +1474,43 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
             } else {
                 for (int t = 0; t < count; ++t)
                     POPCORN_CUDA(launch_kbuild_tc(h[t].P, h[t].n, h[t].d, h[t].ldp, h[t].kp, opt.precision, h[t].K,
-                                                  h[t].ldk, h[t].kdiag, base + tc_off, err, dev->sms, s, nullptr));
+                                                  h[t].ldk, h[t].kdiag, base + tc_off, err, dev->sms, s, nullptr,
+                                                  kPackedSw4));
             }
             cudaEvent_t t0, t1;
             g_events.used = 0;
             POPCORN_TRY(g_events.get(&t0));
             POPCORN_TRY(g_events.get(&t1));
             best.ms = 3.0e38f;
-            static const int kWarpCand[] = {4, 8, 16};
-            static const int kPerSmCand[] = {1, 2};
             for (int seglen : kSegCand)
-                for (int w : kWarpCand)
-                    for (int ps : kPerSmCand) {
-                        BatchPlan cand = bp;
-                        set_seglen(seglen);
-                        cand.units = bp.units;
-                        plan_batched_reduce(&cand, dev->sms, dev->batched_smem, w, ps);
-                        if (cand.warps != w || cand.per_sm != ps) continue;   // does not fit: skip
-                        POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count,
-                                                     cudaMemcpyHostToDevice, s));
-                        POPCORN_CUDA(launch_batched_reduce(dI, cand, 0, s));   // warm-up
-                        float ms = 3.0e38f;
-                        for (int rep = 0; rep < 2; ++rep) {
-                            POPCORN_CUDA(cudaEventRecord(t0, s));
-                            POPCORN_CUDA(launch_batched_reduce(dI, cand, 0, s));
-                            POPCORN_CUDA(cudaEventRecord(t1, s));
-                            POPCORN_CUDA(cudaEventSynchronize(t1));
-                            float e = 0.f;
-                            POPCORN_CUDA(cudaEventElapsedTime(&e, t0, t1));
-                            ms = e < ms ? e : ms;
-                        }
-                        ++tune_cands;
-                        if (ms < best.ms) {
-                            best.ms = ms;
-                            best.p[0] = seglen;
-                            best.p[1] = w;
-                            best.p[2] = ps;
-                            best.p[3] = 0;
-                        }
+                for (int ps : {1, 2}) {
+                    BatchPlan cand = bp;
+                    set_seglen(seglen);
+                    cand.units = bp.units;
+                    if (!plan_batched_tiles(&cand, dev->sms, ps) || cand.per_sm != ps) continue;   // does not fit: skip
+                    POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count,
+                                                 cudaMemcpyHostToDevice, s));
+                    POPCORN_CUDA(upload_units());
+                    POPCORN_CUDA(launch_batched_tiles(dI, dunits, cand, err, 0, s));   // warm-up
+                    float ms = 3.0e38f;
+                    for (int rep = 0; rep < 2; ++rep) {
+                        POPCORN_CUDA(cudaEventRecord(t0, s));
+                        POPCORN_CUDA(launch_batched_tiles(dI, dunits, cand, err, 0, s));
+                        POPCORN_CUDA(cudaEventRecord(t1, s));
+                        POPCORN_CUDA(cudaEventSynchronize(t1));
+                        float e = 0.f;
+                        POPCORN_CUDA(cudaEventElapsedTime(&e, t0, t1));
+                        ms = e < ms ? e : ms;
                     }
+                    ++tune_cands;
+                    if (ms < best.ms) {
+                        best.ms = ms;
+                        best.p[0] = seglen;
+                        best.p[1] = cand.warps;
+                        best.p[2] = ps;
+                        best.p[3] = 0;
+                    }
+                }
             int herr = 0;
             POPCORN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
             POPCORN_CUDA(cudaStreamSynchronize(s));
@@ -1504,13 +1519,15 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
             tune_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - w0).count();
             tune_store(key, best);
         }
-        sched[0] = best.p[0];
+        sched[0] = std::max(best.p[0], min_seglen);   // (units and Spart are sized for min_seglen)
         sched[1] = best.p[1];
         sched[2] = best.p[2];
     }
     if (!half) {
         set_seglen(sched[0]);
-        plan_batched_reduce(&bp, dev->sms, dev->batched_smem, sched[1], sched[2]);
+        POPCORN_CUDA(upload_units());
+        if (!plan_batched_tiles(&bp, dev->sms, sched[2]))
+            return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
         sched[1] = bp.warps;
         sched[2] = bp.per_sm;
     } else {
@@ -1546,7 +1563,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         for (int t = 0; t < count && cap == POPCORN_OK; ++t) {
             const BatchInst& b = h[t];
             step(launch_kbuild_tc(b.P, b.n, b.d, b.ldp, b.kp, opt.precision, b.K, b.ldk, b.kdiag, base + tc_off, err,
-                                  dev->sms, cs, &launches),
+                                  dev->sms, cs, &launches, half ? 0 : kPackedSw4),
                  "tensor-core K build");
         }
     }
@@ -1567,18 +1584,18 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         if (stall_ms < 0 || stall_ms > 10000) stall_ms = 0;
     }
     auto pass = [&](int eval) -> cudaError_t {
-        if (!half) return launch_batched_pass(dI, bp, eval, cs);
-        const cudaError_t e = launch_batched_mma_stream(dI, dunits, bp, err, eval, cs, stall_ms);
+        const cudaError_t e = half ? launch_batched_mma_stream(dI, dunits, bp, err, eval, cs, stall_ms)
+                                   : launch_batched_tiles(dI, dunits, bp, err, eval, cs);
         stall_ms = 0;
         return e != cudaSuccess ? e : launch_batched_finish(dI, bp, eval, cs);
     };
     for (int it = 0; it < max_iter && cap == POPCORN_OK; ++it) {
         step(pass(0), "batched pass");
-        launches += half ? 4 : 3;
+        launches += 4;
     }
     step(pass(1), "batched objective pass");
     step(launch_batched_copy_labels(dI, bp, cs), "batched label copy");
-    launches += half ? 4 : 3;
+    launches += 4;
     cudaGraph_t graph = nullptr;
     cudaError_t ec = cudaStreamEndCapture(cs, &graph);
     if (cap != POPCORN_OK) {

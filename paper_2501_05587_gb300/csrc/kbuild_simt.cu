@@ -563,8 +563,8 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
 
 // All instances of a batch: flattened tile b belongs to the instance whose
 // tile0 is the largest one <= b.
-// TK float: each instance's FP32 square, row-major (K, ldk); TK __half / __nv_bfloat16: its
-// square as half tiles (Kh, kPackedSw128H), for the tensor-core batched stream.
+// TK float: each instance's FP32 block-packed triangle (K, kPackedSw4); TK __half / __nv_bfloat16:
+// its square as half tiles (Kh, kPackedSw128H), for the tensor-core batched stream.
 template <typename TK>
 __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst* I, int count) {
     const long long b = blockIdx.x;
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst*
     const BatchInst& x = I[lo];
     const long long t = b - x.tile0;
     __shared__ __align__(16) TileSmem sm;   // one copy for the three kernel functions
-    constexpr int PK = sizeof(TK) == 2 ? kPackedSw128H : 0;
+    constexpr int PK = sizeof(TK) == 2 ? kPackedSw128H : kPackedSw4;
     TK* K = sizeof(TK) == 2 ? reinterpret_cast<TK*>(x.Kh) : reinterpret_cast<TK*>(x.K);
     switch (x.kp.kind) {
         case POPCORN_LINEAR:

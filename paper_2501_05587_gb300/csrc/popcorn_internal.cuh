@@ -50,7 +50,7 @@ struct LoopState {
 // Variants of the K-streaming reduction, by how a warp reduces its per-lane
 // partials at the end of a unit: butterfly over 4 or 8 clusters, or the
 // rotated row walk for larger k.
-enum { kReduceBfly4 = 0, kReduceBfly8 = 1, kReduceRotated = 2 };
+enum { kReduceBfly4 = 0, kReduceBfly8 = 1, kReduceRotated = 2, kReduceTiles = 3 /* reduce_tiles.cu */ };
 
 // Launch geometry of the K-streaming reduction (segment-split rows).
 struct ReducePlan {
@@ -77,6 +77,7 @@ struct ReducePlan {
 constexpr int kSymMaxK = 32;
 constexpr int kSymBranchMaxK = 8;
 constexpr int kSymAutoMinN = 8192;   // the automatic choice takes the symmetric pass from here
+constexpr int kTilesMinN = 6145;     // and, with more clusters, the block-row pass over the packed triangle
 struct SymPlan {
     bool ok;
     bool sorted;        // the sorted form (k > kSymBranchMaxK, or a forced super-tile edge > 1)
@@ -357,7 +358,8 @@ struct PassBuffers {
     double* J_hist;       // [max(1, max_iter)]
     int32_t* changed_hist;
     float* E_out;         // optional n x k
-    uint8_t* sym_meta;    // sorted form of the symmetric pass: the label-sorted lists of every block
+    uint8_t* sym_meta;    // sorted form of the symmetric pass: the label-sorted lists of every block; block-row
+                          // pass: the label records
     const int* sym_order; // symmetric pass: super-tiles in processing order (larger first), or null
 };
 
@@ -371,6 +373,17 @@ cudaError_t launch_recompute_pass(const PassBuffers& b, KernParams kp, const Rec
 // (||c||^2, 1/|L_c|, J); blocks of kZReduceRows rows.
 constexpr int kZReduceRows = 1024;
 cudaError_t launch_zreduce(const PassBuffers& b, int nseg, int eval, cudaStream_t s);
+
+// The K stream over the block-packed triangle (kPackedSw4, FP32) with a lane to a row
+// (reduce_tiles.cu), any k.  Plan: nseg slots of Spart, seglen columns each; the ring depth in
+// `warps`.  Same outputs as launch_reduce; *err as launch_reduce_sym, stall_ms too.  Each pass
+// first writes the columns' label records (sym_meta, tiles_record_bytes).
+constexpr int kTilesRecord = 144;     // bytes a 32-column piece
+size_t tiles_record_bytes(int n);
+bool plan_reduce_tiles(int n, int k, int num_sms, ReducePlan* p);
+cudaError_t configure_reduce_tiles(int smem_optin);
+cudaError_t launch_reduce_tiles(const PassBuffers& b, const ReducePlan& plan, int* err, int eval_only, cudaStream_t s,
+                                int stall_ms);
 
 // One assignment pass = reduction (E, z, J) + distance/argmin.
 cudaError_t launch_reduce(const PassBuffers& b, const ReducePlan& plan, int eval_only,
@@ -406,11 +419,11 @@ struct BatchInst {
     int32_t* changed_hist;
     const int32_t* init_labels;
     int32_t* labels_out;
-    int unit0, zblock0, ablock0, lblock0;
+    int zblock0, ablock0, lblock0;
     // FP16 / BF16 K (batched_mma.cu): every tile of the square in kPackedSw128H, tile (I, J) at
     // Kh + (I T + J) 32 KB; the per-pass one-hot operands of the T blocks, N rows each
     unsigned char* Kh;
-    unsigned char* V;
+    unsigned char* V;         // (FP32 K: the label records of reduce_tiles.cu)
     int N;                    // accumulator columns: k rounded up to 16
     long long htile0;         // first flattened tile of the square
     int vblock0;              // first flattened 128-block
@@ -421,7 +434,7 @@ struct BatchPlan {
     long long tiles;          // K tiles of all instances
     int units, zblocks, ablocks, lblocks;
     int kmax;
-    int warps, grid, per_sm;  // batched K-stream launch
+    int warps, grid, per_sm;  // batched K-stream launch (FP32 K)
     size_t smem;
     // FP16 / BF16 K: the tensor-core stream over (instance, row block) units
     int half;                 // 0, or the k_storage of every instance's K
@@ -434,17 +447,20 @@ struct BatchPlan {
 };
 
 constexpr int kBatchLabelThreads = 256;
-constexpr int kBatchSeg = 8192;       // columns per K-stream unit in batched mode (whole rows for n <= 8192)
-// K-stream units of one instance in batched mode
-inline int batch_units(int n, int nseg) { return n * nseg; }
+constexpr int kBatchSeg = 8192;       // most columns a K-stream unit takes in batched mode (whole rows for n <= 8192)
 
 // per instance: loop state, labels/counts, (after the K build) trace of K
 cudaError_t launch_batched_init(const BatchInst* dI, const BatchPlan& bp, int max_iter, int check_conv, double tol,
                                 cudaStream_t s);
 cudaError_t launch_batched_trace(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
 cudaError_t launch_batched_kbuild_simt(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
-// one pass over every instance that has not stopped (K stream, z, argmin)
-cudaError_t launch_batched_pass(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
+// FP32 K, the packed triangle (reduce_tiles.cu): the K stream of a pass over every instance that
+// has not stopped, its units (instance, segment x T + row block) in the caller's order, segments of
+// seglen columns (a multiple of 128).  Plan: ring depth (mstages), CTAs an SM (per_sm_req caps it),
+// shared memory for sums of kmax clusters.
+bool plan_batched_tiles(BatchPlan* bp, int num_sms, int per_sm_req = 0);
+cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err, int eval,
+                                 cudaStream_t s);
 // the rest of a pass after its K stream: z (with per-instance finalization) and the argmin
 cudaError_t launch_batched_finish(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
 cudaError_t launch_batched_copy_labels(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
@@ -460,11 +476,6 @@ cudaError_t configure_batched_mma(int smem_optin);
 cudaError_t launch_batched_pack_half(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
 cudaError_t launch_batched_mma_stream(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err,
                                       int eval, cudaStream_t s, int stall_ms = 0);
-// warps / grid / shared memory of the batched K stream for clusters up to kmax;
-// warps = 0 / per_sm = 0 pick the largest that fits / the occupancy limit
-void plan_batched_reduce(BatchPlan* bp, int num_sms, int smem_budget, int warps = 0, int per_sm = 0);
-// the batched K stream alone (what the autotuner times)
-cudaError_t launch_batched_reduce(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
 
 // ---- autotune cache (autotune.cu) ---------------------------------------------
 struct TuneKey {
@@ -480,6 +491,5 @@ struct TuneValue {
 int32_t log2_bucket(double x);   // round(4 log2 x): quarter-octave buckets
 bool tune_lookup(const TuneKey& k, TuneValue* v);
 void tune_store(const TuneKey& k, const TuneValue& v);
-cudaError_t configure_batched(int smem_optin);
 
 }  // namespace popcorn
