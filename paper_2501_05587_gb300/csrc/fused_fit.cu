@@ -15,11 +15,19 @@
 //               go to its slot.
 //   exchange A  every CTA reads all partials and adds them in the same fixed order:
 //               ||c_c||^2, 1/|L_c| and J, identical in every CTA; CTA 0 records them.
-//   argmin      D_ic = K_ii - 2 E_ic + ||c_c||^2 in FP64 for the CTA's rows (ties to the
-//               lowest index, empty clusters skipped), new labels; the histogram of the
-//               CTA's new labels and its change count go to its slot.
+//   argmin      D_ic = K_ii - 2 E_ic + ||c_c||^2 for the CTA's rows (ties to the lowest
+//               index, empty clusters skipped), screened in FP32 and decided in FP64 at
+//               near-ties as the pass kernels do (iterate.cu), new labels; the histogram of
+//               the CTA's new labels and its change count go to its slot.
 //   exchange B  every CTA reads all labels, sums the histograms (the next pass's counts)
 //               and the change counts, and takes the same loop decision.
+//
+// What bounds a pass is its chain of latencies, not work (n = 2,000: 16 us of which the row sums
+// are 1.5), so what a later step does not need at once is off the chain: 1/|L_c| is formed while
+// the z partials are, J by one warp that has no rows while the others take their argmin (adding
+// the clusters up in every thread cost 16 FP64 additions x 512 threads, 2 us at GB300's FP64
+// rate), and the four columns of a float4 load their bins together.
+// n = 2,000, k = 8, 30 passes: the kernel 467 -> 395 us, the whole call 605 -> 532.
 //
 // An exchange is a grid barrier (one arrival counter, acquire-release) after which the CTAs
 // read the slots from L2.  The pass semantics (stopping
@@ -67,20 +75,18 @@ struct FusedArgs {
 };
 
 // Dynamic shared memory, in order: per-warp bins [kFusedWarps][k][32] floats, the row
-// sums of the CTA's rows [rows_max][k] floats, then cnorm and 1/|L_c| ([k] doubles each),
+// sums of the CTA's rows [rows_max][k] floats, then
 // the next labels' histogram and the current counts ([k] ints each), the CTA's diag K
 // [rows_max] floats, the labels of
 // all points (n rounded up to 16) and, when cache_k, the CTA's rows of K [rows_max][ldk].
 struct FusedLayout {
-    size_t bins, S, cn, iv, hist, m, kd, lab, Kc, bytes;
+    size_t bins, S, hist, m, kd, lab, Kc, bytes;
 };
 __host__ __device__ inline FusedLayout fused_layout(int n, int k, int rows_max, int64_t ldk, int cache_k) {
     FusedLayout L;
     L.bins = 0;
     L.S = L.bins + (size_t)kFusedWarps * k * 32 * 4;
-    L.cn = (L.S + (size_t)rows_max * k * 4 + 15) & ~(size_t)15;
-    L.iv = L.cn + (size_t)k * 8;
-    L.hist = L.iv + (size_t)k * 8;
+    L.hist = (L.S + (size_t)rows_max * k * 4 + 15) & ~(size_t)15;
     L.m = L.hist + (size_t)k * 4;
     L.kd = (L.m + (size_t)k * 4 + 15) & ~(size_t)15;
     L.lab = (L.kd + (size_t)rows_max * 4 + 15) & ~(size_t)15;
@@ -99,6 +105,24 @@ template <bool CACHED>
 __device__ __forceinline__ float kload(const float* p) {
     if constexpr (CACHED) return *p;
     else return __ldcg(p);
+}
+
+// Adds a float4 of K to a lane's bins: the four bins are loaded together and equal labels are
+// chained in registers (the same additions in the same order as one after the other).
+__device__ __forceinline__ void add4(float* __restrict__ b, const uchar4& l, const float4& v) {
+    float* p0 = b + l.x * 32;
+    float* p1 = b + l.y * 32;
+    float* p2 = b + l.z * 32;
+    float* p3 = b + l.w * 32;
+    const float a0 = *p0, a1 = *p1, a2 = *p2, a3 = *p3;
+    const float r0 = a0 + v.x;
+    const float r1 = (l.y == l.x ? r0 : a1) + v.y;
+    const float r2 = (l.z == l.y ? r1 : l.z == l.x ? r0 : a2) + v.z;
+    const float r3 = (l.w == l.z ? r2 : l.w == l.y ? r1 : l.w == l.x ? r0 : a3) + v.w;
+    *p0 = r0;
+    *p1 = r1;
+    *p2 = r2;
+    *p3 = r3;
 }
 
 // S_ic of rows [lo, hi) into S[(i - lo) k + c], from the labels in lab_s; rows of K from
@@ -124,19 +148,13 @@ __device__ void row_sums(const FusedArgs& a, int lo, int hi, const uint8_t* __re
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const uchar4 l4 = *reinterpret_cast<const uchar4*>(lab_s + 4 * (q + 32 * u));
-                b[l4.x * 32 + lane] += v[u].x;
-                b[l4.y * 32 + lane] += v[u].y;
-                b[l4.z * 32 + lane] += v[u].z;
-                b[l4.w * 32 + lane] += v[u].w;
+                add4(b + lane, l4, v[u]);
             }
         }
         for (; q < n4; q += 32) {
             const float4 v = kload4<CACHED>(row4 + q);
             const uchar4 l4 = *reinterpret_cast<const uchar4*>(lab_s + 4 * q);
-            b[l4.x * 32 + lane] += v.x;
-            b[l4.y * 32 + lane] += v.y;
-            b[l4.z * 32 + lane] += v.z;
-            b[l4.w * 32 + lane] += v.w;
+            add4(b + lane, l4, v);
         }
         for (int j = 4 * n4 + lane; j < n; j += 32) b[lab_s[j] * 32 + lane] += kload<CACHED>(row + j);
         __syncwarp();
@@ -151,60 +169,74 @@ __device__ void row_sums(const FusedArgs& a, int lo, int hi, const uint8_t* __re
     }
 }
 
-// The CTA's FP64 partials of sum_{i in L_c} S_ic over its rows, in row order.
+// Per-cluster values every thread of the CTA reads.
+struct ClusterVals {
+    double cn[kFusedMaxK], iv[kFusedMaxK];   // ||c_c||^2, 1/|L_c|
+    double jc[kFusedMaxK];                   // (1/m_c) sum_{i in L_c} S_ic
+    float cn32[kFusedMaxK], iv32[kFusedMaxK];
+    double J;
+};
+
+// The CTA's FP64 partials of sum_{i in L_c} S_ic over its rows, in row order (threads 0 .. k - 1),
+// and 1/|L_c| (the next warp).
 __device__ void z_partials(const FusedArgs& a, int lo, int hi, const uint8_t* __restrict__ lab_s,
-                           const float* __restrict__ S) {
-    const int k = a.k;
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        double t = 0.0;
+                           const float* __restrict__ S, const int* __restrict__ m, ClusterVals& cv) {
+    const int k = a.k, t = (int)threadIdx.x;
+    if (t < k) {
+        double z = 0.0;
+#pragma unroll 4
         for (int i = lo; i < hi; ++i)
-            if ((int)lab_s[i] == c) t += (double)S[(size_t)(i - lo) * k + c];
-        a.zpart[(size_t)blockIdx.x * k + c] = t;
+            if ((int)lab_s[i] == t) z += (double)S[(size_t)(i - lo) * k + t];
+        a.zpart[(size_t)blockIdx.x * k + t] = z;
+    } else if (t >= 32 && t < 32 + k) {
+        const double mc = (double)m[t - 32];
+        const double inv = mc > 0 ? 1.0 / mc : 0.0;
+        cv.iv[t - 32] = inv;
+        cv.iv32[t - 32] = (float)inv;
     }
 }
 
 // After barrier 1, in every CTA: sum_{i in L_c} S_ic from the partials (warp w takes
 // clusters w, w + 16, ...; lanes split the CTAs, a butterfly adds them: the same order in
-// every CTA), ||c_c||^2 = (1/m_c^2) sum (Eq. 13/14), 1/m_c, and
-// J = trace K - sum_c (1/m_c) sum_{i in L_c} S_ic.  CTA 0 also stores them where the pass
-// kernels would.  Returns J.
-__device__ double finalize(const FusedArgs& a, const int* __restrict__ m, double trace, double* cn_s,
-                           double* iv_s) {
-    __shared__ double jpart[kFusedWarps];
+// every CTA) and ||c_c||^2 = (1/m_c^2) sum (Eq. 13/14).  CTA 0 also stores them where the pass
+// kernels would.
+__device__ void finalize(const FusedArgs& a, ClusterVals& cv) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int k = a.k, G = gridDim.x;
-    double jw = 0.0;
     for (int c = warp; c < k; c += kFusedWarps) {
         double t = 0.0;
         for (int b = lane; b < G; b += 32) t += __ldcg(a.zpart + (size_t)b * k + c);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        const double mc = (double)m[c];
-        const double inv = mc > 0 ? 1.0 / mc : 0.0;
         if (lane == 0) {
-            cn_s[c] = t * inv * inv;
-            iv_s[c] = inv;
+            const double inv = cv.iv[c], cn = t * inv * inv;
+            cv.cn[c] = cn;
+            cv.cn32[c] = (float)cn;
+            cv.jc[c] = t * inv;
             if (blockIdx.x == 0) {
                 a.zsum[c] = t;
                 a.invm[c] = inv;
-                a.cnorm[c] = t * inv * inv;
+                a.cnorm[c] = cn;
             }
         }
-        jw += t * inv;
     }
-    if (lane == 0) jpart[warp] = jw;
     __syncthreads();
-    double J = trace;
-    for (int w = 0; w < kFusedWarps; ++w) J -= jpart[w];
-    __syncthreads();   // jpart is reused by the next call
-    return J;
+}
+
+// J = trace K - sum_c (1/m_c) sum_{i in L_c} S_ic, clusters in order, by the CTA's last thread
+// (read by the others after the next __syncthreads).
+__device__ __forceinline__ void objective(const FusedArgs& a, double trace, ClusterVals& cv) {
+    if (threadIdx.x == kFusedThreads - 1) {
+        double J = trace;
+        for (int c = 0; c < a.k; ++c) J -= cv.jc[c];
+        cv.J = J;
+    }
 }
 
 // Distances and argmin for rows [lo, hi) (thread t: row lo + t), new labels, and into the
 // CTA's slot the histogram of its new labels and its number of changed labels.
 __device__ void assign_rows(const FusedArgs& a, int lo, int hi, const float* __restrict__ S,
-                            const double* __restrict__ cn_s, const double* __restrict__ iv_s,
-                            const int* __restrict__ m, int* hist, const uint8_t* __restrict__ lab_s,
+                            const ClusterVals& cv, const int* __restrict__ m, int* hist, const uint8_t* __restrict__ lab_s,
                             const float* __restrict__ kd_s, int* hslot, int* cslot) {
     const int k = a.k;
     for (int c = threadIdx.x; c < k; c += blockDim.x) hist[c] = 0;
@@ -216,17 +248,47 @@ __device__ void assign_rows(const FusedArgs& a, int lo, int hi, const float* __r
         const bool own = i < hi;
         if (own) {
             const int li = lab_s[i];
-            const double kd = (double)kd_s[i - lo];
-            double best = cuda::std::numeric_limits<double>::infinity();
+            const float* Si = S + (size_t)(i - lo) * k;
             int bi = li;
-            for (int c = 0; c < k; ++c) {
-                const double E = (double)S[(size_t)(i - lo) * k + c] * iv_s[c];   // (K V^T)_ic
-                if (a.E_out) a.E_out[(int64_t)i * k + c] = (float)E;
-                if (m[c] == 0) continue;
-                const double D = fma(-2.0, E, kd + cn_s[c]);
-                if (D < best) {
-                    best = D;
-                    bi = c;
+            // screened in FP32 (the rule and its bound: assign_body, iterate.cu)
+            bool decided = false;
+            if (!a.E_out) {
+                const float kd = kd_s[i - lo];
+                float b1 = cuda::std::numeric_limits<float>::infinity(), b2 = b1, emax = 0.f, cmax = 0.f;
+                int c1 = li;
+#pragma unroll 4
+                for (int c = 0; c < k; ++c) {
+                    if (m[c] == 0) continue;
+                    const float E = Si[c] * cv.iv32[c];
+                    const float D = fmaf(-2.f, E, kd + cv.cn32[c]);
+                    emax = fmaxf(emax, fabsf(E));
+                    cmax = fmaxf(cmax, fabsf(cv.cn32[c]));
+                    if (D < b1) {
+                        b2 = b1;
+                        b1 = D;
+                        c1 = c;
+                    } else if (D < b2) {
+                        b2 = D;
+                    }
+                }
+                const float B = 16.f * 0x1p-24f * (fabsf(kd) + cmax + emax);
+                if (b2 - b1 > 2.f * B) {
+                    bi = c1;
+                    decided = true;
+                }
+            }
+            if (!decided) {
+                const double kd = (double)kd_s[i - lo];
+                double best = cuda::std::numeric_limits<double>::infinity();
+                for (int c = 0; c < k; ++c) {
+                    const double E = (double)Si[c] * cv.iv[c];   // (K V^T)_ic
+                    if (a.E_out) a.E_out[(int64_t)i * k + c] = (float)E;
+                    if (m[c] == 0) continue;
+                    const double D = fma(-2.0, E, kd + cv.cn[c]);
+                    if (D < best) {
+                        best = D;
+                        bi = c;
+                    }
                 }
             }
             newl = bi;
@@ -268,8 +330,7 @@ __device__ void fit_body(const FusedArgs& a, unsigned char* smem) {
     const FusedLayout L = fused_layout(a.n, a.k, a.rows_max, a.ldk, CACHED ? 1 : 0);
     float* bins = reinterpret_cast<float*>(smem + L.bins);
     float* S = reinterpret_cast<float*>(smem + L.S);
-    double* cn_s = reinterpret_cast<double*>(smem + L.cn);
-    double* iv_s = reinterpret_cast<double*>(smem + L.iv);
+    __shared__ ClusterVals cv;
     int* hist = reinterpret_cast<int*>(smem + L.hist);
     int* m_s = reinterpret_cast<int*>(smem + L.m);
     float* kd_s = reinterpret_cast<float*>(smem + L.kd);
@@ -297,13 +358,13 @@ __device__ void fit_body(const FusedArgs& a, unsigned char* smem) {
         for (int q = threadIdx.x; q < nl16; q += blockDim.x)
             reinterpret_cast<uint4*>(lab_s)[q] = __ldcg(reinterpret_cast<const uint4*>(a.lab8) + q);
     };
-    // S, the CTA's z partials and exchange A; then in every CTA ||c||^2, 1/|L_c| and J
-    auto reduce = [&](double* J) -> bool {
+    // S, the CTA's z partials and exchange A; then in every CTA ||c||^2 and 1/|L_c|
+    auto reduce = [&]() -> bool {
         row_sums<CACHED>(a, lo, hi, lab_s, bins, S, Kc);
         __syncthreads();
-        z_partials(a, lo, hi, lab_s, S);
+        z_partials(a, lo, hi, lab_s, S, m_s, cv);
         if (!gsync::grid_barrier(bar, err, a.wait_ns)) return false;
-        *J = finalize(a, m_s, trace, cn_s, iv_s);
+        finalize(a, cv);
         return true;
     };
     load_labels();
@@ -314,14 +375,15 @@ __device__ void fit_body(const FusedArgs& a, unsigned char* smem) {
     bool done = max_iter <= 0;
     if (a.stall && blockIdx.x == 0) return;   // the test hook: this CTA never arrives
     while (!done) {
-        double J;
-        if (!reduce(&J)) return;
+        if (!reduce()) return;
+        objective(a, trace, cv);
+        assign_rows(a, lo, hi, S, cv, m_s, hist, lab_s, kd_s, hslot, cslot);
+        if (!gsync::grid_barrier(bar, err, a.wait_ns)) return;
+        const double J = cv.J;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             a.J_hist[it] = J;
             st->J_last = J;
         }
-        assign_rows(a, lo, hi, S, cn_s, iv_s, m_s, hist, lab_s, kd_s, hslot, cslot);
-        if (!gsync::grid_barrier(bar, err, a.wait_ns)) return;
         // exchange B: the next pass's labels (loaded whether or not there is one), its counts
         // and this pass's change count; then the loop decision, taken alike in every CTA
         // (iterate.cu's assign pass)
@@ -355,9 +417,9 @@ __device__ void fit_body(const FusedArgs& a, unsigned char* smem) {
         if (blockIdx.x == 0 && threadIdx.x == 0) st->J_eval = J_last;
         return;
     }
-    double J;
-    if (!reduce(&J)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) st->J_eval = J;
+    if (!reduce()) return;
+    objective(a, trace, cv);
+    if (blockIdx.x == 0 && threadIdx.x == kFusedThreads - 1) st->J_eval = cv.J;
 }
 
 __global__ void __launch_bounds__(kFusedThreads, 1) fit_fused_kernel(FusedArgs a) {
