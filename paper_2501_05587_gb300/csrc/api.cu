@@ -342,7 +342,9 @@ popcorn_status fit_recompute(const float* P, int64_t n, int32_t d, int64_t ldp, 
     POPCORN_TRY(ws.alloc(&rb.blockhist, (size_t)nb * k, "sort histograms"));
     POPCORN_TRY(ws.alloc(&rb.blockoff, (size_t)nb * k, "sort offsets"));
     POPCORN_TRY(ws.alloc(&rb.maxkn, 1, "largest row exponent"));
+    POPCORN_TRY(ws.alloc(&rb.crange, (size_t)k, "cluster slots"));
     PassBuffers b{};
+    b.crange = rb.crange;
     float* kdiag;
     POPCORN_TRY(ws.alloc(&kdiag, (size_t)ni, "diag(K)"));
     const size_t nlab = ((size_t)ni + 15) & ~(size_t)15;

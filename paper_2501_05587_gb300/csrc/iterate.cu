@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(kReduceMaxWarps * 32, 2) reduce_kernel(ReduceA
 
 struct AssignArgs {
     int n, k, nseg;
+    const int2* crange;    // recompute path: the slots [x, y] that hold cluster c (null: all nseg)
     const float* Spart;
     const float* kdiag;
     const double* cnorm;
@@ -279,6 +280,39 @@ struct AssignArgs {
     int32_t* changed_hist;
     float* E_out;
 };
+
+// The float-float sums of clusters c0 .. c0 + 7 of a row over its slots, in slot order; the loads
+// of a slot (with crange: of each cluster's first two) are in flight together.
+__device__ __forceinline__ void slot_sums(const AssignArgs& a, const float* Si, int c0, float (&hi)[8], float (&lo)[8]) {
+    const size_t cs = (size_t)a.n, ss = (size_t)a.k * a.n;
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) hi[u] = lo[u] = 0.f;
+    if (!a.crange) {
+        for (int s = 0; s < a.nseg; ++s) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = c0 + u < a.k ? Si[s * ss + (size_t)(c0 + u) * cs] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ff_add(hi[u], lo[u], v[u]);
+        }
+        return;
+    }
+    int2 r[8];
+    float w[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) r[u] = c0 + u < a.k ? __ldg(a.crange + c0 + u) : make_int2(1, 0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        v[u] = r[u].x <= r[u].y ? Si[r[u].x * ss + (size_t)(c0 + u) * cs] : 0.f;
+        w[u] = r[u].x < r[u].y ? Si[(r[u].x + 1) * ss + (size_t)(c0 + u) * cs] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        ff_add(hi[u], lo[u], v[u]);
+        ff_add(hi[u], lo[u], w[u]);
+        for (int s = r[u].x + 2; s <= r[u].y; ++s) ff_add(hi[u], lo[u], Si[s * ss + (size_t)(c0 + u) * cs]);
+    }
+}
 
 // One block of the distance/argmin pass: rows [block * blockDim, ...), and
 // the pass's loop control when this is the last of nblocks blocks to finish.
@@ -309,7 +343,6 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
         double best = cuda::std::numeric_limits<double>::infinity();
         int bi = li;
         const float* Si = a.Spart + i;               // [s][c][i]: consecutive threads, consecutive rows
-        const size_t cs = (size_t)n, ss = (size_t)k * n;
         // The argmin in FP32, screened: GB300 runs FP64 at a small fraction of the FP32 rate,
         // and a pass has n k distances.  Each FP32 distance is within
         //   B = 16 u (|K_ii| + max_c ||c||^2 + max_c |E_ic|),  u = 2^-24,
@@ -319,7 +352,7 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
         // (near-ties) the row is decided in FP64 below.
         // E on request: (hi + lo) / |L_c| with the reciprocal as a pair of floats too, 2^-46 off
         // the FP64 product before its rounding to FP32.  (In FP64, with the argmin, and stored a
-        // float at a time, an assignment at n = 10,007, k = 32 took 111 us; now 61.)
+        // float at a time, the argmin at n = 10,007, k = 32 took 111 us; now 60.)
         bool decided = false;
         const bool evec = a.E_out && (k & 3) == 0 && ((uintptr_t)a.E_out & 15) == 0;
         {
@@ -327,21 +360,8 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
             float b1 = cuda::std::numeric_limits<float>::infinity(), b2 = b1, emax = 0.f, cmax = 0.f;
             int c1 = li;
             for (int c0 = 0; c0 < k; c0 += 8) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = c0 + u < k ? Si[(size_t)(c0 + u) * cs] : 0.f;
                 float hi[8], lo[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    hi[u] = lo[u] = 0.f;
-                    ff_add(hi[u], lo[u], v[u]);
-                }
-                for (int s = 1; s < a.nseg; ++s) {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) v[u] = c0 + u < k ? Si[s * ss + (size_t)(c0 + u) * cs] : 0.f;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) ff_add(hi[u], lo[u], v[u]);
-                }
+                slot_sums(a, Si, c0, hi, lo);
                 if (a.E_out) {
                     float e[8];
 #pragma unroll
@@ -385,19 +405,10 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
                 decided = true;
             }
         }
-        // 8 clusters at a time: their segment sums are loaded before any is used, so a thread
-        // keeps 8 loads in flight instead of one (the same additions in the same order)
+        // near-ties in FP64, from the same sums
         for (int c0 = 0; c0 < k && !decided; c0 += 8) {
             float hi[8], lo[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) hi[u] = lo[u] = 0.f;
-            for (int s = 0; s < a.nseg; ++s) {
-                float v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = c0 + u < k ? Si[s * ss + (size_t)(c0 + u) * cs] : 0.f;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) ff_add(hi[u], lo[u], v[u]);
-            }
+            slot_sums(a, Si, c0, hi, lo);
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const int c = c0 + u;
@@ -467,6 +478,7 @@ __global__ void __launch_bounds__(kAssignThreads) assign_kernel(AssignArgs a) {
 // (deterministic), then the last block finalizes the pass.
 struct ZArgs {
     int n, k, nseg;
+    const int2* crange;
     const float* Spart;
     const uint8_t* lab8;
     double* zpart;
@@ -504,7 +516,9 @@ __device__ __forceinline__ void zreduce_body(const ZArgs& a, int block, int nblo
         l = a.lab8[i];
         const float* Si = a.Spart + (size_t)l * a.n + i;
         float hi = 0.f, lo = 0.f;
-        for (int s = 0; s < a.nseg; ++s) ff_add(hi, lo, Si[(size_t)s * a.k * a.n]);
+        const int2 r = a.crange ? __ldg(a.crange + l) : make_int2(0, a.nseg - 1);
+#pragma unroll 4
+        for (int s = r.x; s <= r.y; ++s) ff_add(hi, lo, Si[(size_t)s * a.k * a.n]);
         v = (double)hi + (double)lo;
     }
     __syncthreads();
@@ -756,6 +770,7 @@ cudaError_t launch_zreduce(const PassBuffers& b, int nseg, int eval, cudaStream_
     a.n = b.n;
     a.k = b.k;
     a.nseg = nseg;
+    a.crange = b.crange;
     a.Spart = b.Spart;
     a.lab8 = b.lab8;
     a.zpart = b.zpart;
@@ -781,6 +796,7 @@ cudaError_t launch_assign(const PassBuffers& b, const ReducePlan& plan, cudaStre
     a.n = b.n;
     a.k = b.k;
     a.nseg = plan.nseg;
+    a.crange = b.crange;
     a.Spart = b.Spart;
     a.kdiag = b.kdiag;
     a.cnorm = b.cnorm;
@@ -869,6 +885,7 @@ __global__ void __launch_bounds__(kZReduceRows) batched_zreduce_kernel(const Bat
     a.n = b.n;
     a.k = b.k;
     a.nseg = b.nseg;
+    a.crange = nullptr;
     a.Spart = b.Spart;
     a.lab8 = b.lab8;
     a.zpart = b.zpart;
@@ -889,6 +906,7 @@ __global__ void __launch_bounds__(kAssignThreads) batched_assign_kernel(const Ba
     a.n = b.n;
     a.k = b.k;
     a.nseg = b.nseg;
+    a.crange = nullptr;
     a.Spart = b.Spart;
     a.kdiag = b.kdiag;
     a.cnorm = b.cnorm;

@@ -317,6 +317,7 @@ struct RecomputeBuffers {
     uint8_t* slab;        // ncols labels in cluster order (0xFF on padding)
     int* blockhist;       // sort blocks x k
     int* blockoff;        // sort blocks x k
+    int2* crange;         // [k] first and last Spart slot of a cluster (PassBuffers.crange)
     int* maxkn;           // bits of max_i |c2| r_i (Gaussian; zeroed before quantize)
 };
 
@@ -360,6 +361,7 @@ struct PassBuffers {
     float* E_out;         // optional n x k
     uint8_t* sym_meta;    // sorted form of the symmetric pass: the label-sorted lists of every block; block-row
                           // pass: the label records
+    const int2* crange;   // recompute path: cluster c's sums are in Spart slots [x, y] only (none: x > y); else null
     const int* sym_order; // symmetric pass: super-tiles in processing order (larger first), or null
 };
 
