@@ -783,8 +783,8 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
                            plan_reduce_tiles(ni, k, dev->sms, &plan);
     const int64_t tri_tiles = (int64_t)((ni + 127) / 128) * ((ni + 127) / 128 + 1) / 2;
     // A half K read as the full square (k > kSymMaxK, or k_pass = 2) goes through the tensor
-    // cores, as batched mode's one-instance form: every tile of the square in the half tile
-    // layout, each 128-row block's tiles MMA'd against the one-hot label operands with the
+    // cores, as batched mode's one-instance form: the packed triangle of half tiles, each
+    // 128-row block's tiles (those below the diagonal transposed) MMA'd against the one-hot label operands with the
     // row sums in TMEM, one segment, then the z reduction.  Taken when the K build runs on
     // the tensor cores (they write no row-major half K) or K outgrows L2; below that the
     // CUDA-core full-square pass reads the row-major half K.
@@ -802,7 +802,7 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     sym.packed = use_sym;
     const size_t k_bytes = sym.packed ? (size_t)sym.items * 128 * 128 * kelem
                            : use_tiles ? (size_t)tri_tiles * 128 * 128 * kelem
-                           : mma_full ? (size_t)Tf * Tf * 32768
+                           : mma_full ? (size_t)tri_tiles * 32768
                                       : (size_t)ni * (size_t)ldk * kelem;
     const int nslots = use_sym ? sym.nslots : mma_full ? 1 : plan.nseg;
     if (use_sym || mma_full) plan.nseg = 1;   // the assignment reads one (folded) segment
@@ -810,7 +810,6 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     if (mma_full) {
         bpf.count = 1;
         bpf.half = ks;
-        bpf.htiles = (long long)Tf * Tf;
         bpf.vblocks = Tf;
         bpf.nunits = Tf;
         bpf.Nmax = (k + 15) / 16 * 16;
@@ -927,34 +926,30 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     }
     POPCORN_CUDA(cudaMemsetAsync(b.counts, 0, 2 * (size_t)k * sizeof(int32_t), s));
     POPCORN_CUDA(launch_init_state(b.st, max_iter, opt.check_convergence ? 1 : 0, tol, s));
-    if (sym.packed && sym.ebytes == 2 && opt.precision != POPCORN_FP32) {
+    if (((sym.packed && sym.ebytes == 2) || mma_full) && opt.precision != POPCORN_FP32) {
         // half layout from the tensor-core build: its epilogue rounds and stores the tiles
         POPCORN_TRY(build_kernel_matrix(Pd, ni, d, ldpd, kp, opt.precision, K, ldk, ks, kdiag, &ws,
                                         &b.st->wait_err, dev->sms, s, &launches, kPackedSw128H));
-    } else if (sym.packed && sym.ebytes == 2) {
+    } else if ((sym.packed && sym.ebytes == 2) || mma_full) {
         // half layout from the FP32 build: it writes the FP32 triangle into a temporary, one
         // pack launch rounds it into K (and rounds diag K with it), and the temporary goes back
         float* kf;
-        POPCORN_TRY(ws.alloc(&kf, (size_t)sym.items * 128 * 128, "FP32 kernel matrix"));
+        POPCORN_TRY(ws.alloc(&kf, (size_t)tri_tiles * 128 * 128, "FP32 kernel matrix"));
         POPCORN_TRY(build_kernel_matrix(Pd, ni, d, ldpd, kp, opt.precision, kf, ldk, POPCORN_K_FP32, kdiag, &ws,
                                         &b.st->wait_err, dev->sms, s, &launches, kPackedSw4));
         POPCORN_CUDA(launch_pack_half(kf, K, ks, ni, kdiag, s));
         ++launches;
         ws.release(kf);
-    } else if (mma_full) {
-        // the FP32 square (either build) into a temporary, rounded into the half tiles of K by
-        // the batched pack kernel (diag K with it); the temporary goes back
-        const int64_t ld32 = (n + 3) / 4 * 4;
-        float* kf;
-        POPCORN_TRY(ws.alloc(&kf, (size_t)ni * ld32, "FP32 kernel matrix"));
-        POPCORN_TRY(build_kernel_matrix(Pd, ni, d, ldpd, kp, opt.precision, kf, ld32, POPCORN_K_FP32, kdiag, &ws,
-                                        &b.st->wait_err, dev->sms, s, &launches));
+    } else {
+        POPCORN_TRY(build_kernel_matrix(Pd, ni, d, ldpd, kp, opt.precision, K, ldk, ks, kdiag, &ws,
+                                        &b.st->wait_err, dev->sms, s, &launches,
+                                        sym.packed ? sym.layout : use_tiles ? kPackedSw4 : 0));
+    }
+    if (mma_full) {
         POPCORN_TRY(ws.alloc(&Vf, (size_t)Tf * bpf.Nmax * 256, "one-hot operands"));
         BatchInst hf;
         memset(&hf, 0, sizeof hf);
         hf.T = Tf;
-        hf.K = kf;
-        hf.ldk = ld32;
         hf.kdiag = kdiag;
         hf.n = ni;
         hf.k = k;
@@ -973,13 +968,6 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
         POPCORN_TRY(ws.alloc(&unitsf, (size_t)Tf, "row-block units"));
         POPCORN_CUDA(cudaMemcpyAsync(dIf, &hf, sizeof hf, cudaMemcpyHostToDevice, s));
         POPCORN_CUDA(cudaMemcpyAsync(unitsf, hu.data(), sizeof(int2) * hu.size(), cudaMemcpyHostToDevice, s));
-        POPCORN_CUDA(launch_batched_pack_half(dIf, bpf, s));
-        ++launches;
-        ws.release(kf);
-    } else {
-        POPCORN_TRY(build_kernel_matrix(Pd, ni, d, ldpd, kp, opt.precision, K, ldk, ks, kdiag, &ws,
-                                        &b.st->wait_err, dev->sms, s, &launches,
-                                        sym.packed ? sym.layout : use_tiles ? kPackedSw4 : 0));
     }
     POPCORN_CUDA(launch_trace(kdiag, ni, b.st, s));
     POPCORN_CUDA(launch_init_labels(Ld, ni, k, b.lab32, b.lab8, b.counts, b.st, s));
@@ -1358,17 +1346,14 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         bp.lblocks += (n + kBatchLabelThreads - 1) / kBatchLabelThreads;
         if (k > bp.kmax) bp.kmax = k;
         const int zb = (n + kZReduceRows - 1) / kZReduceRows;
-        // FP32 K: the packed triangle the K stream reads.  Half K: the tensor-core builds write
-        // the FP32 square that the pack rounds into half tiles (the FP32 build writes those directly)
-        o[t].K = !half ? take((size_t)b.T * (b.T + 1) / 2 * 65536)
-                 : opt.precision != POPCORN_FP32 ? take((size_t)n * b.ldk * 4) : 0;
+        // the packed triangle the K stream reads, FP32 or half tiles
+        const size_t tiles = (size_t)b.T * (b.T + 1) / 2;
+        o[t].K = !half ? take(tiles * 65536) : 0;
         if (half) {
             b.N = (k + 15) / 16 * 16;
-            b.htile0 = bp.htiles;
-            bp.htiles += (long long)b.T * b.T;
             bp.nunits += b.T;
             if (b.N > bp.Nmax) bp.Nmax = b.N;
-            o_kh[t] = take((size_t)b.T * b.T * 32768);
+            o_kh[t] = take(tiles * 32768);
         }
         b.vblock0 = bp.vblocks;
         bp.vblocks += b.T;
@@ -1417,7 +1402,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     POPCORN_TRY(ws.alloc(&base, bytes, "batch workspace"));
     for (int t = 0; t < count; ++t) {
         BatchInst& b = h[t];
-        b.K = (!half || opt.precision != POPCORN_FP32) ? reinterpret_cast<float*>(base + o[t].K) : nullptr;
+        b.K = !half ? reinterpret_cast<float*>(base + o[t].K) : nullptr;
         b.kdiag = reinterpret_cast<float*>(base + o[t].kdiag);
         b.lab32 = reinterpret_cast<int32_t*>(base + o[t].lab32);
         b.lab8 = base + o[t].lab8;
@@ -1564,15 +1549,11 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     } else {
         for (int t = 0; t < count && cap == POPCORN_OK; ++t) {
             const BatchInst& b = h[t];
-            step(launch_kbuild_tc(b.P, b.n, b.d, b.ldp, b.kp, opt.precision, b.K, b.ldk, b.kdiag, base + tc_off, err,
-                                  dev->sms, cs, &launches, half ? 0 : kPackedSw4),
+            step(launch_kbuild_tc(b.P, b.n, b.d, b.ldp, b.kp, opt.precision,
+                                  half ? reinterpret_cast<float*>(b.Kh) : b.K, b.ldk, b.kdiag, base + tc_off, err,
+                                  dev->sms, cs, &launches, half ? kPackedSw128H : kPackedSw4, 0, half),
                  "tensor-core K build");
         }
-    }
-    if (half && opt.precision != POPCORN_FP32) {
-        // the tensor-core builds write FP32 squares: rounded into half tiles (diag K too)
-        step(launch_batched_pack_half(dI, bp, cs), "batched half-K pack");
-        launches += 1;
     }
     step(launch_batched_trace(dI, bp, cs), "batched trace");
     launches += 1;

@@ -6,13 +6,21 @@
 // 1 / |L_c| scale): an MMA chain of M = 128 rows, N = k rounded up to 16, reduction over
 // the instance's n columns.  A half entry times 1 or 0 is exact and the tensor cores add in
 // FP32, so S is the cluster sums of the rounded K up to the order of the FP32 additions.
-// The instances are small (n up to a few thousand), so the square is read whole: no slots,
-// no fold, S written once a row.
+// No slots, no fold: S is written once a row.
 //
-// After the build, batched_pack_half_kernel rounds each instance's FP32 square into tiles
-// of the 128-byte-swizzled half layout (kPackedSw128H: two boxes of 128 rows x 64 columns,
-// entries past n zero), tile (I, J) at Kh + (I T + J) 32 KB: the K-major A operand of the
-// MMAs as it lies in memory.  Per pass batched_onehot_kernel writes every block's one-hot
+// K is stored as the packed upper triangle in the 128-byte-swizzled half layout
+// (kPackedSw128H: two boxes of 128 rows x 64 columns, entries past n zero), written by the
+// builds' epilogues (or packed from the FP32 triangle): tile (I, J), I <= J, is the K-major A
+// operand of block I's MMAs as it lies in memory, and through the transpose bit the MN-major
+// one of block J's.  Block row I takes its columns in the order J = (s - I) mod T: blocks I
+// and J are at their tile in the same step s, so its second read comes from L2 and HBM
+// delivers half of the square a pass (as in reduce_tiles.cu).  What bounds the stream is then
+// what an SM takes in from L2 (36 bytes a clock: 32 KB of tile and up to 16 KB of one-hot
+// operand a tile).  Batch of 256 instances, n 500 to 8,000, k up to 64, BF16: 1.75 -> 1.31 ms a pass
+// (HBM 7.4 GB for the 12.1 GB of squares, which it read whole before), the build 13.6 -> 11.5 ms;
+// one fit of n = 30,011, k = 64, BF16: 0.31 -> 0.27 ms a pass, its build 4.65 -> 0.37 ms (no FP32
+// square and no pack launch).
+// Per pass batched_onehot_kernel writes every block's one-hot
 // operand, and batched_mma_kernel (persistent, one CTA an SM) takes the units (instance,
 // row block) in the caller's order: warp 0 bulk-copies each tile of the unit's block row
 // with V_J into a ring of stages, warp 1 issues 8 MMAs a tile into a TMEM accumulator
@@ -25,7 +33,6 @@
 
 #include <type_traits>
 
-#include "half_common.cuh"
 #include "popcorn_internal.cuh"
 #include "tc_common.cuh"
 
@@ -35,7 +42,6 @@ namespace {
 constexpr int kB = 128;
 constexpr int kTileBytes = 32768;
 constexpr int kMmaThreads = 192;
-constexpr int kPackThreads = 256;
 constexpr int kMaxStages = 6;
 
 // the instance holding flattened index x of a prefix field that ascends with the instance
@@ -48,56 +54,6 @@ __device__ __forceinline__ int inst_of(const BatchInst* I, int count, long long 
         else hi = mid - 1;
     }
     return lo;
-}
-
-using hstore::pack2;
-using hstore::round_trip;
-
-// One tile of one instance's square, a 64-column box at a time: the FP32 rows (row-major,
-// ldk) into shared memory, then each 32-bit word of the box (row (w >> 5), columns
-// 64 box + 8 (((w >> 2) & 7) ^ (row & 7)) + 2 (w & 3) + {0, 1}), zeros past n.
-template <typename TH>
-__global__ void __launch_bounds__(kPackThreads) batched_pack_half_kernel(const BatchInst* I, int count) {
-    __shared__ float half_tile[kB][65];   // 128 rows x 64 columns (+1 against bank conflicts)
-    const long long g = blockIdx.x;
-    const int t = inst_of(I, count, g, [](const BatchInst& x) { return x.htile0; });
-    const BatchInst& b = I[t];
-    const int lt = (int)(g - b.htile0);
-    const int bi = lt / b.T, bj = lt - bi * b.T;
-    const int rows = b.n - bi * kB, cols = b.n - bj * kB;
-    const float* src = b.K + (int64_t)bi * kB * b.ldk + (int64_t)bj * kB;
-    uint32_t* dst = reinterpret_cast<uint32_t*>(b.Kh + (size_t)lt * kTileBytes);
-    for (int box = 0; box < 2; ++box) {
-        if (box) __syncthreads();   // the previous box is written out
-        // 2048 float4 a box, 8 a thread, all loads issued before the first store
-        float4 x[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int q = threadIdx.x + kPackThreads * e;   // float4 q: row q >> 4, columns 4 (q & 15) + 0..3
-            const int r = q >> 4, c = 64 * box + 4 * (q & 15);
-            // ldk is a multiple of 4 and the rows start 16-byte aligned; a float4 past n is read
-            // only where its first column is below n (the row padding up to ldk is allocated)
-            x[e] = (r < rows && c < cols) ? __ldg(reinterpret_cast<const float4*>(src + (int64_t)r * b.ldk + c))
-                                          : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int q = threadIdx.x + kPackThreads * e;
-            const int r = q >> 4, c = 4 * (q & 15), c0 = 64 * box + c;
-            half_tile[r][c] = x[e].x;
-            half_tile[r][c + 1] = c0 + 1 < cols ? x[e].y : 0.f;
-            half_tile[r][c + 2] = c0 + 2 < cols ? x[e].z : 0.f;
-            half_tile[r][c + 3] = c0 + 3 < cols ? x[e].w : 0.f;
-        }
-        __syncthreads();
-        if (bi == bj && threadIdx.x < rows && (threadIdx.x >> 6) == box)
-            b.kdiag[bi * kB + threadIdx.x] = round_trip<TH>(half_tile[threadIdx.x][threadIdx.x & 63]);
-        for (int w = threadIdx.x; w < 4096; w += kPackThreads) {
-            const int r = w >> 5;
-            const int c = 8 * (((w >> 2) & 7) ^ (r & 7)) + 2 * (w & 3);
-            dst[4096 * box + w] = pack2<TH>(half_tile[r][c], half_tile[r][c + 1]);
-        }
-    }
 }
 
 // One 128-block's one-hot operand: V[c][i] = 1 if point 128 X + i has label c (0 past n),
@@ -124,13 +80,6 @@ __global__ void __launch_bounds__(kB) batched_onehot_kernel(const BatchInst* I, 
             w[e] = (lab[i0 + 2 * e] == c ? one : 0u) | ((lab[i0 + 2 * e + 1] == c ? one : 0u) << 16);
         dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
     }
-}
-
-// kind::f16 instruction descriptor, FP32 accumulate, A and B both FP16 or both BF16, both
-// K-major; N >> 3 at bit 17, M >> 4 at bit 24.
-__device__ __forceinline__ uint32_t idesc_half_kmajor(bool bf16, int N) {
-    return (1u << 4) | ((bf16 ? 1u : 0u) << 7) | ((bf16 ? 1u : 0u) << 10) | ((uint32_t)(N >> 3) << 17) |
-           ((uint32_t)(kB >> 4) << 24);
 }
 
 struct BatchedMmaArgs {
@@ -193,7 +142,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) batched_mma_kernel(BatchedMmaA
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- producer: the tiles of the unit's block row with their V_J
-            const uint64_t stream_once = tc::l2_evict_first();   // each tile is read once a pass
             const long long skip = blockIdx.x == 0 ? (long long)a.stall_block - 1 : -1;
             long long t = 0;
             int s = 0;
@@ -204,7 +152,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) batched_mma_kernel(BatchedMmaA
                 const BatchInst& b = a.I[w.x];
                 if (pass_skip(b.st, a.eval)) continue;
                 const uint32_t vbytes = (uint32_t)b.N * kB * 2;
-                for (int J = 0; J < b.T; ++J) {
+                for (int x = 0; x < b.T; ++x) {
+                    const int I = w.y, J = x >= I ? x - I : x - I + b.T, lo = min(I, J);
                     if (t >= S && !tc::mbar_wait_for(empty_bar(s), ph ^ 1u, abort_flag, a.err, a.wait_ns)) {
                         ok = false;
                         break;
@@ -212,8 +161,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) batched_mma_kernel(BatchedMmaA
                     if (t != skip) {   // the test hook: this tile never arrives
                         tc::mbar_arrive_expect_tx(full_bar(s), (uint32_t)kTileBytes + vbytes);
                         const uint32_t dst = sbase + (uint32_t)s * (uint32_t)a.stage_bytes;
-                        tc::bulk_load_1d_hint(dst, b.Kh + ((size_t)w.y * b.T + J) * kTileBytes,
-                                              (uint32_t)kTileBytes, full_bar(s), stream_once);
+                        const size_t tri = (size_t)lo * b.T - (size_t)lo * (lo - 1) / 2 + (size_t)(max(I, J) - lo);
+                        tc::bulk_load_1d(dst, b.Kh + tri * kTileBytes, (uint32_t)kTileBytes, full_bar(s));
                         tc::bulk_load_1d(dst + kTileBytes, b.V + (size_t)J * vbytes, vbytes, full_bar(s));
                     }
                     ++t;
@@ -254,9 +203,11 @@ __global__ void __launch_bounds__(kMmaThreads, 1) batched_mma_kernel(BatchedMmaA
                 }
                 tc::tc_fence_after();
                 const int N = b.N;
-                const uint32_t idesc = idesc_half_kmajor(BF16, N);
+                const uint32_t idesc_row = tc::idesc_half(BF16, false, kB, N), idesc_col = tc::idesc_half(BF16, true, kB, N);
                 const uint32_t d = tmem + (uint32_t)buf * half_cols;
-                for (int J = 0; J < b.T; ++J) {
+                for (int x = 0; x < b.T; ++x) {
+                    const int J = x >= w.y ? x - w.y : x - w.y + b.T;
+                    const bool rows = w.y <= J;
                     if (!tc::mbar_wait_for(full_bar(s), ph, abort_flag, a.err, a.wait_ns)) {
                         ok = false;
                         break;
@@ -264,11 +215,21 @@ __global__ void __launch_bounds__(kMmaThreads, 1) batched_mma_kernel(BatchedMmaA
                     tc::tc_fence_after();
                     const uint32_t st = sbase + (uint32_t)s * (uint32_t)a.stage_bytes;
                     const uint32_t v = st + kTileBytes;
+                    if (rows) {
+                        // 16 columns of the tile: 32 bytes along a row, the second box 16 KB on
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        tc::mma_bf16(d, tc::sw128_desc(st + (kk >> 2) * 16384 + (kk & 3) * 32),
-                                     tc::sw128_desc(v + (kk >> 2) * (N * 128) + (kk & 3) * 32), idesc,
-                                     (J | kk) ? 1u : 0u);
+                        for (int kk = 0; kk < 8; ++kk)
+                            tc::mma_bf16(d, tc::sw128_desc(st + (kk >> 2) * 16384 + (kk & 3) * 32),
+                                         tc::sw128_desc(v + (kk >> 2) * (N * 128) + (kk & 3) * 32), idesc_row,
+                                         (x | kk) ? 1u : 0u);
+                    } else {
+                        // the transposed tile: 16 of its rows, 2 KB on, its two 64-column atoms 16 KB apart
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            tc::mma_bf16(d, tc::sw128_desc_mn(st + kk * 2048, 16384, 1024),
+                                         tc::sw128_desc(v + (kk >> 2) * (N * 128) + (kk & 3) * 32), idesc_col,
+                                         (x | kk) ? 1u : 0u);
+                    }
                     tc::mma_commit(empty_bar(s));   // the stage is free once these MMAs have read it
                     if (++s == S) {
                         s = 0;
@@ -362,15 +323,6 @@ cudaError_t configure_batched_mma(int smem_optin) {
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-cudaError_t launch_batched_pack_half(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s) {
-    if (bp.htiles <= 0 || bp.htiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    if (bp.half == POPCORN_K_BF16)
-        batched_pack_half_kernel<__nv_bfloat16><<<(unsigned)bp.htiles, kPackThreads, 0, s>>>(dI, bp.count);
-    else
-        batched_pack_half_kernel<__half><<<(unsigned)bp.htiles, kPackThreads, 0, s>>>(dI, bp.count);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_batched_mma_stream(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err, int eval,

@@ -296,11 +296,11 @@ __device__ __forceinline__ void kbuild_tile(const float* __restrict__ P, int n, 
     }
 
     if constexpr (PACKED == kPackedSw128H) {
-        // FP16 / BF16 square as 32 KB tiles (batched mode): tile (I, J) at K + (I T + J) 32 KB,
+        // FP16 / BF16 packed upper triangle (batched mode): 32 KB a tile in row-by-row order,
         // two boxes of 128 rows x 64 columns in the 128-byte swizzle, element (r, c) at byte
         // 16384 (c >> 6) + 128 r + 16 (((c >> 3) & 7) ^ (r & 7)) + 2 (c & 7); entries past n
         // are zeros.  A thread's 4 consecutive columns (4-aligned) are 8 bytes of one 16-byte
-        // chunk; so are its 4 consecutive rows in the transposed tile (J, I).
+        // chunk.
         static_assert(sizeof(TK) == 2, "half tiles hold FP16 / BF16 K");
         unsigned char* base = reinterpret_cast<unsigned char*>(K);
         auto off = [](int r, int c) { return 16384 * (c >> 6) + 128 * r + 16 * (((c >> 3) & 7) ^ (r & 7)) + 2 * (c & 7); };
@@ -317,7 +317,7 @@ __device__ __forceinline__ void kbuild_tile(const float* __restrict__ P, int n, 
             }
             *reinterpret_cast<uint2*>(p) = u;
         };
-        unsigned char* Bd = base + ((size_t)bi * T + bj) * 32768;
+        unsigned char* Bd = base + (size_t)tile * 32768;
 #pragma unroll
         for (int x = 0; x < RPT; ++x) {
             const int rl = ty * 4 + (x & 3) + RS * (x >> 2);
@@ -328,20 +328,6 @@ __device__ __forceinline__ void kbuild_tile(const float* __restrict__ P, int n, 
                 const float* v = &acc[x][4 * h];
                 put(Bd + off(rl, cl), rv && c < n ? v[0] : 0.f, rv && c + 1 < n ? v[1] : 0.f,
                     rv && c + 2 < n ? v[2] : 0.f, rv && c + 3 < n ? v[3] : 0.f);
-            }
-        }
-        if (bi != bj) {   // rows of block bi < bj are all below n
-            unsigned char* Bt = base + ((size_t)bj * T + bi) * 32768;
-#pragma unroll
-            for (int y = 0; y < 8; ++y) {
-                const int cl = tx * 4 + (y & 3) + 64 * (y >> 2);
-                const bool cv = col0 + cl < n;
-#pragma unroll
-                for (int g = 0; g < RPT / 4; ++g) {
-                    const int rl = RS * g + ty * 4;
-                    put(Bt + off(cl, rl), cv ? acc[4 * g][y] : 0.f, cv ? acc[4 * g + 1][y] : 0.f,
-                        cv ? acc[4 * g + 2][y] : 0.f, cv ? acc[4 * g + 3][y] : 0.f);
-                }
             }
         }
         return;
@@ -564,7 +550,7 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
 // All instances of a batch: flattened tile b belongs to the instance whose
 // tile0 is the largest one <= b.
 // TK float: each instance's FP32 block-packed triangle (K, kPackedSw4); TK __half / __nv_bfloat16:
-// its square as half tiles (Kh, kPackedSw128H), for the tensor-core batched stream.
+// its triangle of half tiles (Kh, kPackedSw128H), for the tensor-core batched stream.
 template <typename TK>
 __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst* I, int count) {
     const long long b = blockIdx.x;

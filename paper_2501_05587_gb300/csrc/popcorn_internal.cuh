@@ -422,12 +422,11 @@ struct BatchInst {
     const int32_t* init_labels;
     int32_t* labels_out;
     int zblock0, ablock0, lblock0;
-    // FP16 / BF16 K (batched_mma.cu): every tile of the square in kPackedSw128H, tile (I, J) at
-    // Kh + (I T + J) 32 KB; the per-pass one-hot operands of the T blocks, N rows each
+    // FP16 / BF16 K (batched_mma.cu): the packed triangle in kPackedSw128H; the per-pass one-hot
+    // operands of the T blocks, N rows each
     unsigned char* Kh;
     unsigned char* V;         // (FP32 K: the label records of reduce_tiles.cu)
     int N;                    // accumulator columns: k rounded up to 16
-    long long htile0;         // first flattened tile of the square
     int vblock0;              // first flattened 128-block
 };
 
@@ -440,7 +439,6 @@ struct BatchPlan {
     size_t smem;
     // FP16 / BF16 K: the tensor-core stream over (instance, row block) units
     int half;                 // 0, or the k_storage of every instance's K
-    long long htiles;         // tiles of every instance's square
     int vblocks;              // 128-blocks of every instance
     int nunits;               // (instance, row block) units
     int Nmax;                 // widest accumulator
@@ -467,15 +465,13 @@ cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const B
 cudaError_t launch_batched_finish(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
 cudaError_t launch_batched_copy_labels(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
 // FP16 / BF16 K in batched mode (batched_mma.cu).  Plan: ring depth, grid and shared memory of
-// the stream for accumulators up to Nmax columns (false if it does not fit).  Pack: every
-// instance's FP32 square (K, ldk) rounded into its half tiles Kh, diag K rounded with it.
+// the stream for accumulators up to Nmax columns (false if it does not fit).
 // Pass: the one-hot operands, then the stream over the units (instance, row block), ordered
 // by the caller (larger instances first), writing each row's k sums to Spart (one segment);
 // *err is set when a bounded wait runs out.  stall_ms > 0 (error-path tests only): CTA 0
 // leaves its first tile's copies out and every wait gives up after stall_ms.
 bool plan_batched_mma(BatchPlan* bp, int num_sms, int smem_optin);
 cudaError_t configure_batched_mma(int smem_optin);
-cudaError_t launch_batched_pack_half(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
 cudaError_t launch_batched_mma_stream(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err,
                                       int eval, cudaStream_t s, int stall_ms = 0);
 

@@ -93,27 +93,6 @@ __global__ void __launch_bounds__(kOneHotThreads) sym_onehot_kernel(const uint8_
     }
 }
 
-// Instruction descriptor of kind::f16 with FP32 accumulation: A and B both FP16 (format 0)
-// or both BF16 (format 1); A MN-major when a_mn (bit 15), B K-major; N >> 3 at bit 17,
-// M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t idesc_half(bool bf16, bool a_mn, int M, int N) {
-    return (1u << 4) | ((bf16 ? 1u : 0u) << 7) | ((bf16 ? 1u : 0u) << 10) | ((a_mn ? 1u : 0u) << 15) |
-           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// Shared-memory descriptor of an MN-major operand in the 128-byte swizzle: atoms of 64
-// elements along M (one 128-byte row) by 8 along the reduction; lbo = bytes between atoms
-// along M, sbo = bytes between groups of 8 reduction rows; version 1, swizzle mode 2.
-__device__ __forceinline__ uint64_t sw128_desc_mn(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
 // N consecutive TMEM columns of this thread's lane (32x32b shape), as floats.
 template <int N>
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[N]) {
@@ -257,8 +236,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) reduce_sym_mma_kernel(MmaArgs 
     } else if (warp == 1) {
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
-            constexpr uint32_t kIdescRow = idesc_half(BF16, false, kB, N);
-            constexpr uint32_t kIdescCol = idesc_half(BF16, true, kB, N);
+            constexpr uint32_t kIdescRow = tc::idesc_half(BF16, false, kB, N);
+            constexpr uint32_t kIdescCol = tc::idesc_half(BF16, true, kB, N);
             int s = 0;
             uint32_t ph = 0;
             int lt = 0;
@@ -300,7 +279,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) reduce_sym_mma_kernel(MmaArgs 
                             const uint32_t acc_c = (touched >> (A + y)) & 1u;
 #pragma unroll
                             for (int kk = 0; kk < 8; ++kk)
-                                tc::mma_bf16(dcol, sw128_desc_mn(st + kk * 2048, 16384, 1024),
+                                tc::mma_bf16(dcol, tc::sw128_desc_mn(st + kk * 2048, 16384, 1024),
                                              tc::sw128_desc(vI + (kk >> 2) * (N * 128) + (kk & 3) * 32), kIdescCol,
                                              (acc_c | (uint32_t)kk) ? 1u : 0u);
                             touched |= 1u << (A + y);
