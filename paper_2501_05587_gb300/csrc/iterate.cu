@@ -282,23 +282,32 @@ struct AssignArgs {
 };
 
 // The float-float sums of clusters c0 .. c0 + 7 of a row over its slots, in slot order; the loads
-// of a slot (with crange: of each cluster's first two) are in flight together.
+// of two slots (with crange: of each cluster's first two) are in flight together.
 __device__ __forceinline__ void slot_sums(const AssignArgs& a, const float* Si, int c0, float (&hi)[8], float (&lo)[8]) {
     const size_t cs = (size_t)a.n, ss = (size_t)a.k * a.n;
     float v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) hi[u] = lo[u] = 0.f;
+    float w[8];
     if (!a.crange) {
-        for (int s = 0; s < a.nseg; ++s) {
+        // two slots at a time: 16 loads in flight a thread
+        for (int s = 0; s < a.nseg; s += 2) {
+            const bool two = s + 1 < a.nseg;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = c0 + u < a.k ? Si[s * ss + (size_t)(c0 + u) * cs] : 0.f;
+            for (int u = 0; u < 8; ++u) {
+                const float* p = Si + s * ss + (size_t)(c0 + u) * cs;
+                v[u] = c0 + u < a.k ? *p : 0.f;
+                w[u] = two && c0 + u < a.k ? p[ss] : 0.f;
+            }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) ff_add(hi[u], lo[u], v[u]);
+            for (int u = 0; u < 8; ++u) {
+                ff_add(hi[u], lo[u], v[u]);
+                if (two) ff_add(hi[u], lo[u], w[u]);
+            }
         }
         return;
     }
     int2 r[8];
-    float w[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) r[u] = c0 + u < a.k ? __ldg(a.crange + c0 + u) : make_int2(1, 0);
 #pragma unroll
