@@ -216,13 +216,16 @@ def pass_roofline(wl, prof, pk, k_storage="fp32"):
 
 
 def kbuild_roofline(wl, precision, kb_ms, pk, k_storage="fp32"):
-    """Roofline of the K build.  FP32 (CUDA cores): bound by the FP32 lanes -- a Gaussian entry
+    """Roofline of the K build.  FP32 on CUDA cores: bound by the FP32 lanes -- a Gaussian entry
     takes a subtract and a multiply-add per coordinate, a polynomial / linear one a multiply-add,
     over the n (n + 1) / 2 unique pairs; peak = 128 lanes x 152 SMs x the maximum SM clock.
-    BF16 / BF16X3 (tcgen05): the executed MMA flops of the row-pair tiles (BF16X3: three
-    products per k-step) against the measured BF16 peak."""
+    On tensor cores (BF16, BF16X3, FP32 as two FP16 parts): the executed MMA flops of the tiles,
+    a row block against a pair of column blocks (BF16X3: three products per k-step, FP32: four),
+    against the measured BF16 peak."""
     n, d = float(wl.n), float(wl.d)
     sec = kb_ms / 1e3
+    T = (wl.n + 127) // 128
+    split = False
     if precision == "fp32":
         # the Gaussian's distance form, decided as the library decides it: the norm expansion
         # (one multiply-add a coordinate) when 4 sqrt(d) u max_i r_i gamma / sigma^2 <= 1e-6,
@@ -235,6 +238,11 @@ def kbuild_roofline(wl, precision, kb_ms, pk, k_storage="fp32"):
             expand = 4.0 * np.sqrt(d) * 2.0 ** -24 * maxr * c <= 1e-6
             form = "norm expansion (Eq. 12)" if expand else "coordinate differences"
             per = 1.0 if expand else 2.0
+        # the split build's lines (kbuild_split_applies, split_decide_kernel in csrc/kbuild_tc.cu)
+        fill = float(np.count_nonzero(wl.P)) / (n * d)
+        split = (max(136, T * (T + 1) // 2) * wl.d >= 65000 and per == 1.0
+                 and (wl.d >= 48 if form else wl.d >= 128 and d * fill * fill >= 128))
+    if precision == "fp32" and not split:
         ops = per * n * (n + 1) / 2 * d
         peak = FP32_LANES_PER_CLK_SM * GB300_SMS * pk["sm_mhz"] * 1e6 / 1e12
         ach = ops / sec / 1e12
@@ -246,11 +254,10 @@ def kbuild_roofline(wl, precision, kb_ms, pk, k_storage="fp32"):
                 "peak_source": f"{FP32_LANES_PER_CLK_SM} FP32 lanes/clk/SM x {GB300_SMS} SMs x "
                                f"{pk['sm_mhz']:.0f} MHz (unit counts and clock)",
                 "algorithmic_lane_ops_per_launch": ops, "avg_launch_ms": kb_ms, "distance_form": form}
-    T = (wl.n + 127) // 128
     T2 = (T + 1) // 2
-    tiles = T2 * T - T2 * (T2 - 1)
-    dpad = (wl.d + 63) // 64 * 64
-    depth = dpad * (3 if precision == "bf16x3" else 1)
+    tiles = T2 * (T2 + 1) - (T & 1)
+    block = 64 if precision == "bf16" else 32
+    depth = (wl.d + block - 1) // block * block * {"bf16": 1, "bf16x3": 3, "fp32": 4}[precision]
     flops = tiles * 2.0 * 128 * 128 * 2.0 * depth
     ach = flops / sec / 1e12
     return {"kernel": "kbuild_tc_kernel", "bound": "tensor", "achieved": ach, "peak": pk["bf16"], "unit": "TFLOP/s",

@@ -77,7 +77,10 @@ typedef struct {
 
 /* Arithmetic used to form B = P P^T for the kernel matrix. */
 typedef enum {
-    POPCORN_FP32 = 0,    /* FP32 CUDA-core arithmetic; Gaussian distances from coordinate differences */
+    POPCORN_FP32 = 0,    /* FP32: multiply-adds on CUDA cores, or, where the device finds it as exact, tensor
+                            cores on the points split into two FP16 parts, FP32 accumulate; Gaussian
+                            distances by the norm expansion where its error bound allows, else from
+                            coordinate differences                                             */
     POPCORN_BF16 = 1,    /* tcgen05 tensor cores, BF16 operands, FP32 accumulate                       */
     POPCORN_BF16X3 = 2,  /* tcgen05, split-BF16 (hi*hi + hi*lo + lo*hi), FP32 accumulate              */
     POPCORN_FP8 = 3      /* tcgen05, FP8 E4M3 operands with per-row scales s_i = max|p_i| / 448, FP32
@@ -106,11 +109,11 @@ typedef struct {
     int32_t k_storage;          /* popcorn_k_storage of the stored K; 0 = FP32.  FP16 / BF16
                                    from any build, rounded once.  A pass reads it on the tensor
                                    cores: the symmetric pass's tensor-core form (k <= 32), or,
-                                   read as the full square (k > 32 or k_pass = 2), 32 KB half
-                                   tiles of the square with each 128-row block's row sums as
-                                   MMAs against one-hot label operands (any k; for the FP32
-                                   build from n = 8192, below which a CUDA-core pass reads a
-                                   row-major half K)                                         */
+                                   read by block rows (k > 32 or k_pass = 2), the packed
+                                   triangle of 32 KB half tiles with each 128-row block's row
+                                   sums as MMAs against one-hot label operands, tiles below the
+                                   diagonal transposed (any k; for the FP32 build from n = 8192,
+                                   below which a CUDA-core pass reads a row-major half K)    */
     int32_t autotune;           /* 1: pick the schedule by timing candidates on this workload
                                    (first call per workload signature; later calls reuse the
                                    cached choice, see popcorn_autotune_entries); 0: fixed
@@ -122,10 +125,11 @@ typedef struct {
                                    default): the symmetric read below for n >= 8192 (where K
                                    outgrows L2 and reading half of it pays; measured faster
                                    on GB300 for every k up to 32), and at every n for an
-                                   FP16 / BF16 K from a BF16 / BF16X3 build; else the full
-                                   square.
-                                   1 = symmetric (k <= 32; larger k falls back to the full
-                                   square): only the 128 x 128 blocks on and above the
+                                   FP16 / BF16 K from a BF16 / BF16X3 build; with more than 32
+                                   clusters and an FP32 K from n = 6145 the packed triangle by
+                                   block rows (each 128-block for its rows and, transposed, for
+                                   its columns, the second time from L2); else the full square.
+                                   1 = symmetric (k <= 32; larger k as under 0): only the 128 x 128 blocks on and above the
                                    diagonal (K is symmetric, and is then stored as that packed
                                    triangle; an FP16 / BF16 K is written as half tiles by a
                                    BF16 / BF16X3 build, or rounded from the FP32 build's
@@ -191,7 +195,8 @@ typedef struct {
                                   zeros otherwise                                           */
     double fold_ms;            /* symmetric pass: the slot fold kernel, summed over passes
                                   (part of reduce_ms), when timing = 1                      */
-    int32_t k_pass_used;       /* stored K: 1 = symmetric pass, 2 = full square, 3 = the whole
+    int32_t k_pass_used;       /* stored K: 1 = symmetric pass, 2 = full square (row by row or by
+                                  block rows), 3 = the whole
                                   fit in one cooperative launch (automatic choice for an FP32
                                   K that sits in L2: n <= 6144, k <= 32; it reads the full
                                   square); 0 recompute                                     */
@@ -394,12 +399,11 @@ POPCORN_API popcorn_status popcorn_kmeanspp(const float* P, int64_t n, int32_t d
  * CUDA graph and launched on `stream`; an instance that converges stops
  * doing work on the device while the others go on.  Instances of uneven n,
  * d, k and kernel share every launch: work is flattened over (instance,
- * tile / row segment / row block).  options.k_storage FP16 / BF16 stores every
- * instance's square as 32 KB half tiles (written by the FP32 build, or rounded
- * from a BF16 / BF16X3 build's FP32 square) and each pass reads them on the
- * tensor cores: per 128-row block, MMAs of its tiles against one-hot label
- * operands, the row sums in TMEM.  k_pass and sym_tile do not apply here (each
- * square is read whole).
+ * tile / row block).  K is stored as the packed upper triangle and read by
+ * block rows; options.k_storage FP16 / BF16 stores it as 32 KB half tiles, which
+ * each pass reads on the tensor cores: per 128-row block, MMAs of its tiles
+ * (those below the diagonal transposed) against one-hot label operands, the row
+ * sums in TMEM.  k_pass and sym_tile do not apply here.
  *
  *   instances        host array of `count` descriptors.
  *   objectives_out   host, count doubles: J(labels_out) per instance.
