@@ -180,7 +180,8 @@ typedef struct {
     double tune_ms;            /* host wall time this call spent timing candidates           */
     int32_t schedule[4];       /* the schedule used (tuned or heuristic):
                                   batched: {columns per K-stream unit, warps per block,
-                                            blocks per SM, 0};
+                                            blocks per SM (tuned: 1, or 2 for as
+                                            many as fit), 0};
                                   recompute: {row blocks per tile, column segments,
                                               units per SM target, 0};
                                   symmetric pass: {super-tile edge, block ring depth,

@@ -1428,7 +1428,10 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     int* err = reinterpret_cast<int*>(base + err_off);
     POPCORN_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
 
-    // ---- schedule of the batched K stream: unit length, blocks per SM (4 consumer warps a block)
+    // ---- schedule of the batched K stream: unit length, blocks per SM (4 consumer warps a block).
+    // A tuned schedule says 1, or 2 for as many as fit: two where three fit took 178 ms for a batch
+    // that takes 142 ms so (256 instances of
+    // n = 500 .. 8,000, 30 passes).
     auto set_seglen = [&](int seglen) {
         bp.units = 0;
         for (int t = 0; t < count; ++t) {
@@ -1446,7 +1449,8 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
             sum_n2 += (double)h[t].n * h[t].n;
             max_n = h[t].n > max_n ? h[t].n : max_n;
         }
-        const TuneKey key{1, opt.precision, count, bp.kmax, log2_bucket(sum_n2), log2_bucket(max_n),
+        // (4: the block-row stream; files may hold schedules of the row-by-row stream under 1)
+        const TuneKey key{4, opt.precision, count, bp.kmax, log2_bucket(sum_n2), log2_bucket(max_n),
                           opt.k_storage, dev->sms};
         TuneValue best{};
         if (tune_lookup(key, &best)) {
@@ -1474,7 +1478,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
                     BatchPlan cand = bp;
                     set_seglen(seglen);
                     cand.units = bp.units;
-                    if (!plan_batched_tiles(&cand, dev->sms, ps) || cand.per_sm != ps) continue;   // does not fit: skip
+                    if (!plan_batched_tiles(&cand, dev->sms, ps == 2 ? 0 : ps) || cand.per_sm < ps) continue;   // does not fit
                     POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count,
                                                  cudaMemcpyHostToDevice, s));
                     POPCORN_CUDA(upload_units());
@@ -1489,6 +1493,9 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
                         POPCORN_CUDA(cudaEventElapsedTime(&e, t0, t1));
                         ms = e < ms ? e : ms;
                     }
+                    // the argmin and the z reduction read every segment's slot, at about 1 TB/s (shorter
+                    // units alone stream up to a tenth faster, and lost more than that there)
+                    for (int t = 0; t < count; ++t) ms += (float)(4.0 * h[t].nseg * h[t].k * h[t].n / 1e9);
                     ++tune_cands;
                     if (ms < best.ms) {
                         best.ms = ms;
@@ -1513,10 +1520,11 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     if (!half) {
         set_seglen(sched[0]);
         POPCORN_CUDA(upload_units());
-        if (!plan_batched_tiles(&bp, dev->sms, sched[2]))
+        const bool tuned = sched[2] != 0;
+        if (!plan_batched_tiles(&bp, dev->sms, sched[2] == 1 ? 1 : 0))
             return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
         sched[1] = bp.warps;
-        sched[2] = bp.per_sm;
+        sched[2] = tuned ? std::min(bp.per_sm, 2) : bp.per_sm;
     } else {
         sched[0] = 0;            // whole 128-row blocks a unit
         sched[1] = bp.mstages;   // ring depth of the tensor-core stream

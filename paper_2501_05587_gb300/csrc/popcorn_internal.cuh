@@ -477,7 +477,7 @@ cudaError_t launch_batched_mma_stream(const BatchInst* dI, const int2* units, co
 
 // ---- autotune cache (autotune.cu) ---------------------------------------------
 struct TuneKey {
-    int32_t target;       // 1: batched K stream, 2: recompute pass
+    int32_t target;       // 2: recompute pass, 3: K-build schedule, 4: batched K stream
     int32_t precision;
     int32_t a, b, c, d, e;   // target-specific size buckets
     int32_t sms;
