@@ -17,6 +17,8 @@
 #include "popcorn_internal.cuh"
 #include "stream_common.cuh"
 
+#include <utility>
+
 #include <cooperative_groups.h>
 #include <cuda/std/limits>
 #include <cuda_bf16.h>
@@ -653,13 +655,17 @@ __device__ __forceinline__ double trace_part(const float* __restrict__ kdiag, in
 }
 
 // sum of diag(K): one cluster of 8 blocks, whose sums the first adds in order (one block's FP64,
-// 2 additions a clock, took 36 us on average over n = 2,000 to 200,000)
+// 2 additions a clock, took 36 us on average over n = 2,000 to 200,000).  A block's shared memory
+// may be written from outside only once the block has started: every block arrives at its start,
+// and waits for the others (behind its own sum) before the store.
 constexpr int kTraceBlocks = 8;
 __global__ void __cluster_dims__(kTraceBlocks, 1, 1) __launch_bounds__(512)
     trace_kernel(const float* __restrict__ kdiag, int n, LoopState* st) {
     __shared__ double sums[kTraceBlocks];
     auto cluster = cooperative_groups::this_cluster();
+    auto started = cluster.barrier_arrive();
     const double t = trace_part(kdiag, n, (int)(blockIdx.x * blockDim.x + threadIdx.x), (int)(gridDim.x * blockDim.x));
+    cluster.barrier_wait(std::move(started));
     if (threadIdx.x == 0) *cluster.map_shared_rank(&sums[blockIdx.x], 0) = t;
     cluster.sync();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
