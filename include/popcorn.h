@@ -77,8 +77,12 @@ typedef struct {
 
 /* Arithmetic used to form B = P P^T for the kernel matrix. */
 typedef enum {
-    POPCORN_FP32 = 0,    /* FP32: multiply-adds on CUDA cores, or, where the device finds it as exact, tensor
-                            cores on the points split into two FP16 parts, FP32 accumulate; Gaussian
+    POPCORN_FP32 = 0,    /* FP32: multiply-adds on CUDA cores, or tensor cores on the points split into
+                            two FP16 parts (23 bits), FP32 accumulate, where the device finds the
+                            points' values close enough together for it: the error of p_i . p_j
+                            relative to |p_i| |p_j| is then no larger than the multiply-adds'.  The
+                            parts take 4 n ceil32(d) + 4 n bytes of workspace during the build; where
+                            these cannot be had, CUDA cores.  Gaussian
                             distances by the norm expansion where its error bound allows, else from
                             coordinate differences                                             */
     POPCORN_BF16 = 1,    /* tcgen05 tensor cores, BF16 operands, FP32 accumulate                       */

@@ -208,7 +208,7 @@ popcorn_status check_kernel(const popcorn_kernel& kern, KernParams* kp) {
 }
 
 // K = kappa(P P^T) on stream s.  FP32: CUDA-core tiles, or tcgen05 tiles of the points split
-// into two FP16 parts where that is as exact (decided on the device).  BF16 / BF16X3: tcgen05
+// into two FP16 parts where their values are close enough together (decided on the device).  BF16 / BF16X3: tcgen05
 // tiles.  Operand copies come from `ws`, and *err (device) reports a timed-out wait inside a
 // kernel.
 // packed: the build writes the block-packed upper triangle (symmetric pass only).

@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(128, 2) kbuild_dot_kernel(const float* __restr
                                                             float expand_coef, const SplitState* __restrict__ split,
                                                             long long tiles) {
     __shared__ __align__(16) TileSmem sm;
-    if (split && split->use) return;   // the tensor-core build has written K
+    if (split && split_taken(split)) return;   // the tensor-core build has written K
     if (KIND == kGaussExpand && !expansion_applies(rn, maxr, expand_coef)) return;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x)
         kbuild_tile<KIND, float, false, PACKED, 16>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full, rn);

@@ -36,9 +36,9 @@
 //           the Gaussian's cancellation needs) -- 2 d loaded instead of the 3 d
 //           a [hi|hi|lo] x [hi|lo|hi] GEMM would stream.
 //   FP32    (SPLIT) W = [hi | lo] in FP16 of the points times a power of two s:
-//           hi = fp16(s p), lo = fp16(s p - hi), which represent p to 2^-24 of itself
-//           (hi and lo carry 11 bits each and lo's sign one more; column-wise the
-//           error is below 2^-26 of the column's largest value, see split_decide_kernel).
+//           hi = fp16(s p), lo = fp16(s p - hi), which represent p to 2^-23 of itself
+//           (hi and lo carry 11 bits each and lo's sign one more: 1 + 2^-12 + 2^-23 is 2^-23 off), or
+//           to 2^-27 of its row's and column's largest value (see split_decide_kernel).
 //           The products are exact in FP32, but the tensor core adds them with
 //           truncation: left in TMEM over a long row the sum drifts low by half an ulp an
 //           MMA (measured at d = 784 on uniform points: relative error 6.1e-6 against
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                      const __grid_constant__ CUtensorMap map_kd, const __grid_constant__ CUtensorMap map_kt,
                      TcArgs a) {
     constexpr bool SPLIT = MODE == kModeSplit, X3 = MODE != kModeBf16;
-    if (SPLIT && !a.split->use) return;   // the CUDA-core build takes this matrix
+    if (SPLIT && !split_taken(a.split)) return;   // the CUDA-core build takes this matrix
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -691,36 +691,86 @@ __global__ void __launch_bounds__(256) prep_operands_kernel(const float* __restr
 
 // ---- FP32 operands as two FP16 parts (SPLIT) ----------------------------------------------
 
-// Largest |p| of every column (bit patterns: non-negative floats order like them, and NaN and
-// infinity lie above every finite value), and the number of nonzero entries.  A block takes
-// `rows` rows, a thread columns.
-__global__ void __launch_bounds__(256) split_colmax_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
-                                                           int rows, unsigned* __restrict__ colmax,
-                                                           unsigned long long* __restrict__ nonzero) {
-    const int64_t r0 = (int64_t)blockIdx.x * rows;
-    const int64_t r1 = r0 + rows < n ? r0 + rows : n;
+// Largest |p| of every column and, where rowmax is given, of every row (bit patterns: non-negative
+// floats order like them, and NaN and infinity lie above every finite value), and the number of
+// nonzero entries.  A block takes `rows` rows (a multiple of 64) of 128 columns, a warp eight rows at
+// a time with a lane to four columns (one 16-byte load each where rows are aligned); its eight row
+// maxima leave in one instruction.  (A thread to a column, with a reduction and a shared-memory
+// atomic a row of 32 columns, took 70 us at n = 20,000, d = 784.)
+constexpr int kScanCols = 128, kScanStep = 64;
+__global__ void __launch_bounds__(256) split_scan_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
+                                                         int rows, unsigned* __restrict__ colmax,
+                                                         unsigned* __restrict__ rowmax,
+                                                         unsigned long long* __restrict__ nonzero) {
+    __shared__ unsigned cm[8][kScanCols];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t r0 = (int64_t)blockIdx.x * rows, r1 = r0 + rows < n ? r0 + rows : n;
+    const bool vec = (ldp & 3) == 0 && ((uintptr_t)P & 15) == 0;
     unsigned nz = 0u;
-    for (int l = blockIdx.y * blockDim.x + threadIdx.x; l < d; l += gridDim.y * blockDim.x) {
-        unsigned m = 0u;
-#pragma unroll 8
-        for (int64_t r = r0; r < r1; ++r) {
-            const unsigned v = __float_as_uint(P[r * ldp + l]) & 0x7fffffffu;
-            m = max(m, v);
-            nz += v != 0u;
+    for (int c0 = blockIdx.y * kScanCols; c0 < d; c0 += gridDim.y * kScanCols) {
+        const int l = c0 + 4 * lane;
+        unsigned m[4] = {0u, 0u, 0u, 0u};
+        for (int64_t r = r0 + 8 * warp; r < r1; r += kScanStep) {
+            float v[8][4];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+                const float* p = P + (r + x < r1 ? r + x : r1 - 1) * ldp + l;   // (past the end: the last row again)
+                if (vec && l + 3 < d) {
+                    const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+                    v[x][0] = f.x, v[x][1] = f.y, v[x][2] = f.z, v[x][3] = f.w;
+                } else {
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) v[x][y] = l + y < d ? __ldg(p + y) : 0.f;
+                }
+            }
+            unsigned mine = 0u;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+                unsigned w = 0u;
+#pragma unroll
+                for (int y = 0; y < 4; ++y) {
+                    const unsigned b = __float_as_uint(v[x][y]) & 0x7fffffffu;
+                    m[y] = max(m[y], b);
+                    w = max(w, b);
+                    nz += b != 0u && r + x < r1;
+                }
+                if (rowmax) {
+                    w = __reduce_max_sync(0xffffffffu, w);
+                    if (lane == x) mine = w;
+                }
+            }
+            if (rowmax && lane < 8 && r + lane < r1 && mine) atomicMax(rowmax + r + lane, mine);
         }
-        if (m) atomicMax(colmax + l, m);
+#pragma unroll
+        for (int y = 0; y < 4; ++y) cm[warp][4 * lane + y] = m[y];
+        __syncthreads();
+        if (threadIdx.x < kScanCols && c0 + (int)threadIdx.x < d) {
+            unsigned t = 0u;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) t = max(t, cm[w][threadIdx.x]);
+            if (t) atomicMax(colmax + c0 + threadIdx.x, t);
+        }
+        __syncthreads();
     }
     nz = __reduce_add_sync(0xffffffffu, nz);
-    if ((threadIdx.x & 31) == 0 && nz) atomicAdd(nonzero, (unsigned long long)nz);
+    if (lane == 0 && nz) atomicAdd(nonzero, (unsigned long long)nz);
 }
 
 // The scale, and whether the split build takes the matrix.  s is the power of two that puts
 // the largest |p| into [2^14, 2^15).  hi = fp16(s p) keeps 11 bits, lo = fp16(s p - hi) the
-// next 11 and a sign while |s p| >= 2^-2; below that lo is subnormal and the error at most
-// 2^-25.  Every column's largest value must be at least 2^2 (after the scale): an element's
-// error is then at most 2^-24 of itself or 2^-27 of its column's largest value.  Columns
+// next 11 and a sign while |s p| >= 2^-2: p to 2^-23 of itself.  Below that lo is subnormal and the
+// error at most 2^-25.  Every column's largest value must be at least 2^2 (after the scale), and for
+// dot products every nonzero row's too: an element's error is then at most 2^-23 of itself or 2^-27
+// of its column's and its row's largest value.  (Of the row's: K_ij of two short rows is small too,
+// and has to be as exact as FP32 makes it.  Normal points, n = 300, d = 512, one row 1e4, 1e6, 1e7,
+// 1e9 times as long: the representation alone puts K_ij of the others off by at most 0.4, 11, 165
+// and 10,650 times 2^-24 |p_i| |p_j|, FP32 FMAs by 18.  The Gaussian's distances are compared with
+// the largest norm by its own rule, and take no line for rows.)  Columns or rows
 // further apart than that (a factor of 4096), values outside 2^+-40 (whose products could
-// leave FP32) and non-finite points stay on CUDA cores.  So do dot products of few nonzero
+// leave FP32) and non-finite points stay on CUDA cores, and so do dot products of points more than
+// 1 / kSplitLowPart of whose nonzero entries are below 2^-2 (counted where the operands are written;
+// of normal points it is 1 in 100,000): blocks of columns, each large in other rows, pass
+// the maxima, and the products between blocks are of small entries only.  So do dot products of few nonzero
 // terms, where FP32 FMAs round less than the truncated chunks: with a fraction f of nonzero
 // entries a pair adds about d f^2 of them, and the two errors cross near 20 (measured, linear
 // kernel, 80% zeros: d = 256 5.6e-8 in FMAs against 6.8e-8, d = 512 7.4e-8 in both).  The line
@@ -729,22 +779,31 @@ __global__ void __launch_bounds__(256) split_colmax_kernel(const float* __restri
 // -1.0e-7 against -1.3e-7, d = 256 -4e-8 against 1.4e-7).  The Gaussian has no such line: its error is that of the last rounding (3.6e-8
 // either way), and the split takes it where the norm expansion applies (kbuild_simt.cu).
 constexpr float kSplitMinTerms = 128.f;
+constexpr unsigned long long kSplitLowPart = 64;
 constexpr int kSplitMinD = 48;   // the Gaussian's line
-__global__ void __launch_bounds__(256) split_decide_kernel(const unsigned* __restrict__ colmax,
-                                                           const unsigned long long* __restrict__ nonzero, int n, int d,
-                                                           int gaussian, const unsigned* maxr, float expand_coef,
-                                                           SplitState* __restrict__ st) {
+constexpr int kDecideThreads = 1024;
+__global__ void __launch_bounds__(kDecideThreads)
+    split_decide_kernel(const unsigned* __restrict__ colmax, const unsigned* __restrict__ rowmax,
+                        const unsigned long long* __restrict__ nonzero, int n, int d, int gaussian, const unsigned* maxr,
+                        float expand_coef, SplitState* __restrict__ st) {
     __shared__ unsigned mx_s, mn_s;
     if (threadIdx.x == 0) {
         mx_s = 0u;
         mn_s = 0xffffffffu;
     }
     __syncthreads();
-    unsigned mx = 0u, mn = 0xffffffffu;
+    unsigned mx = 0u, mn = 0xffffffffu;   // the largest entry; the smallest nonzero maximum of a column or row
     for (int l = threadIdx.x; l < d; l += blockDim.x) {
         const unsigned v = colmax[l];
         mx = max(mx, v);
         if (v) mn = min(mn, v);
+    }
+    if (rowmax) {
+#pragma unroll 8
+        for (int r = threadIdx.x; r < n; r += blockDim.x) {
+            const unsigned v = rowmax[r];
+            mn = min(mn, v ? v : 0xffffffffu);
+        }
     }
     atomicMax(&mx_s, mx);
     atomicMin(&mn_s, mn);
@@ -763,15 +822,17 @@ __global__ void __launch_bounds__(256) split_decide_kernel(const unsigned* __res
     st->use = use ? 1 : 0;
     st->scale = use ? ldexpf(1.f, e) : 0.f;
     st->unscale = use ? ldexpf(1.f, -2 * e) : 0.f;
+    st->low = 0ull;
+    st->low_max = gaussian ? ~0ull : *nonzero / kSplitLowPart;
 }
 
 // FP32 rows -> W = [hi | lo] in FP16, zero padding.  A thread takes four columns of a row
 // (float4 loads when rows are 16-byte aligned), 8-byte stores.
 __global__ void __launch_bounds__(256) split_operands_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
-                                                             int dpad, const SplitState* __restrict__ st,
-                                                             __half* __restrict__ W) {
+                                                             int dpad, SplitState* st, __half* __restrict__ W) {
     if (!st->use) return;
     const float s = st->scale;
+    unsigned low = 0u;
     const bool vec = (ldp & 3) == 0 && ((uintptr_t)P & 15) == 0;
     const int q4 = dpad / 4;
     const int64_t total = (int64_t)n * q4, step = (int64_t)gridDim.x * blockDim.x;
@@ -791,6 +852,7 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const float* __rest
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
             const float f0 = v[2 * x] * s, f1 = v[2 * x + 1] * s;
+            low += (f0 != 0.f && fabsf(f0) < 0.25f) + (f1 != 0.f && fabsf(f1) < 0.25f);
             hi[x] = __floats2half2_rn(f0, f1);
             const float2 h = __half22float2(hi[x]);
             lo[x] = __floats2half2_rn(f0 - h.x, f1 - h.y);
@@ -799,6 +861,8 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const float* __rest
         *reinterpret_cast<uint2*>(w) = *reinterpret_cast<const uint2*>(hi);
         *reinterpret_cast<uint2*>(w + dpad) = *reinterpret_cast<const uint2*>(lo);
     }
+    low = __reduce_add_sync(0xffffffffu, low);
+    if ((threadIdx.x & 31) == 0 && low) atomicAdd(&st->low, (unsigned long long)low);
 }
 
 }  // namespace
@@ -964,7 +1028,8 @@ bool kbuild_split_applies(int n, int d, bool dot) {
 
 size_t kbuild_split_workspace(int n, int d) {
     const size_t dpad = ((size_t)d + 31) / 32 * 32;
-    return (((size_t)n * 2 * dpad * 2 + 255) & ~(size_t)255) + (((size_t)d * 4 + 255) & ~(size_t)255) + 512;
+    return (((size_t)n * 2 * dpad * 2 + 255) & ~(size_t)255) + (((size_t)d * 4 + 255) & ~(size_t)255) + (size_t)n * 4 +
+           512;
 }
 
 cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernParams kp, float* K, int64_t ldk,
@@ -978,17 +1043,19 @@ cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernP
     __half* W = reinterpret_cast<__half*>(w);
     unsigned long long* nonzero = reinterpret_cast<unsigned long long*>(w + ops);
     unsigned* colmax = reinterpret_cast<unsigned*>(w + ops + 256);
-    SplitState* st = reinterpret_cast<SplitState*>(w + ops + 256 + cols);
-    cudaError_t e = cudaMemsetAsync(w + ops, 0, 256 + cols, s);
+    SplitState* st = reinterpret_cast<SplitState*>(w + ops + 128);
+    const bool dot = kp.kind != POPCORN_GAUSSIAN;
+    unsigned* rowmax = dot ? reinterpret_cast<unsigned*>(w + ops + 256 + cols) : nullptr;
+    cudaError_t e = cudaMemsetAsync(w + ops, 0, 256 + cols + (dot ? (size_t)n * 4 : 0), s);
     if (e != cudaSuccess) return e;
-    // about eight blocks an SM over (row chunk, 256 columns), at least 32 rows a block
-    const int cy = (d + 255) / 256;
-    int rows = (int)(((int64_t)n * cy + 8 * num_sms - 1) / (8 * num_sms));
-    if (rows < 32) rows = 32;
-    split_colmax_kernel<<<dim3((unsigned)((n + rows - 1) / rows), (unsigned)(cy < 65535 ? cy : 65535)), 256, 0, s>>>(
-        P, n, d, ldp, rows, colmax, nonzero);
+    // about eight blocks an SM over (rows, columns)
+    const int cy = (d + kScanCols - 1) / kScanCols;
+    int64_t rows = ((int64_t)n * cy + 8 * num_sms - 1) / (8 * num_sms);
+    rows = ((rows < n ? rows : n) + kScanStep - 1) / kScanStep * kScanStep;
+    split_scan_kernel<<<dim3((unsigned)((n + rows - 1) / rows), (unsigned)(cy < 65535 ? cy : 65535)), 256, 0, s>>>(
+        P, n, d, ldp, (int)rows, colmax, rowmax, nonzero);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    split_decide_kernel<<<1, 256, 0, s>>>(colmax, nonzero, n, d, kp.kind == POPCORN_GAUSSIAN ? 1 : 0, maxr, expand_coef, st);
+    split_decide_kernel<<<1, kDecideThreads, 0, s>>>(colmax, rowmax, nonzero, n, d, dot ? 0 : 1, maxr, expand_coef, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t work = (int64_t)n * (dpad / 4);
     const int64_t blocks = (work + 255) / 256;

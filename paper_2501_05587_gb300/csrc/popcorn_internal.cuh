@@ -226,7 +226,9 @@ struct SplitState {
     int use;
     float scale;     // s: operands are s p
     float unscale;   // s^-2
+    unsigned long long low, low_max;   // nonzero entries whose low part is subnormal; the most there may be
 };
+__device__ __forceinline__ bool split_taken(const SplitState* st) { return st->use && st->low <= st->low_max; }
 bool kbuild_split_applies(int n, int d, bool dot);   // dot: linear or polynomial kernel
 size_t kbuild_split_workspace(int n, int d);
 // FP32 K as launch_kbuild_simt writes it (packed 0, kPackedSw16 or kPackedSw4; full).  rn / maxr /
