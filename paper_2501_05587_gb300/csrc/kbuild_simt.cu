@@ -409,16 +409,15 @@ __global__ void __launch_bounds__(256) kbuild_simt_kernel(const float* __restric
                                                           KernParams kp, TK* __restrict__ K, int64_t ldk,
                                                           float* __restrict__ kdiag, int T, int full,
                                                           const float* __restrict__ rn, const unsigned* maxr,
-                                                          float expand_coef, int dot_expands, long long tiles) {
+                                                          float expand_coef, int dot_expands) {
     __shared__ __align__(16) TileSmem sm;
     const bool expand = KIND == POPCORN_GAUSSIAN && expansion_applies(rn, maxr, expand_coef);
     if (expand && dot_expands) return;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-        if (expand)
-            kbuild_tile<kGaussExpand, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full, rn);
-        else
-            kbuild_tile<KIND, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full);
-    }
+    if (expand)
+        kbuild_tile<kGaussExpand, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, (long long)blockIdx.x, sm,
+                                                     full, rn);
+    else
+        kbuild_tile<KIND, TK, false, PACKED>(P, n, d, ldp, kp, K, ldk, kdiag, T, (long long)blockIdx.x, sm, full);
 }
 
 // The dot-product kinds (linear, polynomial, the Gaussian by the norm expansion) on FP32 K:
@@ -431,11 +430,12 @@ __global__ void __launch_bounds__(128, 2) kbuild_dot_kernel(const float* __restr
                                                             float* __restrict__ kdiag, int T, int full,
                                                             const float* __restrict__ rn, const unsigned* maxr,
                                                             float expand_coef, const SplitState* __restrict__ split,
-                                                            long long tiles) {
+                                                            long long tiles, int each) {
     __shared__ __align__(16) TileSmem sm;
     if (split && split_taken(split)) return;   // the tensor-core build has written K
     if (KIND == kGaussExpand && !expansion_applies(rn, maxr, expand_coef)) return;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x)
+    const long long t0 = (long long)blockIdx.x * each;
+    for (long long t = t0; t < min(tiles, t0 + each); ++t)
         kbuild_tile<KIND, float, false, PACKED, 16>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full, rn);
 }
 
@@ -477,10 +477,6 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
     const long long tiles = full ? (long long)T * T : (long long)T * (T + 1) / 2;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     dim3 grid((unsigned)tiles), block(256);
-    // d > KC: blocks walk the tiles in strides of a grid of at most 8 blocks an SM, so that a
-    // launch whose work another kernel took costs one short wave (images: 150,000 empty blocks
-    // took 0.23 ms) and tiles of equal cost still spread evenly
-    const dim3 wgrid((unsigned)(num_sms > 0 && tiles > 8ll * num_sms ? 8ll * num_sms : tiles));
     if (d <= KC) {
         switch (kp.kind) {
             case POPCORN_LINEAR:
@@ -508,40 +504,48 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
                                                       err, num_sms, s, launches, PACKED, full, &split);
             if (e != cudaSuccess) return e;
         }
+        // A dot-product launch that another kernel may have taken the work of has at most 512 blocks an
+        // SM, several consecutive tiles each from there (images: 150,000 empty blocks took 0.23 ms).
+        // Points the split refuses pay for it where a block's tiles are more than a few in 100 of what an
+        // SM's slots take in turn: linear, n = 30,000, d = 128, 2.68 ms without the split build, 2.70 so,
+        // 2.75 with at most 128 blocks an SM and 2.78 with 8; n = 20,000, d = 784 5.45, 5.45 and (8) 5.62.
+        const long long most = 512ll * num_sms;
+        const long long each = (split || rn) && num_sms > 0 && tiles > most ? (tiles + most - 1) / most : 1;
+        const dim3 wgrid((unsigned)((tiles + each - 1) / each));
         switch (kp.kind) {
             case POPCORN_LINEAR:
                 kbuild_dot_kernel<POPCORN_LINEAR, PACKED><<<wgrid, dblock, 0, s>>>(
-                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles);
+                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles, (int)each);
                 return cudaGetLastError();
             case POPCORN_POLYNOMIAL:
                 kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED><<<wgrid, dblock, 0, s>>>(
-                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles);
+                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles, (int)each);
                 return cudaGetLastError();
             default:
                 if (rn) {
                     kbuild_dot_kernel<kGaussExpand, PACKED><<<wgrid, dblock, 0, s>>>(
-                        P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles);
+                        P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles, (int)each);
                     cudaError_t e = cudaGetLastError();
                     if (e != cudaSuccess) return e;
                     if (launches) ++*launches;
                 }
-                kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED><<<wgrid, block, 0, s>>>(
-                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 1, tiles);
+                kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED><<<grid, block, 0, s>>>(
+                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 1);
                 return cudaGetLastError();
         }
     }
     switch (kp.kind) {
         case POPCORN_LINEAR:
             kbuild_simt_kernel<POPCORN_LINEAR, TK, PACKED>
-                <<<wgrid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0, tiles);
+                <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0);
             break;
         case POPCORN_POLYNOMIAL:
             kbuild_simt_kernel<POPCORN_POLYNOMIAL, TK, PACKED>
-                <<<wgrid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0, tiles);
+                <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0);
             break;
         default:
             kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED>
-                <<<wgrid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0, tiles);
+                <<<grid, block, 0, s>>>(P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 0);
             break;
     }
     return cudaGetLastError();

@@ -691,18 +691,93 @@ __global__ void __launch_bounds__(256) prep_operands_kernel(const float* __restr
 
 // ---- FP32 operands as two FP16 parts (SPLIT) ----------------------------------------------
 
+// The scale, and whether the split build takes the matrix.  s is the power of two that puts
+// the largest |p| into [2^14, 2^15).  hi = fp16(s p) keeps 11 bits, lo = fp16(s p - hi) the
+// next 11 and a sign while |s p| >= 2^-2: p to 2^-23 of itself.  Below that lo is subnormal and the
+// error at most 2^-25.  Every column's largest value must be at least 2^2 (after the scale), and for
+// dot products every nonzero row's too: an element's error is then at most 2^-23 of itself or 2^-27
+// of its column's and its row's largest value.  (Of the row's: K_ij of two short rows is small too,
+// and has to be as exact as FP32 makes it.  Normal points, n = 300, d = 512, one row 1e4, 1e6, 1e7,
+// 1e9 times as long: the representation alone puts K_ij of the others off by at most 0.4, 11, 165
+// and 10,650 times 2^-24 |p_i| |p_j|, FP32 FMAs by 18.  The Gaussian's distances are compared with
+// the largest norm by its own rule, and take no line for rows.)  Columns or rows
+// further apart than that (a factor of 4096), values outside 2^+-40 (whose products could
+// leave FP32) and non-finite points stay on CUDA cores, and so do dot products of points more than
+// 1 / kSplitLowPart of whose nonzero entries are below 2^-2 (counted where the operands are written;
+// of normal points it is 1 in 100,000): blocks of columns, each large in other rows, pass
+// the maxima, and the products between blocks are of small entries only.  So do dot products of few nonzero
+// terms, where FP32 FMAs round less than the truncated chunks: with a fraction f of nonzero
+// entries a pair adds about d f^2 of them, and the two errors cross near 20 (measured, linear
+// kernel, 80% zeros: d = 256 5.6e-8 in FMAs against 6.8e-8, d = 512 7.4e-8 in both).  The line
+// is at 128 terms, four chunks a row: from there the objective of a fit, J = trace K - ..., is
+// no further off either (2,000-point clusters, polynomial: d = 100 -3e-7 against -9e-8, d = 128
+// -1.0e-7 against -1.3e-7, d = 256 -4e-8 against 1.4e-7).  The Gaussian has no such line: its error is that of the last rounding (3.6e-8
+// either way), and the split takes it where the norm expansion applies (kbuild_simt.cu).
+constexpr float kSplitMinTerms = 128.f;
+constexpr unsigned long long kSplitLowPart = 64;
+constexpr int kSplitMinD = 48;   // the Gaussian's line
+// (All 256 threads of one block.)
+__device__ void split_decide(const unsigned* colmax, const unsigned* rowmax, const unsigned long long* nonzero, int n,
+                             int d, const unsigned* maxr, float expand_coef, SplitState* st) {
+    __shared__ unsigned mx_s, mn_s;
+    if (threadIdx.x == 0) {
+        mx_s = 0u;
+        mn_s = 0xffffffffu;
+    }
+    __syncthreads();
+    unsigned mx = 0u, mn = 0xffffffffu;   // the largest entry; the smallest nonzero maximum of a column or row
+    auto least = [&](unsigned v) { mn = min(mn, v ? v : 0xffffffffu); };
+    for (int l = threadIdx.x; l < d; l += blockDim.x) {
+        const unsigned v = __ldcg(colmax + l);
+        mx = max(mx, v);
+        least(v);
+    }
+    if (rowmax) {
+        const uint4* r4 = reinterpret_cast<const uint4*>(rowmax);   // (zeros up to a multiple of four)
+#pragma unroll 8
+        for (int q = threadIdx.x; q < (n + 3) / 4; q += blockDim.x) {
+            const uint4 v = __ldcg(r4 + q);
+            least(v.x), least(v.y), least(v.z), least(v.w);
+        }
+    }
+    atomicMax(&mx_s, mx);
+    atomicMin(&mn_s, mn);
+    __syncthreads();
+    if (threadIdx.x) return;
+    mx = mx_s;
+    mn = mn_s;
+    const bool gaussian = !rowmax;
+    const unsigned long long nz = __ldcg(nonzero);
+    const float fill = (float)nz / ((float)n * (float)d);
+    bool use = gaussian ? __uint_as_float(*maxr) * expand_coef <= 1e-6f : (float)d * fill * fill >= kSplitMinTerms;
+    int e = 0;   // s = 2^e
+    if (mx) {
+        e = 14 + 127 - (int)(mx >> 23);
+        use = use && mx >= __float_as_uint(0x1p-40f) && mx < __float_as_uint(0x1p40f) &&
+              ldexpf(__uint_as_float(mn), e) >= 4.f;
+    }
+    st->use = use ? 1 : 0;
+    st->scale = use ? ldexpf(1.f, e) : 0.f;
+    st->unscale = use ? ldexpf(1.f, -2 * e) : 0.f;
+    st->low = 0ull;
+    st->low_max = gaussian ? ~0ull : nz / kSplitLowPart;
+}
+
 // Largest |p| of every column and, where rowmax is given, of every row (bit patterns: non-negative
 // floats order like them, and NaN and infinity lie above every finite value), and the number of
 // nonzero entries.  A block takes `rows` rows (a multiple of 64) of 128 columns, a warp eight rows at
 // a time with a lane to four columns (one 16-byte load each where rows are aligned); its eight row
 // maxima leave in one instruction.  (A thread to a column, with a reduction and a shared-memory
-// atomic a row of 32 columns, took 70 us at n = 20,000, d = 784.)
+// atomic a row of 32 columns, took 70 us at n = 20,000, d = 784.)  The last block to finish takes the
+// decision.
 constexpr int kScanCols = 128, kScanStep = 64;
 __global__ void __launch_bounds__(256) split_scan_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
                                                          int rows, unsigned* __restrict__ colmax,
                                                          unsigned* __restrict__ rowmax,
-                                                         unsigned long long* __restrict__ nonzero) {
+                                                         unsigned long long* __restrict__ nonzero, unsigned* ticket,
+                                                         const unsigned* maxr, float expand_coef, SplitState* st) {
     __shared__ unsigned cm[8][kScanCols];
+    __shared__ int am_last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t r0 = (int64_t)blockIdx.x * rows, r1 = r0 + rows < n ? r0 + rows : n;
     const bool vec = (ldp & 3) == 0 && ((uintptr_t)P & 15) == 0;
@@ -754,76 +829,13 @@ __global__ void __launch_bounds__(256) split_scan_kernel(const float* __restrict
     }
     nz = __reduce_add_sync(0xffffffffu, nz);
     if (lane == 0 && nz) atomicAdd(nonzero, (unsigned long long)nz);
-}
-
-// The scale, and whether the split build takes the matrix.  s is the power of two that puts
-// the largest |p| into [2^14, 2^15).  hi = fp16(s p) keeps 11 bits, lo = fp16(s p - hi) the
-// next 11 and a sign while |s p| >= 2^-2: p to 2^-23 of itself.  Below that lo is subnormal and the
-// error at most 2^-25.  Every column's largest value must be at least 2^2 (after the scale), and for
-// dot products every nonzero row's too: an element's error is then at most 2^-23 of itself or 2^-27
-// of its column's and its row's largest value.  (Of the row's: K_ij of two short rows is small too,
-// and has to be as exact as FP32 makes it.  Normal points, n = 300, d = 512, one row 1e4, 1e6, 1e7,
-// 1e9 times as long: the representation alone puts K_ij of the others off by at most 0.4, 11, 165
-// and 10,650 times 2^-24 |p_i| |p_j|, FP32 FMAs by 18.  The Gaussian's distances are compared with
-// the largest norm by its own rule, and take no line for rows.)  Columns or rows
-// further apart than that (a factor of 4096), values outside 2^+-40 (whose products could
-// leave FP32) and non-finite points stay on CUDA cores, and so do dot products of points more than
-// 1 / kSplitLowPart of whose nonzero entries are below 2^-2 (counted where the operands are written;
-// of normal points it is 1 in 100,000): blocks of columns, each large in other rows, pass
-// the maxima, and the products between blocks are of small entries only.  So do dot products of few nonzero
-// terms, where FP32 FMAs round less than the truncated chunks: with a fraction f of nonzero
-// entries a pair adds about d f^2 of them, and the two errors cross near 20 (measured, linear
-// kernel, 80% zeros: d = 256 5.6e-8 in FMAs against 6.8e-8, d = 512 7.4e-8 in both).  The line
-// is at 128 terms, four chunks a row: from there the objective of a fit, J = trace K - ..., is
-// no further off either (2,000-point clusters, polynomial: d = 100 -3e-7 against -9e-8, d = 128
-// -1.0e-7 against -1.3e-7, d = 256 -4e-8 against 1.4e-7).  The Gaussian has no such line: its error is that of the last rounding (3.6e-8
-// either way), and the split takes it where the norm expansion applies (kbuild_simt.cu).
-constexpr float kSplitMinTerms = 128.f;
-constexpr unsigned long long kSplitLowPart = 64;
-constexpr int kSplitMinD = 48;   // the Gaussian's line
-constexpr int kDecideThreads = 1024;
-__global__ void __launch_bounds__(kDecideThreads)
-    split_decide_kernel(const unsigned* __restrict__ colmax, const unsigned* __restrict__ rowmax,
-                        const unsigned long long* __restrict__ nonzero, int n, int d, int gaussian, const unsigned* maxr,
-                        float expand_coef, SplitState* __restrict__ st) {
-    __shared__ unsigned mx_s, mn_s;
-    if (threadIdx.x == 0) {
-        mx_s = 0u;
-        mn_s = 0xffffffffu;
-    }
+    __threadfence();
     __syncthreads();
-    unsigned mx = 0u, mn = 0xffffffffu;   // the largest entry; the smallest nonzero maximum of a column or row
-    for (int l = threadIdx.x; l < d; l += blockDim.x) {
-        const unsigned v = colmax[l];
-        mx = max(mx, v);
-        if (v) mn = min(mn, v);
-    }
-    if (rowmax) {
-#pragma unroll 8
-        for (int r = threadIdx.x; r < n; r += blockDim.x) {
-            const unsigned v = rowmax[r];
-            mn = min(mn, v ? v : 0xffffffffu);
-        }
-    }
-    atomicMax(&mx_s, mx);
-    atomicMin(&mn_s, mn);
+    if (threadIdx.x == 0) am_last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1;
     __syncthreads();
-    if (threadIdx.x) return;
-    mx = mx_s;
-    mn = mn_s;
-    const float fill = (float)*nonzero / ((float)n * (float)d);
-    bool use = gaussian ? __uint_as_float(*maxr) * expand_coef <= 1e-6f : (float)d * fill * fill >= kSplitMinTerms;
-    int e = 0;   // s = 2^e
-    if (mx) {
-        e = 14 + 127 - (int)(mx >> 23);
-        use = use && mx >= __float_as_uint(0x1p-40f) && mx < __float_as_uint(0x1p40f) &&
-              ldexpf(__uint_as_float(mn), e) >= 4.f;
-    }
-    st->use = use ? 1 : 0;
-    st->scale = use ? ldexpf(1.f, e) : 0.f;
-    st->unscale = use ? ldexpf(1.f, -2 * e) : 0.f;
-    st->low = 0ull;
-    st->low_max = gaussian ? ~0ull : *nonzero / kSplitLowPart;
+    if (!am_last) return;
+    __threadfence();
+    split_decide(colmax, rowmax, nonzero, n, d, maxr, expand_coef, st);
 }
 
 // FP32 rows -> W = [hi | lo] in FP16, zero padding.  A thread takes four columns of a row
@@ -1028,8 +1040,8 @@ bool kbuild_split_applies(int n, int d, bool dot) {
 
 size_t kbuild_split_workspace(int n, int d) {
     const size_t dpad = ((size_t)d + 31) / 32 * 32;
-    return (((size_t)n * 2 * dpad * 2 + 255) & ~(size_t)255) + (((size_t)d * 4 + 255) & ~(size_t)255) + (size_t)n * 4 +
-           512;
+    return (((size_t)n * 2 * dpad * 2 + 255) & ~(size_t)255) + (((size_t)d * 4 + 255) & ~(size_t)255) +
+           ((size_t)n + 3) / 4 * 16 + 512;
 }
 
 cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernParams kp, float* K, int64_t ldk,
@@ -1042,20 +1054,19 @@ cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernP
     const size_t cols = ((size_t)d * 4 + 255) & ~(size_t)255;
     __half* W = reinterpret_cast<__half*>(w);
     unsigned long long* nonzero = reinterpret_cast<unsigned long long*>(w + ops);
+    unsigned* ticket = reinterpret_cast<unsigned*>(w + ops + 64);
     unsigned* colmax = reinterpret_cast<unsigned*>(w + ops + 256);
     SplitState* st = reinterpret_cast<SplitState*>(w + ops + 128);
     const bool dot = kp.kind != POPCORN_GAUSSIAN;
     unsigned* rowmax = dot ? reinterpret_cast<unsigned*>(w + ops + 256 + cols) : nullptr;
-    cudaError_t e = cudaMemsetAsync(w + ops, 0, 256 + cols + (dot ? (size_t)n * 4 : 0), s);
+    cudaError_t e = cudaMemsetAsync(w + ops, 0, 256 + cols + (dot ? ((size_t)n + 3) / 4 * 16 : 0), s);
     if (e != cudaSuccess) return e;
     // about eight blocks an SM over (rows, columns)
     const int cy = (d + kScanCols - 1) / kScanCols;
     int64_t rows = ((int64_t)n * cy + 8 * num_sms - 1) / (8 * num_sms);
     rows = ((rows < n ? rows : n) + kScanStep - 1) / kScanStep * kScanStep;
     split_scan_kernel<<<dim3((unsigned)((n + rows - 1) / rows), (unsigned)(cy < 65535 ? cy : 65535)), 256, 0, s>>>(
-        P, n, d, ldp, (int)rows, colmax, rowmax, nonzero);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    split_decide_kernel<<<1, kDecideThreads, 0, s>>>(colmax, rowmax, nonzero, n, d, dot ? 0 : 1, maxr, expand_coef, st);
+        P, n, d, ldp, (int)rows, colmax, rowmax, nonzero, ticket, maxr, expand_coef, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t work = (int64_t)n * (dpad / 4);
     const int64_t blocks = (work + 255) / 256;
@@ -1064,7 +1075,7 @@ cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernP
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = launch_tiles(kModeSplit, W, n, 2 * (int64_t)dpad, dpad, st, kp, rn, K, ldk, kdiag, err, num_sms, s,
                      packed_out(packed), full && !packed ? 1 : 0);
-    if (launches) *launches += 4;
+    if (launches) *launches += 3;
     *state = st;
     return e;
 }
