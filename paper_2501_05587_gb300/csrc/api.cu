@@ -866,7 +866,10 @@ popcorn_status popcorn_fit(const float* P, int64_t n, int32_t d, int64_t ldp, in
     b.sym_meta = nullptr;
     b.sym_order = nullptr;
     if (use_sym && sym.meta_bytes) POPCORN_TRY(ws.alloc(&b.sym_meta, sym.meta_bytes, "block label metadata"));
-    if (use_tiles) POPCORN_TRY(ws.alloc(&b.sym_meta, tiles_record_bytes(ni), "label records"));
+    if (use_tiles) {
+        POPCORN_TRY(ws.alloc(&b.sym_meta, tiles_record_bytes(ni), "label records"));
+        POPCORN_TRY(ws.alloc(&b.Srun, (size_t)nslots * ni * k, "running segment sums"));
+    }
     std::vector<int> sym_order;
     if (use_sym && sym.units > 1 && !capturing) {   // (the natural order inside a caller's capture)
         sym_unit_order(sym, &sym_order);
@@ -1287,7 +1290,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         return o;
     };
     struct Offs {
-        size_t K, kdiag, lab32, lab8, counts, Spart, zpart, zsum, cnorm, invm, st, J, ch;
+        size_t K, kdiag, lab32, lab8, counts, Spart, Srun, zpart, zsum, cnorm, invm, st, J, ch;
     };
     std::vector<Offs> o(count);
     // FP16 / BF16 K: every instance's square as half tiles read by the tensor-core stream
@@ -1363,6 +1366,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         o[t].lab8 = take(((size_t)n + 15) & ~(size_t)15);
         o[t].counts = take(2 * (size_t)k * 4);
         o[t].Spart = take((size_t)n * b.nseg * k * 4);
+        o[t].Srun = half ? 0 : take((size_t)n * b.nseg * k * 8);
         o[t].zpart = take((size_t)zb * k * 8);
         o[t].zsum = take((size_t)k * 8);
         o[t].cnorm = take((size_t)k * 8);
@@ -1408,6 +1412,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.lab8 = base + o[t].lab8;
         b.counts = reinterpret_cast<int32_t*>(base + o[t].counts);
         b.Spart = reinterpret_cast<float*>(base + o[t].Spart);
+        b.Srun = half ? nullptr : reinterpret_cast<float2*>(base + o[t].Srun);
         b.zpart = reinterpret_cast<double*>(base + o[t].zpart);
         b.zsum = reinterpret_cast<double*>(base + o[t].zsum);
         b.cnorm = reinterpret_cast<double*>(base + o[t].cnorm);

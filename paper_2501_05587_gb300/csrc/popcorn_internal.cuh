@@ -353,6 +353,7 @@ struct PassBuffers {
     uint8_t* lab8;        // n rounded up to 16, zero padded
     int32_t* counts;      // [2][k] ping-pong, indexed by pass parity
     float* Spart;         // [nseg][k][n] per-segment cluster sums (row index fastest)
+    float2* Srun;         // block-row pass: sums that are still growing, as pairs of floats, laid out alike
     double* zpart;        // [grid][k]
     double* zsum;         // [k]
     double* cnorm;        // [k]
@@ -414,6 +415,7 @@ struct BatchInst {
     int32_t* lab32;
     int32_t* counts;
     float* Spart;
+    float2* Srun;             // FP32 K: sums that are still growing, as pairs of floats, laid out alike
     double* zpart;
     double* zsum;
     double* cnorm;

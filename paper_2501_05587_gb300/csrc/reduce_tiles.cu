@@ -30,8 +30,18 @@
 // (1.38).  Batch of 256 instances, n 500 to 8,000, k up to 64: 4.7 -> 3.9 ms a pass.  A first form
 // with 32 x 32 pieces of row-major rows (128 bytes at a 120 KB stride) stayed at 3.2 TB/s.
 //
-// A sum runs over 64 k columns (as long as the symmetric pass's register sums) before it is added
-// to the segment's in Spart; the segments are added in float-float.
+// Every so many column blocks a cluster's sums join the segment's, a pair of floats (Srun) until the
+// unit's end; the segments are added in float-float too.  How often goes by the cluster's size m:
+// after 4 sqrt(m) of its columns (at least 32), rounded to a power of two of blocks (tile_plan).  A
+// chain of L additions of one size is off by about 0.4 u sqrt(L / 3) of its own sum (u = 2^-24), m / L
+// such chains by 0.4 u L / sqrt(3 m), and L = 4 sqrt(2 m) makes that the 1.3 u of the row-major stream
+// (32 lanes' partial sums, added one after the other): so S is no further off than there for clusters
+// of any size, with few joins (their traffic stays in L2, but 1 in 8 KB read was enough to be seen).
+// A cluster that holds four times its share of a block's columns (points in the order of their
+// classes) joins at the block's end, and equal labels among four columns are added up first.  As runs of 64 k columns for
+// all clusters, joined in FP32, a row's sum over one cluster of 30,011 was 1.5e-6 off at k = 100 and
+// 4.5e-6 at 256; now below 2.6e-7.  The joins are fewer than those were: 30 passes at n = 30,011, k = 40
+// 20.9 -> 18.8 ms, 64 25.2 -> 22.2.
 #include <algorithm>
 #include <cmath>
 
@@ -48,7 +58,12 @@ using namespace tc;
 constexpr int kTilesThreads = 160;        // four consumer warps, one producer
 constexpr int kPiece = 16 * 1024;         // 32 columns x 128 rows
 constexpr int kRecord = kTilesRecord;     // the piece's labels: 32 byte offsets into a row of sums (label x 512), then
-                                          // a word whose bit m says that columns 4 m .. 4 m + 3 have four labels
+                                          // a word whose bit m says that columns 4 m .. 4 m + 3 have four labels, and, in
+                                          // a block's last piece, 12 bytes: the number of clusters that hold far more of
+                                          // the block than their share, and their labels
+constexpr int kDense = 11;                // the most of those
+constexpr int kPlanUpto = 16;             // the plan behind the records: upto[j], the clusters that join every 2^j
+constexpr int kPlanBytes = 4 * kPlanUpto + kMaxClusters;   // blocks or more often; the clusters, in that order
 constexpr int kStage = kPiece + 256;
 constexpr int kTilesMaxStages = 4;
 constexpr int kTilesBars = 2 * kTilesMaxStages;
@@ -60,6 +75,7 @@ struct TilesArgs {
     const uint8_t* lab8;
     const unsigned char* rec;
     float* Spart;
+    float2* Srun;
     double* zpart;
     double* zsum;
     double* cnorm;
@@ -85,8 +101,8 @@ struct TileUnit {
     const unsigned char* rec; // the pieces' label records
     const uint8_t* lab;
     float* S;                 // this segment's sums [c][i]
+    float2* run;              // and, while they grow, pairs of floats
     int n, k, T, I, s0, s1;
-    int sub;                  // column blocks a sum runs over
 };
 
 __device__ __forceinline__ const unsigned char* tile_at(const TileUnit& u, int I, int J) {
@@ -121,34 +137,95 @@ __device__ __forceinline__ void add4(uint32_t acc, const uint4& o, bool apart, f
         sts(p2, a2 + v2);
         sts(p3, a3 + v3);
     } else {
-        sts(p0, lds(p0) + v0);
-        sts(p1, lds(p1) + v1);
-        sts(p2, lds(p2) + v2);
-        sts(p3, lds(p3) + v3);
+        // equal labels are added up first
+        const float a0 = lds(p0), a1 = lds(p1), a2 = lds(p2), a3 = lds(p3);
+        float s3 = v3, s2 = v2, s1 = v1, s0 = v0;
+        s2 = p2 == p3 ? s2 + s3 : s2;
+        s0 = p0 == p1 ? s0 + s1 : s0;
+        const float r0 = a0 + (p0 == p2 ? s0 + s2 : p0 == p3 ? s0 + s3 : s0);
+        const float r1 = a1 + (p1 == p2 ? s1 + s2 : p1 == p3 ? s1 + s3 : s1);
+        sts(p3, a3 + s3);
+        sts(p2, a2 + s2);
+        sts(p1, r1);
+        sts(p0, r0);
     }
 }
 
-// The label records of a pass, a warp a piece of 32 columns (past n: label 0, never added).
-__device__ __forceinline__ void write_record(const uint8_t* __restrict__ lab, int n, int piece, unsigned char* rec) {
-    const int lane = threadIdx.x & 31, col = 32 * piece + lane;
-    const uint32_t l = col < n ? lab[col] : 0u;
-    // (every lane takes part in every exchange)
-    const uint32_t l1 = __shfl_xor_sync(0xffffffffu, l, 1), l2 = __shfl_xor_sync(0xffffffffu, l, 2),
-                   l3 = __shfl_xor_sync(0xffffffffu, l, 3);
-    const unsigned eq = __ballot_sync(0xffffffffu, l == l1 || l == l2 || l == l3);
-    uint32_t* r = reinterpret_cast<uint32_t*>(rec + (size_t)piece * kRecord);
-    r[lane] = l * 512u;
-    if (lane < 4) {
-        unsigned m = 0u;
-        for (int q = 0; q < 8; ++q) m |= (eq >> (4 * q) & 15u ? 0u : 1u) << q;
-        r[32 + lane] = m;
+// The plan of a pass, by one block: after how many column blocks (2^j) each cluster's sums join the
+// segment's, as an order of the clusters by j (equal ones in any order: their sums are their own).
+__device__ __forceinline__ void tile_plan(int n, int k, const int32_t* __restrict__ m, unsigned char* plan) {
+    __shared__ int upto[kPlanUpto], at[kPlanUpto];
+    if (threadIdx.x < kPlanUpto) upto[threadIdx.x] = 0;
+    __syncthreads();
+    int js[(kMaxClusters + 127) / 128];
+#pragma unroll
+    for (int x = 0; x < (kMaxClusters + 127) / 128; ++x) {
+        const int c = threadIdx.x + 128 * x;
+        js[x] = kPlanUpto - 1;   // an empty cluster, or none
+        if (c < k && m[c] > 0) {
+            const float mc = (float)m[c], blocks = fmaxf(32.f, 4.f * sqrtf(mc)) * (float)n / (128.f * mc);
+            js[x] = min(kPlanUpto - 2, max(0, (int)floorf(log2f(blocks) + 0.5f)));
+        }
+        if (c < k) atomicAdd(&upto[js[x]], 1);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int j = 0; j < kPlanUpto; ++j) {
+            at[j] = t;
+            t += upto[j];
+            upto[j] = t;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < (kMaxClusters + 127) / 128; ++x) {
+        const int c = threadIdx.x + 128 * x;
+        if (c < k) plan[4 * kPlanUpto + atomicAdd(&at[js[x]], 1)] = (unsigned char)c;
+    }
+    if (threadIdx.x < kPlanUpto) reinterpret_cast<int*>(plan)[threadIdx.x] = upto[threadIdx.x];
 }
-__global__ void __launch_bounds__(128) tile_records_kernel(const uint8_t* __restrict__ lab, int n, unsigned char* rec,
+
+// The label records of column block J, a warp a piece of 32 columns (past n: label 0, never added),
+// and the clusters that hold more than four times their share of it and 10 columns.  m: the clusters'
+// sizes.
+__device__ __forceinline__ void write_records(const uint8_t* __restrict__ lab, int n, int k, int J,
+                                              const int32_t* __restrict__ m, unsigned char* rec) {
+    __shared__ int hist[kMaxClusters], dense;
+    for (int c = threadIdx.x; c < k; c += blockDim.x) hist[c] = 0;
+    if (threadIdx.x == 0) dense = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, piece = 4 * J + (threadIdx.x >> 5), pieces = (n + 31) / 32;
+    if (piece < pieces) {
+        const int col = 32 * piece + lane;
+        const uint32_t l = col < n ? lab[col] : 0u;
+        // (every lane takes part in every exchange)
+        const uint32_t l1 = __shfl_xor_sync(0xffffffffu, l, 1), l2 = __shfl_xor_sync(0xffffffffu, l, 2),
+                       l3 = __shfl_xor_sync(0xffffffffu, l, 3);
+        const unsigned eq = __ballot_sync(0xffffffffu, l == l1 || l == l2 || l == l3);
+        if (col < n) atomicAdd(&hist[l], 1);
+        uint32_t* r = reinterpret_cast<uint32_t*>(rec + (size_t)piece * kRecord);
+        r[lane] = l * 512u;
+        if (lane < 4) {
+            unsigned f = 0u;
+            for (int q = 0; q < 8; ++q) f |= (eq >> (4 * q) & 15u ? 0u : 1u) << q;
+            r[32 + lane] = lane == 0 ? f : 0u;
+        }
+    }
+    __syncthreads();
+    unsigned char* list = rec + (size_t)min(4 * J + 3, pieces - 1) * kRecord + 4 * 33;
+    for (int c = threadIdx.x; c < k; c += blockDim.x)
+        if (hist[c] > 10 && (float)hist[c] > 512.f * (float)m[c] / (float)n + 10.f)
+            list[1 + atomicAdd(&dense, 1)] = (unsigned char)c;   // (11 columns each, of 128: at most kDense)
+    __syncthreads();
+    if (threadIdx.x == 0) list[0] = (unsigned char)dense;
+    if (J == 0) tile_plan(n, k, m, rec + (size_t)pieces * kRecord);
+}
+__global__ void __launch_bounds__(128) tile_records_kernel(const uint8_t* __restrict__ lab, int n, int k,
+                                                           const int32_t* __restrict__ counts, unsigned char* rec,
                                                            const LoopState* st, int eval) {
     if (pass_skip(st, eval)) return;
-    const int piece = blockIdx.x * 4 + (threadIdx.x >> 5);
-    if (piece < (n + 31) / 32) write_record(lab, n, piece, rec);
+    write_records(lab, n, k, (int)blockIdx.x, counts + (size_t)(st->iter & 1) * k, rec);
 }
 // a block a 128-column block of an instance
 __global__ void __launch_bounds__(128) batched_records_kernel(const BatchInst* I, int count, int eval) {
@@ -160,12 +237,11 @@ __global__ void __launch_bounds__(128) batched_records_kernel(const BatchInst* I
     }
     const BatchInst& b = I[lo];
     if (pass_skip(b.st, eval)) return;
-    const int piece = 4 * ((int)blockIdx.x - b.vblock0) + (threadIdx.x >> 5);
-    if (piece < (b.n + 31) / 32) write_record(b.lab8, b.n, piece, b.V);
+    write_records(b.lab8, b.n, b.k, (int)blockIdx.x - b.vblock0, b.counts + (size_t)(b.st->iter & 1) * b.k, b.V);
 }
 
-template <bool BATCH>
-__global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a) {
+template <bool BATCH, int CTAS>
+__global__ void __launch_bounds__(kTilesThreads, CTAS) reduce_tiles_kernel(TilesArgs a) {
     if constexpr (!BATCH) {
         if (pass_skip(a.st, a.eval_only)) {
             // J(final labels) is already known when the last pass changed nothing
@@ -213,6 +289,7 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
             u->s0 = q * (b.seglen >> 7);
             u->s1 = min(b.T, u->s0 + (b.seglen >> 7));
             u->S = b.Spart + (size_t)q * b.k * b.n;
+            u->run = b.Srun + (size_t)q * b.k * b.n;
         } else {
             q = x / a.T;
             u->I = x - q * a.T;
@@ -225,8 +302,8 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
             u->s0 = q * a.segblocks;
             u->s1 = min(a.T, u->s0 + a.segblocks);
             u->S = a.Spart + (size_t)q * a.k * a.n;
+            u->run = a.Srun + (size_t)q * a.k * a.n;
         }
-        u->sub = max(1, u->k / 2);   // 64 columns a cluster
         return true;
     };
     int stage = 0;
@@ -301,9 +378,16 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
             const int li = i < u.n ? (int)u.lab[i] : -1;
             float own = 0.f;   // (one fit) the row's sum over its own cluster
             float* out = u.S + i;
+            float2* run = u.run + i;
+            const int* upto = reinterpret_cast<const int*>(u.rec + (size_t)((u.n + 31) / 32) * kRecord);
+            const unsigned* order = reinterpret_cast<const unsigned*>(upto + kPlanUpto);   // four clusters a word
+            // clusters, from the front of the order, whose sums have joined by the end of step t
+            auto joined = [&](int t) { return t > 0 ? __ldg(upto + (31 - __clz(t))) : 0; };
+            bool all = false;    // all clusters' entries of run are set
             for (int s = u.s0; s < u.s1 && ok; ++s) {
                 const int J = s >= u.I ? s - u.I : s - u.I + u.T;
                 const bool rows = u.I <= J;
+                unsigned d0 = 0u, d1 = 0u, d2 = 0u;   // the block's dense clusters: number and labels
                 for (int p = 0; p < 4 && 128 * J + 32 * p < u.n; ++p) {
                     const int col = 128 * J + 32 * p;
                     const bool got = mbar_wait_for(full_bar(stage), phase, abort_flag, a.err, a.wait_ns);
@@ -314,6 +398,11 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
                     // column x of the piece: row 32 g + lane of a box at x ^ lane, or (transposed) row x
                     // of box g at lane ^ x
                     const uint32_t st = ring + (uint32_t)(stage * kStage), rec = st + kPiece;
+                    d0 = lds_u32(rec + 132);
+                    if (d0) {
+                        d1 = lds_u32(rec + 136);
+                        d2 = lds_u32(rec + 140);
+                    }
                     const uint32_t at = st + (uint32_t)((rows ? (32 * g + lane) * 128 : g * 4096) + 4 * lane);
                     if (col + 32 <= u.n) {
                         float v[32];
@@ -324,10 +413,10 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
 #pragma unroll
                             for (int x2 = 0; x2 < 32; ++x2) v[x2] = lds((at ^ (4u * x2)) + 128u * x2);
                         }
-                        const uint32_t apart = lds_u32(rec + 128);
+                        const uint32_t flags = lds_u32(rec + 128);
 #pragma unroll
                         for (int m = 0; m < 8; ++m)
-                            add4(acc_u, lds4(rec + 16 * m), apart >> m & 1u, v[4 * m], v[4 * m + 1], v[4 * m + 2],
+                            add4(acc_u, lds4(rec + 16 * m), flags >> m & 1u, v[4 * m], v[4 * m + 1], v[4 * m + 2],
                                  v[4 * m + 3]);
                     } else {
                         // the last columns of a ragged matrix (entries past n are not K)
@@ -340,16 +429,50 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
                     if (lane == 0) mbar_arrive(empty_bar(stage));
                     advance();
                 }
-                if (ok && (s + 1 == u.s1 || (s + 1 - u.s0) % u.sub == 0)) {
-                    // the run's sums join the segment's
-                    const bool first = s - u.s0 < u.sub;
-                    if (li >= 0) own += lds(acc_u + 512u * li);
-#pragma unroll 4
-                    for (int c = 0; c < u.k; ++c) {
-                        const float t = lds(acc_u + 512u * c);
+                if (!ok) break;
+                const bool last = s + 1 == u.s1;
+                const int t = s + 1 - u.s0;
+                if (d0 && !last) {
+                    if (!all && li >= 0)
+                        for (int e = joined(t - 1); e < u.k; ++e)
+                            run[(size_t)__ldg(reinterpret_cast<const unsigned char*>(order) + e) * u.n] = make_float2(0.f, 0.f);
+                    all = true;
+                    const int nd = min((int)(d0 & 255u), kDense);
+                    for (int e = 1; e <= nd; ++e) {
+                        const int c = (e < 4 ? d0 : e < 8 ? d1 : d2) >> (8 * (e & 3)) & 255;
+                        const float v = lds(acc_u + 512u * c);
                         sts(acc_u + 512u * c, 0.f);
-                        float* o = out + (size_t)c * u.n;
-                        if (li >= 0) *o = first ? t : *o + t;
+                        if (li < 0) continue;
+                        float2* r = run + (size_t)c * u.n;
+                        float2 h = *r;
+                        ff_add(h.x, h.y, v);
+                        *r = h;
+                    }
+                }
+                // the clusters whose turn it is (all at the end) join the segment's sums
+                const int nj = last ? u.k : __ldg(upto + (__ffs(t) - 1)), had = all ? u.k : nj ? joined(t - 1) : 0;
+                for (int e0 = 0; e0 < nj; e0 += 4) {
+                    const unsigned cs = __ldg(order + (e0 >> 2));
+                    float2 h[4];
+#pragma unroll
+                    for (int x = 0; x < 4; ++x)
+                        h[x] = li >= 0 && e0 + x < min(nj, had) ? run[(size_t)(cs >> (8 * x) & 255u) * u.n]
+                                                                 : make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        if (e0 + x >= nj) break;
+                        const int c = cs >> (8 * x) & 255;
+                        const float v = lds(acc_u + 512u * c);
+                        sts(acc_u + 512u * c, 0.f);
+                        ff_add(h[x].x, h[x].y, v);
+                        if (li < 0) continue;
+                        if (last) {
+                            const float sum = h[x].x + h[x].y;
+                            out[(size_t)c * u.n] = sum;
+                            if (c == li) own = sum;
+                        } else {
+                            run[(size_t)c * u.n] = h[x];
+                        }
                     }
                 }
             }
@@ -383,18 +506,23 @@ __global__ void __launch_bounds__(kTilesThreads) reduce_tiles_kernel(TilesArgs a
     }
 }
 
+// The kernel is built for at least 4 CTAs an SM (83 to 91 registers), and for batches of few clusters,
+// whose shared memory leaves room for a fifth, for 5 (80): left to itself the compiler took 64 and
+// spilled (n = 30,011, k = 100: 27.7 ms for 30 passes where 26.5; batch of k up to 20: 127.6, 129.4
+// with 4 and 123.4 with 5).
+using TilesFn = void (*)(TilesArgs);
+constexpr TilesFn kTilesOne = reduce_tiles_kernel<false, 4>, kTilesBatch = reduce_tiles_kernel<true, 4>,
+                  kTilesBatchFew = reduce_tiles_kernel<true, 5>;
+
 // Ring depth, CTAs an SM and shared memory for sums of up to k clusters: as many CTAs as fit
 // (their warps hide one another's chains of shared-memory additions), then the deeper ring.
-bool tiles_shape(int k, int per_sm_req, int* stages, int* per_sm, size_t* smem) {
+bool tiles_shape(TilesFn fn, int k, int per_sm_req, int* stages, int* per_sm, size_t* smem) {
     int best = 0;
     for (int S = kTilesMaxStages; S >= 2; --S) {
         const size_t bytes = (size_t)S * kStage + (size_t)k * 512 + (size_t)k * 32;
         int c = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, reduce_tiles_kernel<true>, kTilesThreads, bytes);
-        int c2 = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c2, reduce_tiles_kernel<false>, kTilesThreads, bytes);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, fn, kTilesThreads, bytes);
         cudaGetLastError();
-        c = std::min(c, c2);
         if (per_sm_req > 0 && c > per_sm_req) c = per_sm_req;
         if (c > best) {
             best = c;
@@ -409,22 +537,21 @@ bool tiles_shape(int k, int per_sm_req, int* stages, int* per_sm, size_t* smem) 
 }  // namespace
 
 cudaError_t configure_reduce_tiles(int smem_optin) {
-    cudaFuncAttributes f0, f1;
-    cudaError_t e = cudaFuncGetAttributes(&f0, reduce_tiles_kernel<false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&f1, reduce_tiles_kernel<true>);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(reduce_tiles_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 optin_minus_static(smem_optin, f0.sharedSizeBytes));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(reduce_tiles_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 optin_minus_static(smem_optin, f1.sharedSizeBytes));
-    return e;
+    for (TilesFn fn : {kTilesOne, kTilesBatch, kTilesBatchFew}) {
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     optin_minus_static(smem_optin, fa.sharedSizeBytes));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 bool plan_reduce_tiles(int n, int k, int num_sms, ReducePlan* p) {
     int S, per_sm;
     size_t smem;
-    if (!tiles_shape(k, 0, &S, &per_sm, &smem)) return false;
+    if (!tiles_shape(kTilesOne, k, 0, &S, &per_sm, &smem)) return false;
     const int T = (n + 127) / 128, grid = num_sms * per_sm;
     // Segments: whole rounds of the grid's CTAs, against the slots' traffic (8 k n bytes a segment
     // beside 2 n^2 of K, and the argmin's walk over them).
@@ -448,11 +575,11 @@ bool plan_reduce_tiles(int n, int k, int num_sms, ReducePlan* p) {
     return true;
 }
 
-size_t tiles_record_bytes(int n) { return (size_t)((n + 31) / 32) * kRecord; }
+size_t tiles_record_bytes(int n) { return (size_t)((n + 31) / 32) * kRecord + kPlanBytes; }
 
 cudaError_t launch_reduce_tiles(const PassBuffers& b, const ReducePlan& plan, int* err, int eval_only, cudaStream_t s,
                                 int stall_ms) {
-    tile_records_kernel<<<(b.n + 127) / 128, 128, 0, s>>>(b.lab8, b.n, b.sym_meta, b.st, eval_only);
+    tile_records_kernel<<<(b.n + 127) / 128, 128, 0, s>>>(b.lab8, b.n, b.k, b.counts, b.sym_meta, b.st, eval_only);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     TilesArgs a{};
@@ -465,6 +592,7 @@ cudaError_t launch_reduce_tiles(const PassBuffers& b, const ReducePlan& plan, in
     a.lab8 = b.lab8;
     a.rec = b.sym_meta;
     a.Spart = b.Spart;
+    a.Srun = b.Srun;
     a.zpart = b.zpart;
     a.zsum = b.zsum;
     a.cnorm = b.cnorm;
@@ -478,14 +606,16 @@ cudaError_t launch_reduce_tiles(const PassBuffers& b, const ReducePlan& plan, in
     a.err = err;
     a.stall = stall_ms > 0 ? 1 : 0;
     a.wait_ns = stall_ms > 0 ? (unsigned long long)stall_ms * 1000000ull : kWaitLimitNs;
-    reduce_tiles_kernel<false><<<plan.grid, kTilesThreads, plan.smem, s>>>(a);
+    kTilesOne<<<plan.grid, kTilesThreads, plan.smem, s>>>(a);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ batched mode
 
 bool plan_batched_tiles(BatchPlan* bp, int num_sms, int per_sm_req) {
-    if (!tiles_shape(bp->kmax, per_sm_req, &bp->mstages, &bp->per_sm, &bp->smem)) return false;
+    if (!tiles_shape(kTilesBatchFew, bp->kmax, per_sm_req, &bp->mstages, &bp->per_sm, &bp->smem)) return false;
+    if (bp->per_sm < 5 && !tiles_shape(kTilesBatch, bp->kmax, per_sm_req, &bp->mstages, &bp->per_sm, &bp->smem))
+        return false;
     bp->warps = 4;
     bp->grid = num_sms * bp->per_sm;
     return true;
@@ -506,7 +636,7 @@ cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const B
     a.err = err;
     a.wait_ns = kWaitLimitNs;
     const int grid = bp.units < bp.grid ? bp.units : bp.grid;
-    reduce_tiles_kernel<true><<<grid, kTilesThreads, bp.smem, s>>>(a);
+    (bp.per_sm < 5 ? kTilesBatch : kTilesBatchFew)<<<grid, kTilesThreads, bp.smem, s>>>(a);
     return cudaGetLastError();
 }
 
