@@ -19,15 +19,15 @@
 //
 // What bounds it: the chain of a warp's shared-memory additions, with k x 512 bytes of sums a CTA
 // (2 CTAs an SM at k = 100, 3 at 64) to hide it behind; without the additions the stream takes
-// 0.49 ms where it takes 0.75 (k = 100, n = 30,011; HBM delivers 2.05 GB of the 3.6 GB square).
+// 0.49 ms where it takes 0.73 (k = 100, n = 30,011; HBM delivers 2.05 GB of the 3.6 GB square).
 // Two warps a row group, half a piece's columns each with sums of their own (16 consumer warps an
 // SM in place of 12 at k = 64, 8 in one CTA at 100), were slower: 142 -> 153 ms for the batch below
 // (30 passes), 27.0 -> 32.2 ms for 30 passes here.
 // So the labels come as byte offsets with the piece (the record below: no label arithmetic, no
 // global load) and four columns of different labels are added together.  The row-major stream it
 // replaces (iterate.cu: a lane every 32nd float4, k x 32 sums to add up a row, 15 instructions an
-// element) took 1.09 ms there, 0.81 at k = 64 (now 0.71), 0.79 at 40 (0.57) and 1.75 at 200
-// (1.38).  Batch of 256 instances, n 500 to 8,000, k up to 64: 4.7 -> 3.9 ms a pass.  A first form
+// element) took 1.09 ms there, 0.81 at k = 64 (now 0.66), 0.79 at 40 (0.52) and 1.75 at 200
+// (1.36).  Batch of 256 instances, n 500 to 8,000, k up to 64: 4.7 -> 3.6 ms a pass.  A first form
 // with 32 x 32 pieces of row-major rows (128 bytes at a 120 KB stride) stayed at 3.2 TB/s.
 //
 // Every so many column blocks a cluster's sums join the segment's, a pair of floats (Srun) until the
@@ -36,12 +36,13 @@
 // chain of L additions of one size is off by about 0.4 u sqrt(L / 3) of its own sum (u = 2^-24), m / L
 // such chains by 0.4 u L / sqrt(3 m), and L = 4 sqrt(2 m) makes that the 1.3 u of the row-major stream
 // (32 lanes' partial sums, added one after the other): so S is no further off than there for clusters
-// of any size, with few joins (their traffic stays in L2, but 1 in 8 KB read was enough to be seen).
+// of any size, with few joins.
 // A cluster that holds four times its share of a block's columns (points in the order of their
-// classes) joins at the block's end, and equal labels among four columns are added up first.  As runs of 64 k columns for
-// all clusters, joined in FP32, a row's sum over one cluster of 30,011 was 1.5e-6 off at k = 100 and
-// 4.5e-6 at 256; now below 2.6e-7.  The joins are fewer than those were: 30 passes at n = 30,011, k = 40
-// 20.9 -> 18.8 ms, 64 25.2 -> 22.2.
+// classes) joins at the block's end, and equal labels among four columns are added up first.  (As runs
+// of 64 k columns for all clusters, joined in FP32, a row's sum over one cluster of 30,011 was 1.5e-6
+// off at k = 100 and 4.5e-6 at 256; now below 2.6e-7.  There are fewer joins of clusters of one size now,
+// and equal labels do not wait for one another: 30 passes at n = 30,011, k = 40 20.9 -> 19.4 ms, 64
+// 25.4 -> 23.7, 100 27.0 -> 26.5, with 97% in one cluster 27.6 -> 27.3; the batch below 146 -> 136.)
 #include <algorithm>
 #include <cmath>
 
@@ -506,10 +507,10 @@ __global__ void __launch_bounds__(kTilesThreads, CTAS) reduce_tiles_kernel(Tiles
     }
 }
 
-// The kernel is built for at least 4 CTAs an SM (83 to 91 registers), and for batches of few clusters,
-// whose shared memory leaves room for a fifth, for 5 (80): left to itself the compiler took 64 and
-// spilled (n = 30,011, k = 100: 27.7 ms for 30 passes where 26.5; batch of k up to 20: 127.6, 129.4
-// with 4 and 123.4 with 5).
+// The kernel is built for at least 4 CTAs an SM (87 to 89 registers), and for batches of few clusters,
+// whose shared memory leaves room for a fifth, for 5 (72).  Left to itself the compiler takes 64 and
+// spills (with joins every 64 columns a cluster: 27.7 ms for 30 passes at n = 30,011, k = 100
+// where 26.5 with 4; batch of k up to 20 127.6, 129.4 with 4 and 123.4 with 5).
 using TilesFn = void (*)(TilesArgs);
 constexpr TilesFn kTilesOne = reduce_tiles_kernel<false, 4>, kTilesBatch = reduce_tiles_kernel<true, 4>,
                   kTilesBatchFew = reduce_tiles_kernel<true, 5>;
