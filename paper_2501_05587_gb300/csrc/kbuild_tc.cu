@@ -59,6 +59,7 @@
 // runs out sets *err, raises a shared abort flag that ends every role's loop,
 // waits (bounded again) for the CTA's own TMA copies and MMAs in flight,
 // frees TMEM and returns; the host reports POPCORN_ERR_TIMEOUT.
+#include <cstdlib>
 #include <cstring>
 
 #include <cuda.h>
@@ -112,6 +113,10 @@ struct TcArgs {
     float* kdiag;
     const SplitState* split;  // SPLIT: the device's decision and scale
     int* err;
+    // Error-path tests only (0 in every ordinary launch): CTA 0 leaves its first stage's copies out and
+    // every wait of the launch gives up after wait_ns.
+    int stall;
+    unsigned long long wait_ns;
 };
 
 // tile t -> (row block i, column pair q); false for a place of the walk that holds no tile.  The
@@ -414,25 +419,28 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             uint32_t issued_parity[kStages];
             bool issued[kStages];
             for (int s = 0; s < kStages; ++s) issued[s] = false;
-            bool ok = true;
+            bool ok = true, first = true;
             for (long long t = blockIdx.x; t < a.tiles && ok; t += G) {
                 int i, q;
                 if (!tile_coords(t, a.T, a.T2, a.full, &i, &q)) continue;
                 for (int kb = 0; kb < a.nkb; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, a.err)) {
+                    if (!mbar_wait_for(empty_bar(stage), phase ^ 1u, abort_flag, a.err, a.wait_ns)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t st = sbase + (uint32_t)(stage * kStageBytes);
-                    mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kStageBytes);
-                    tma_load_2d(st + kColsHi, &map_c, kb * DK, q * 2 * BM, full_bar(stage));
-                    tma_load_2d(st + kRowsHi, &map_r, kb * DK, i * BM, full_bar(stage));
-                    if constexpr (X3) {
-                        tma_load_2d(st + kColsLo, &map_c, a.dpad + kb * DK, q * 2 * BM, full_bar(stage));
-                        tma_load_2d(st + kRowsLo, &map_r, a.dpad + kb * DK, i * BM, full_bar(stage));
+                    if (!(a.stall && blockIdx.x == 0 && first)) {
+                        const uint32_t st = sbase + (uint32_t)(stage * kStageBytes);
+                        mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kStageBytes);
+                        tma_load_2d(st + kColsHi, &map_c, kb * DK, q * 2 * BM, full_bar(stage));
+                        tma_load_2d(st + kRowsHi, &map_r, kb * DK, i * BM, full_bar(stage));
+                        if constexpr (X3) {
+                            tma_load_2d(st + kColsLo, &map_c, a.dpad + kb * DK, q * 2 * BM, full_bar(stage));
+                            tma_load_2d(st + kRowsLo, &map_r, a.dpad + kb * DK, i * BM, full_bar(stage));
+                        }
+                        issued[stage] = true;
+                        issued_parity[stage] = phase;
                     }
-                    issued[stage] = true;
-                    issued_parity[stage] = phase;
+                    first = false;
                     if (++stage == S) {
                         stage = 0;
                         phase ^= 1u;
@@ -459,7 +467,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint64_t desc0 = DK == 32 ? sw64_desc(sbase) : sw128_desc(sbase);
             // both halves of the next buffer have been read by the epilogue
             auto take_buffer = [&](int ab, uint32_t use) {
-                if (!mbar_wait(acce_bar(ab), (use & 1u) ^ 1u, abort_flag, a.err)) return false;
+                if (!mbar_wait_for(acce_bar(ab), (use & 1u) ^ 1u, abort_flag, a.err, a.wait_ns)) return false;
                 tc_fence_after();
                 return true;
             };
@@ -470,7 +478,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 if (SPLIT && a.full) below = 2 * q < i;
                 if (!SPLIT && !take_buffer(fill & 1, (uint32_t)(fill >> 1))) break;
                 for (int kb = 0; kb < a.nkb && ok; ++kb) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag, a.err)) {
+                    if (!mbar_wait_for(full_bar(stage), phase, abort_flag, a.err, a.wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -584,7 +592,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 for (int x = 0; x < BM / 2; ++x) acc[x] = 0ull;
                 for (int kb = 0; kb < a.nkb; ++kb, ++fill) {
                     const int ab = fill & 1;
-                    const bool got = mbar_wait(accf_bar(ab), (uint32_t)(fill >> 1) & 1u, abort_flag, a.err);
+                    const bool got = mbar_wait_for(accf_bar(ab), (uint32_t)(fill >> 1) & 1u, abort_flag, a.err, a.wait_ns);
                     if (__any_sync(0xffffffffu, !got)) {
                         ok = false;
                         break;
@@ -631,7 +639,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 }
             } else {
                 const int ab = fill & 1;
-                ok = mbar_wait(accf_bar(ab), (uint32_t)(fill >> 1) & 1u, abort_flag, a.err);
+                ok = mbar_wait_for(accf_bar(ab), (uint32_t)(fill >> 1) & 1u, abort_flag, a.err, a.wait_ns);
                 ++fill;
                 if (!named_bar_all(b.bar, 128, ok && !*abort_flag)) break;
                 tc_fence_after();
@@ -992,6 +1000,12 @@ cudaError_t launch_tiles(int mode, const void* W, int n, int64_t ldw, int dpad, 
     a.kdiag = kdiag;
     a.split = split;
     a.err = err;
+    // Error-path test hook: POPCORN_TEST_BUILD_STALL_MS=<ms> in the environment makes one wait of every
+    // tensor-core build run out.  Unset in every ordinary run.
+    const char* env = getenv("POPCORN_TEST_BUILD_STALL_MS");
+    const int stall_ms = env && *env ? atoi(env) : 0;
+    a.stall = stall_ms > 0 && stall_ms <= 10000 ? 1 : 0;
+    a.wait_ns = a.stall ? (unsigned long long)stall_ms * 1000000ull : kWaitLimitNs;
     const int grid = (int)(a.tiles < num_sms ? a.tiles : num_sms);
     tc_fn(mode, out, kp.kind)<<<grid, NTHREADS, kSmemBytes, s>>>(mr, mc, mkd, mkt, a);
     return cudaGetLastError();

@@ -463,8 +463,9 @@ cudaError_t launch_batched_kbuild_simt(const BatchInst* dI, const BatchPlan& bp,
 // seglen columns (a multiple of 128).  Plan: ring depth (mstages), CTAs an SM (per_sm_req caps it),
 // shared memory for sums of kmax clusters.
 bool plan_batched_tiles(BatchPlan* bp, int num_sms, int per_sm_req = 0);
+// stall_ms as launch_reduce_sym.
 cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err, int eval,
-                                 cudaStream_t s);
+                                 cudaStream_t s, int stall_ms = 0);
 // the rest of a pass after its K stream: z (with per-instance finalization) and the argmin
 cudaError_t launch_batched_finish(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
 cudaError_t launch_batched_copy_labels(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);

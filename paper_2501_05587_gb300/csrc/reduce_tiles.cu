@@ -623,7 +623,7 @@ bool plan_batched_tiles(BatchPlan* bp, int num_sms, int per_sm_req) {
 }
 
 cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err, int eval,
-                                 cudaStream_t s) {
+                                 cudaStream_t s, int stall_ms) {
     batched_records_kernel<<<bp.vblocks, 128, 0, s>>>(dI, bp.count, eval);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -635,7 +635,8 @@ cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const B
     a.stages = bp.mstages;
     a.kmax = bp.kmax;
     a.err = err;
-    a.wait_ns = kWaitLimitNs;
+    a.stall = stall_ms > 0 ? 1 : 0;
+    a.wait_ns = stall_ms > 0 ? (unsigned long long)stall_ms * 1000000ull : kWaitLimitNs;
     const int grid = bp.units < bp.grid ? bp.units : bp.grid;
     (bp.per_sm < 5 ? kTilesBatch : kTilesBatchFew)<<<grid, kTilesThreads, bp.smem, s>>>(a);
     return cudaGetLastError();
