@@ -578,17 +578,30 @@ __device__ __forceinline__ void zreduce_body(const ZArgs& a, int block, int nblo
     __syncthreads();
     if (l >= 0) val_s[cnt_s[warp][l] + wrank] = v;
     __syncthreads();
-    // A few lanes a cluster (all clusters at once on the block's 1024 threads): they stride its
-    // sorted rows and add up in a fixed order.  (A warp a cluster spent 160 of its FP64 lane
-    // additions on the butterfly for the 10 to 30 rows it has: 101 us on the 256-instance batch, now 92.)
+    // Clusters of up to 256 of the block's rows: a few lanes each, all clusters at once on the block's
+    // 1024 threads; they stride its sorted rows and add up in a fixed order.  (A warp a cluster spent 160
+    // of its FP64 lane additions on the butterfly for the 10 to 30 rows it has: 101 us on the 256-instance
+    // batch, then 92.)  Larger ones, four a block at most: a warp each, whose chain of additions is a
+    // quarter as long (n = 30,000: k = 1 22.5 -> 19 us, k = 2 18 -> 17, k = 100 with 97% in one cluster
+    // 35.6 -> 32.8; from 64 rows a batch of k = 4 to 8 was 0.3% slower).
+    constexpr int kLarge = 256;
     {
         const int L = a.k <= kZReduceRows / 8 ? 8 : 4;
         const int c = (int)threadIdx.x / L, j = (int)threadIdx.x & (L - 1);
+        const bool mine = c < a.k && cstart[c + 1] - cstart[c] <= kLarge;
         double t = 0.0;
-        if (c < a.k)
+        if (mine)
             for (int r = cstart[c] + j; r < cstart[c + 1]; r += L) t += val_s[r];
         for (int o = L >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (c < a.k && j == 0) a.zpart[(size_t)block * a.k + c] = t;
+        if (mine && j == 0) a.zpart[(size_t)block * a.k + c] = t;
+    }
+    for (int c = warp; c < a.k; c += NW) {
+        if (cstart[c + 1] - cstart[c] <= kLarge) continue;
+        double t = 0.0;
+        for (int r = cstart[c] + lane; r < cstart[c + 1]; r += 32) t += val_s[r];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) a.zpart[(size_t)block * a.k + c] = t;
     }
     __threadfence();
     __syncthreads();
