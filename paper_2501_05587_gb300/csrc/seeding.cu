@@ -222,7 +222,9 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
         }
         __syncthreads();
         // every CTA alike: the running sums of the CTAs in order, the target, and the first CTA
-        // whose running sum exceeds it
+        // whose running sum exceeds it.  (Neighbouring running sums come from scans of different
+        // shape, so one may exceed another by a rounding with nothing added between them: here and below
+        // only what has a positive weight is taken.)
         if (warp == 0) {
             const int per = (G + 31) / 32, b0 = min(G, lane * per), b1 = min(G, b0 + per);
             double s = 0.0;
@@ -239,7 +241,7 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
             double run = before;
             for (int x = b0; x < b1 && b < 0; ++x) {
                 const double next = run + part_s[x];
-                if (next > target) b = x;
+                if (next > target && part_s[x] > 0.0) b = x;
                 else run = next;
             }
             const unsigned have = __ballot_sync(0xffffffffu, b >= 0);
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
                 s += x;
             }
             block_scan(s, inc, wsum);
-            if (inc[threadIdx.x] > tgt) atomicMin(&pick_s, (int)threadIdx.x);
+            if (s > 0.0 && inc[threadIdx.x] > tgt) atomicMin(&pick_s, (int)threadIdx.x);
             if (lastpos >= 0) atomicMax(&pos_s, lastpos);
             __syncthreads();
             const int pick = pick_s;
@@ -285,13 +287,14 @@ __global__ void __launch_bounds__(kSeedThreads, 1) kmeanspp_kernel(SeedArgs a) {
                 double run = pick ? inc[pick - 1] : 0.0;
                 int found = -1;
                 for (int r = r0; r < r1; ++r) {
-                    run += __ldcg(Db + r);
-                    if (run > tgt) {
+                    const double x = __ldcg(Db + r);
+                    run += x;
+                    if (run > tgt && x > 0.0) {
                         found = r;
                         break;
                     }
                 }
-                if (found < 0) found = lastpos >= 0 ? lastpos : max(r0, min(r1, brows) - 1);   // rounding at the chunk's end
+                if (found < 0) found = lastpos;   // rounding at the chunk's end
                 pos_s = found;
             }
             __syncthreads();
