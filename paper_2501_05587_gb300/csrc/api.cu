@@ -1329,7 +1329,6 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.T = (n + 127) / 128;
         b.tile0 = bp.tiles;
         bp.tiles += (long long)b.T * (b.T + 1) / 2;
-        b.ldk = (n + 3) / 4 * 4;
         b.n = n;
         b.k = k;
         if (half) {   // S written once a row
@@ -1427,7 +1426,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     auto upload_units = [&]() {
         return cudaMemcpyAsync(base + units_off, hunits.data(), sizeof(int2) * hunits.size(), cudaMemcpyHostToDevice, s);
     };
-    POPCORN_CUDA(upload_units());
+    if (half) POPCORN_CUDA(upload_units());   // (FP32 K: once the schedule is known)
     BatchInst* dI = reinterpret_cast<BatchInst*>(base + inst_off);
     POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count, cudaMemcpyHostToDevice, s));
     int* err = reinterpret_cast<int*>(base + err_off);
@@ -1470,7 +1469,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
             } else {
                 for (int t = 0; t < count; ++t)
                     POPCORN_CUDA(launch_kbuild_tc(h[t].P, h[t].n, h[t].d, h[t].ldp, h[t].kp, opt.precision, h[t].K,
-                                                  h[t].ldk, h[t].kdiag, base + tc_off, err, dev->sms, s, nullptr,
+                                                  0, h[t].kdiag, base + tc_off, err, dev->sms, s, nullptr,
                                                   kPackedSw4));
             }
             cudaEvent_t t0, t1;
@@ -1563,7 +1562,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         for (int t = 0; t < count && cap == POPCORN_OK; ++t) {
             const BatchInst& b = h[t];
             step(launch_kbuild_tc(b.P, b.n, b.d, b.ldp, b.kp, opt.precision,
-                                  half ? reinterpret_cast<float*>(b.Kh) : b.K, b.ldk, b.kdiag, base + tc_off, err,
+                                  half ? reinterpret_cast<float*>(b.Kh) : b.K, 0, b.kdiag, base + tc_off, err,
                                   dev->sms, cs, &launches, half ? kPackedSw128H : kPackedSw4, 0, half),
                  "tensor-core K build");
         }

@@ -571,13 +571,13 @@ __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst*
     TK* K = sizeof(TK) == 2 ? reinterpret_cast<TK*>(x.Kh) : reinterpret_cast<TK*>(x.K);
     switch (x.kp.kind) {
         case POPCORN_LINEAR:
-            kbuild_tile<POPCORN_LINEAR, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, x.ldk, x.kdiag, x.T, t, sm);
+            kbuild_tile<POPCORN_LINEAR, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, 0, x.kdiag, x.T, t, sm);
             break;
         case POPCORN_POLYNOMIAL:
-            kbuild_tile<POPCORN_POLYNOMIAL, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, x.ldk, x.kdiag, x.T, t, sm);
+            kbuild_tile<POPCORN_POLYNOMIAL, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, 0, x.kdiag, x.T, t, sm);
             break;
         default:
-            kbuild_tile<POPCORN_GAUSSIAN, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, x.ldk, x.kdiag, x.T, t, sm);
+            kbuild_tile<POPCORN_GAUSSIAN, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, 0, x.kdiag, x.T, t, sm);
             break;
     }
 }

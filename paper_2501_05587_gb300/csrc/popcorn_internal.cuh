@@ -407,8 +407,7 @@ struct BatchInst {
     KernParams kp;
     int T;                    // 128-row tiles of K
     long long tile0;          // first flattened upper-triangle tile
-    float* K;
-    int64_t ldk;
+    float* K;                 // FP32 K: the packed triangle
     float* kdiag;
     int n, k, nseg, seglen;
     uint8_t* lab8;
