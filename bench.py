@@ -11,7 +11,7 @@ then per pass the K-streaming segmented reduction (the symmetric pass: blocks on
 and above the diagonal, row and column sums), the self-similarity sums, and the
 distance/argmin/histogram pass.
 
-``value`` is the plain FP32 form (CUDA-core K build).  The same line carries the
+``value`` is the plain FP32 form (K build on the tensor cores from two FP16 parts).  The same line carries the
 BF16X3 and BF16 forms (tensor-core K builds) and BF16X3 with K stored in FP16 (the
 tensor-core symmetric pass) with their objective errors against the FP64 oracle, the
 rooflines of the dominant kernels, and extra legs for the other workloads: rings
@@ -238,7 +238,8 @@ def kbuild_roofline(wl, precision, kb_ms, pk, k_storage="fp32"):
             expand = 4.0 * np.sqrt(d) * 2.0 ** -24 * maxr * c <= 1e-6
             form = "norm expansion (Eq. 12)" if expand else "coordinate differences"
             per = 1.0 if expand else 2.0
-        # the split build's lines (kbuild_split_applies, split_decide_kernel in csrc/kbuild_tc.cu)
+        # the split build's lines (kbuild_split_applies, split_decide in csrc/kbuild_tc.cu; the workloads'
+        # columns and rows are within its range)
         fill = float(np.count_nonzero(wl.P)) / (n * d)
         split = (max(136, T * (T + 1) // 2) * wl.d >= 65000 and per == 1.0
                  and (wl.d >= 48 if form else wl.d >= 128 and d * fill * fill >= 128))
@@ -262,8 +263,9 @@ def kbuild_roofline(wl, precision, kb_ms, pk, k_storage="fp32"):
     ach = flops / sec / 1e12
     return {"kernel": "kbuild_tc_kernel", "bound": "tensor", "achieved": ach, "peak": pk["bf16"], "unit": "TFLOP/s",
             "frac": ach / pk["bf16"],
-            "traffic": (recorded_traffic("kbuild_tc_kernel" + ("" if k_storage == "fp32" else f"[{k_storage} K]"),
-                                         "kbuild_tc.cu", wl.name) if precision == "bf16x3" else None),
+            "traffic": recorded_traffic({("fp32", "fp32"): "kbuild_tc_kernel[fp32 split]",
+                                         ("bf16x3", "fp16"): "kbuild_tc_kernel[fp16 K]"}.get((precision, k_storage), ""),
+                                        "kbuild_tc.cu", wl.name),
             "k_storage": k_storage,
             "peak_source": pk["source"] + " bf16 burst",
             "executed_mma_flops_per_launch": flops, "avg_launch_ms": kb_ms}

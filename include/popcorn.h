@@ -132,7 +132,8 @@ typedef struct {
                                    FP16 / BF16 K from a BF16 / BF16X3 build; with more than 32
                                    clusters and an FP32 K from n = 6145 the packed triangle by
                                    block rows (each 128-block for its rows and, transposed, for
-                                   its columns, the second time from L2); else the full square.
+                                   its columns, the second time from L2; 12 n k bytes of sums a
+                                   segment); else the full square.
                                    1 = symmetric (k <= 32; larger k as under 0): only the 128 x 128 blocks on and above the
                                    diagonal (K is symmetric, and is then stored as that packed
                                    triangle; an FP16 / BF16 K is written as half tiles by a
@@ -376,8 +377,9 @@ typedef struct {
  * floor(u[0] n); for t >= 1, point t is the first i in index order at which the running sum
  * of D exceeds u[t] sum_i D(i) (floor(u[t] n) when that sum is 0, i.e. every point
  * coincides with a chosen one).  labels_out[i] is the index t of i's nearest chosen point
- * (the lowest t on ties).  All sums are taken in a fixed order: repeated calls give the
- * same result.
+ * (the lowest t on ties).  A point with D = 0 is never taken while another has D > 0.  All sums
+ * are taken in a fixed order: repeated calls give the same result.  Workspace: 16 n bytes and a few
+ * KB, besides device copies of host arguments.
  *
  *   P           host or device, n x d FP32, leading dimension ldp >= d.
  *   u           host or device, k doubles in [0, 1).

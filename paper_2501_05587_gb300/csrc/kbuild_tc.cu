@@ -38,7 +38,7 @@
 //   FP32    (SPLIT) W = [hi | lo] in FP16 of the points times a power of two s:
 //           hi = fp16(s p), lo = fp16(s p - hi), which represent p to 2^-23 of itself
 //           (hi and lo carry 11 bits each and lo's sign one more: 1 + 2^-12 + 2^-23 is 2^-23 off), or
-//           to 2^-27 of its row's and column's largest value (see split_decide_kernel).
+//           to 2^-27 of its row's and column's largest value (see split_decide).
 //           The products are exact in FP32, but the tensor core adds them with
 //           truncation: left in TMEM over a long row the sum drifts low by half an ulp an
 //           MMA (measured at d = 784 on uniform points: relative error 6.1e-6 against
@@ -1057,8 +1057,8 @@ cudaError_t launch_kbuild_tc(const float* P, int n, int d, int64_t ldp, KernPara
 }
 
 // Where the split build is the faster one.  The CUDA-core build takes its tiles in waves, each
-// as long as d; the split build costs five more launches (about 25 us) and then a small
-// fraction of that.  Measured (a whole call, us, CUDA cores / split): n = 2,000: d = 400 78 / 77,
+// as long as d; the split build costs four more launches (20 to 25 us, also where it refuses the
+// points) and then a small fraction of that.  Measured (a whole call, us, CUDA cores / split): n = 2,000: d = 400 78 / 77,
 // 512 89 / 78, 784 109 / 91; n = 4,000: d = 128 91 / 88, 256 140 / 95; n = 6,000: d = 48 90 / 101,
 // 96 127 / 103; n = 8,000: d = 64 154 / 134, 784 953 / 266; n = 20,000: d = 48 609 / 441,
 // 784 5397 / 1163.  Below 128 columns the device's rule on the number of terms refuses dot
