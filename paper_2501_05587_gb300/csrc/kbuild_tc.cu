@@ -115,7 +115,7 @@ constexpr uint32_t kTmemCols = 512;          // 2 buffers x 256 columns
 struct TcArgs {
     int n, T, T2, nkb;        // rows, 128-blocks, column pairs, k-blocks per part
     int dpad;                 // elements per part (W row = [hi | lo] for BF16X3 and SPLIT)
-    long long tiles;          // places of the walk over the tiles (tile_coords)
+    long long tiles;
     float* K;                 // row-major square (SPLIT: the diagonal blocks are stored with plain stores)
     int64_t ldk;
     float* Kp;                // block-packed K (tile (I, J), I <= J, at its row-by-row triangle index
@@ -135,43 +135,48 @@ struct TcArgs {
     unsigned long long wait_ns;
 };
 
-// tile t -> (row block i, column pair q); false for a place of the walk that holds no tile.  The
-// walk goes through bands of kBand row blocks, and in a band column pair by column pair, so that
-// the tiles in flight at a time (152) touch kBand row blocks and about 19 column pairs (20 MB of
-// W at d = 784): W is read from HBM once a band.  Row block by row block, it was read once a row
-// block: 64 GB at n = 70,000, as much HBM time as the whole build takes now (11.8 -> 10.9 ms;
-// BF16 4.96 -> 4.17).  Band b of the upper
-// triangle is the rectangle of its row blocks and the pairs from its first diagonal block on
-// (12 places of it lie below the diagonal), and starts at kBand (b T2 - (kBand / 4) b (b - 1)):
-// a binary search over b, no floating point.  The full schedule takes every pair.
+// tile t -> (row block i, column pair q).  The walk goes through bands of kBand row blocks, and in
+// a band column pair by column pair, so that the tiles in flight at a time (152) touch kBand row blocks
+// and about 19 column pairs (20 MB of W at d = 784): W is read from HBM once a band.  Row block by row
+// block, it was read once a row block: 64 GB at n = 70,000, as much HBM time as the whole build takes
+// now (11.8 -> 10.9 ms; BF16 4.96 -> 4.17).  (Bands of 2 gained 3% on rows of 400 KB and lost 10% at
+// d = 30,000.)
+// Band b of the upper triangle holds its row blocks and the pairs from its first diagonal block on;
+// pair j of a band holds the first 2 j + 2 of its R row blocks (block (2q + 1, 2q) is the only one
+// below the diagonal), so the pairs before F = R / 2 hold F (F + 1) tiles and a whole band
+// kBand (kBand - 2) / 4 = 12 fewer than its rectangle.  (Walked with the rectangle's empty places, which
+// the static round-robin gave to CTAs like tiles, BF16X3 took 2.30 ms at n = 10,000, d = 10,000 where it
+// takes 2.11, and 49 at n = 50,000 where 45.6; FP32 68.3 and 63.4.)  A binary search over b, no
+// floating point.  The full schedule takes every pair.
 constexpr int kBand = 8;
-__device__ __forceinline__ bool tile_coords(long long t, int T, int T2, int full, int* i, int* q) {
-    int lo = 0;
-    long long off = 0;
-    if (full) {
-        lo = (int)(t / ((long long)kBand * T2));
-        off = (long long)lo * kBand * T2;
-    } else {
-        int hi = (T - 1) / kBand;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            const long long o = (long long)kBand * ((long long)mid * T2 - (long long)(kBand / 4) * mid * (mid - 1));
-            if (o <= t) lo = mid;
-            else hi = mid - 1;
-        }
-        off = (long long)kBand * ((long long)lo * T2 - (long long)(kBand / 4) * lo * (lo - 1));
-    }
-    const int rows = min(kBand, T - kBand * lo);
-    const int r = (int)(t - off);
-    *i = kBand * lo + r % rows;
-    *q = (full ? 0 : kBand / 2 * lo) + r / rows;
-    return full || 2 * *q + 1 >= *i;
+__host__ __device__ inline long long band_start(long long b, int T2, int full) {
+    if (full) return b * kBand * T2;
+    return b * kBand * T2 - (long long)(kBand * kBand / 4) * b * (b - 1) - b * (kBand * (kBand - 2) / 4);
 }
-// The number of places of the walk.
+__device__ __forceinline__ void tile_coords(long long t, int T, int T2, int full, int* i, int* q) {
+    int lo = 0, hi = (T - 1) / kBand;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (band_start(mid, T2, full) <= t) lo = mid;
+        else hi = mid - 1;
+    }
+    const int R = min(kBand, T - kBand * lo), F = full ? 0 : R / 2;
+    int r = (int)(t - band_start(lo, T2, full));
+    int j;
+    if (r < F * (F + 1)) {
+        j = (r >= 2) + (r >= 6) + (r >= 12);   // (F <= 4)
+        r -= j * (j + 1);
+    } else {
+        r -= F * (F + 1);
+        j = F + r / R;
+        r %= R;
+    }
+    *i = kBand * lo + r;
+    *q = (full ? 0 : kBand / 2 * lo) + j;
+}
 long long tile_count(int T, int T2, int full) {
-    if (full) return (long long)T * T2;
-    const long long b = (T - 1) / kBand;
-    return kBand * (b * T2 - (kBand / 4) * b * (b - 1)) + (T - kBand * b) * (T2 - kBand / 2 * b);
+    const int b = (T - 1) / kBand, R = T - kBand * b, F = full ? 0 : R / 2;
+    return band_start(b, T2, full) + F * (F + 1) + (long long)(T2 - (full ? 0 : kBand / 2 * b) - F) * R;
 }
 
 // The kernel kind is a template parameter: with a runtime branch an element, the epilogue's
@@ -438,7 +443,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             bool ok = true, first = true;
             for (long long t = blockIdx.x; t < a.tiles && ok; t += G) {
                 int i, q;
-                if (!tile_coords(t, a.T, a.T2, a.full, &i, &q)) continue;
+                tile_coords(t, a.T, a.T2, a.full, &i, &q);
                 for (int kb = 0; kb < a.nkb; ++kb) {
                     if (!mbar_wait_for(empty_bar(stage), phase ^ 1u, abort_flag, a.err, a.wait_ns)) {
                         ok = false;
@@ -490,7 +495,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             for (long long t = blockIdx.x; t < a.tiles && ok; t += G) {
                 bool below = false;   // SPLIT: the tile holds a block below the diagonal
                 int i, q;
-                if (!tile_coords(t, a.T, a.T2, a.full, &i, &q)) continue;
+                tile_coords(t, a.T, a.T2, a.full, &i, &q);
                 if (SPLIT && a.full) below = 2 * q < i;
                 if (!SPLIT && !take_buffer(fill & 1, (uint32_t)(fill >> 1))) break;
                 for (int kb = 0; kb < a.nkb && ok; ++kb) {
@@ -573,7 +578,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         int fill = 0, ctr = 0;
         for (long long t = blockIdx.x; t < a.tiles; t += G) {
             int pair;
-            if (!tile_coords(t, a.T, a.T2, a.full, &b.rb, &pair)) continue;
+            tile_coords(t, a.T, a.T2, a.full, &b.rb, &pair);
             b.j = 2 * pair + h;           // 128-column block of K
             b.row = b.rb * BM + b.row_local;
             b.diag = b.rb == b.j;
