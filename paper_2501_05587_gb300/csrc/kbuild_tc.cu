@@ -27,7 +27,11 @@
 // before the operand ring's own writes): the images FP32 build 13.3 -> 11.8 ms.
 // Block (2q + 1, 2q), below the diagonal, is computed and not stored.
 //
-// Precision modes (operand matrix W, one row per point):
+// Precision modes (operand matrix W, one row per point; where there are two parts, 32 columns of hi and
+// the same 32 of lo follow one another, so that a stage's rows are 128 bytes in every mode.  With the
+// parts in two halves of W, read as 64-byte pieces by twice as many loads, BF16X3 took 23.8 ms at
+// n = 10,000, d = 100,000 where it takes 20.0, and 650 at n = 50,000 where 554; FP32 n = 20,001, d = 1,000
+// 1.37 and 1.33):
 //   BF16    W = bf16(P);  norms of the rounded rows, so the Gaussian distance
 //           r_i + r_j - 2 B_ij is the distance of the rounded points.
 //   BF16X3  W = [hi | lo] with hi = bf16(p), lo = bf16(p - hi); each stage
@@ -68,7 +72,7 @@
 //           Images, n = 70,000, d = 784: 10.9 ms (64.7 on CUDA cores); the operand loads allow
 //           8.4 (36 bytes a clock an SM), the MMAs 6.7, and the epilogue's stores (about 2 ms)
 //           are not overlapped: the next tile's MMAs run two chunks ahead.  n = 20,001,
-//           d = 1,000: 6.87 -> 1.43 ms a call.
+//           d = 1,000: 6.87 -> 1.33 ms a call.
 //           Measured on those points: 7.8e-8 (and 5.0e-8 at d = 128, where FMAs give 1.6e-7).
 //
 // Every mbarrier wait is bounded (about 2 s by %globaltimer).  A wait that
@@ -100,6 +104,7 @@ constexpr int BM = 128;                      // block rows / columns
 // depth of a k-block, in 16-bit elements: a stage is 48 KB in every mode (SPLIT: also what a TMEM
 // accumulator holds before it is drained)
 constexpr int kbuild_dk(int mode) { return mode == kModeBf16 ? 64 : 32; }
+constexpr int kRowElems = 64;                // a stage's row: 64 columns, or 32 of hi and the same 32 of lo: 128 bytes
 constexpr int STG_BYTES = 16 * 1024;         // staging of one epilogue warpgroup: a 128 x 32 FP32 chunk, a
                                              // 128 x 64 half box, or a 128 x 16 chunk and its transpose
 constexpr int NTHREADS = 320;                // 10 warps
@@ -114,7 +119,6 @@ constexpr uint32_t kTmemCols = 512;          // 2 buffers x 256 columns
 
 struct TcArgs {
     int n, T, T2, nkb;        // rows, 128-blocks, column pairs, k-blocks per part
-    int dpad;                 // elements per part (W row = [hi | lo] for BF16X3 and SPLIT)
     long long tiles;
     float* K;                 // row-major square (SPLIT: the diagonal blocks are stored with plain stores)
     int64_t ldk;
@@ -427,10 +431,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // stage layout: cols-hi (256 rows of W) | rows-hi (128 rows) [| cols-lo | rows-lo], rows of DK elements
+    // stage layout: columns (256 rows of W) | rows (128 rows), rows of kRowElems; lo 64 bytes behind hi
     constexpr int DK = kbuild_dk(MODE);
-    constexpr uint32_t kBlock = BM * DK * 2;   // 128 rows of one part
-    constexpr uint32_t kColsHi = 0, kRowsHi = 2 * kBlock, kColsLo = 3 * kBlock, kRowsLo = 5 * kBlock;
+    constexpr uint32_t kCols = 0, kRows = 2 * BM * kRowElems * 2, kLo = 64;
     const long long G = gridDim.x;
     if (warp == 0) {
         if (lane == 0) {
@@ -452,12 +455,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     if (!(a.stall && blockIdx.x == 0 && first)) {
                         const uint32_t st = sbase + (uint32_t)(stage * kStageBytes);
                         mbar_arrive_expect_tx(full_bar(stage), (uint32_t)kStageBytes);
-                        tma_load_2d(st + kColsHi, &map_c, kb * DK, q * 2 * BM, full_bar(stage));
-                        tma_load_2d(st + kRowsHi, &map_r, kb * DK, i * BM, full_bar(stage));
-                        if constexpr (X3) {
-                            tma_load_2d(st + kColsLo, &map_c, a.dpad + kb * DK, q * 2 * BM, full_bar(stage));
-                            tma_load_2d(st + kRowsLo, &map_r, a.dpad + kb * DK, i * BM, full_bar(stage));
-                        }
+                        tma_load_2d(st + kCols, &map_c, kb * kRowElems, q * 2 * BM, full_bar(stage));
+                        tma_load_2d(st + kRows, &map_r, kb * kRowElems, i * BM, full_bar(stage));
                         issued[stage] = true;
                         issued_parity[stage] = phase;
                     }
@@ -485,7 +484,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             uint32_t phase = 0;
             int fill = 0;   // accumulator fills: a tile, or (SPLIT) a 32-deep chunk
             bool ok = true;
-            const uint64_t desc0 = DK == 32 ? sw64_desc(sbase) : sw128_desc(sbase);
+            const uint64_t desc0 = sw128_desc(sbase);
             // both halves of the next buffer have been read by the epilogue
             auto take_buffer = [&](int ab, uint32_t use) {
                 if (!mbar_wait_for(acce_bar(ab), (use & 1u) ^ 1u, abort_flag, a.err, a.wait_ns)) return false;
@@ -515,8 +514,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                         }
                         ++fill;
                         const uint64_t sd = desc0 + (uint64_t)(uint32_t)(stage * (kStageBytes >> 4));
-                        const uint64_t rh = sd + (kRowsHi >> 4), rl = sd + (kRowsLo >> 4);
-                        const uint64_t ch = sd + (kColsHi >> 4), cl = sd + (kColsLo >> 4);
+                        const uint64_t rh = sd + (kRows >> 4), rl = rh + (kLo >> 4);
+                        const uint64_t ch = sd + (kCols >> 4), cl = ch + (kLo >> 4);
                         const uint32_t d_tmem = tmem + (uint32_t)(ab * 2 * BM);
                         // the small products first; hi.lo and lo.hi in the order of the
                         // transposed block below the diagonal (full schedule): K stays symmetric
@@ -533,8 +532,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                         mma_commit(accf_bar(ab));
                     } else {
                         const uint64_t sd = desc0 + (uint64_t)(uint32_t)(stage * (kStageBytes >> 4));
-                        const uint64_t rh = sd + (kRowsHi >> 4), rl = sd + (kRowsLo >> 4);
-                        const uint64_t ch = sd + (kColsHi >> 4), cl = sd + (kColsLo >> 4);
+                        const uint64_t rh = sd + (kRows >> 4), rl = rh + (kLo >> 4);
+                        const uint64_t ch = sd + (kCols >> 4), cl = ch + (kLo >> 4);
                         const uint32_t d_tmem = tmem + (uint32_t)((fill & 1) * 2 * BM);
 #pragma unroll
                         for (int kk = 0; kk < DK / 16; ++kk) {
@@ -688,8 +687,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
 }
 
-// FP32 rows -> BF16 operand rows W (BF16X3: [hi | lo]), zero padding, FP32 norms
-// of the represented rows.  One warp per row.
+// FP32 rows -> BF16 operand rows W (BF16X3: 32 columns of hi, then the same 32 of lo, and so on), zero
+// padding, FP32 norms of the represented rows.  One warp per row.
 __global__ void __launch_bounds__(256) prep_operands_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
                                                             int dpad, int x3, __nv_bfloat16* __restrict__ W,
                                                             float* __restrict__ norms) {
@@ -700,16 +699,17 @@ __global__ void __launch_bounds__(256) prep_operands_kernel(const float* __restr
     __nv_bfloat16* wr = W + (int64_t)warp * ldw;
     float nrm = 0.f;
     for (int l = lane; l < dpad; l += 32) {
+        const int at = x3 ? 2 * (l & ~31) + (l & 31) : l;
         const float p = l < d ? P[(int64_t)warp * ldp + l] : 0.f;
         const __nv_bfloat16 hi = __float2bfloat16_rn(p);
         const float hf = __bfloat162float(hi);
-        wr[l] = hi;
+        wr[at] = hi;
         if (!x3) {
             nrm = fmaf(hf, hf, nrm);
         } else {
             const __nv_bfloat16 lo = __float2bfloat16_rn(p - hf);
             const float rep = hf + __bfloat162float(lo);
-            wr[dpad + l] = lo;
+            wr[at + 32] = lo;
             nrm = fmaf(rep, rep, nrm);
         }
     }
@@ -867,8 +867,8 @@ __global__ void __launch_bounds__(256) split_scan_kernel(const float* __restrict
     split_decide(colmax, rowmax, nonzero, n, d, maxr, expand_coef, st);
 }
 
-// FP32 rows -> W = [hi | lo] in FP16, zero padding.  A thread takes four columns of a row
-// (float4 loads when rows are 16-byte aligned), 8-byte stores.
+// FP32 rows -> W in FP16, hi and lo by 32 columns as above, zero padding.  A thread takes four columns of
+// a row (float4 loads when rows are 16-byte aligned), 8-byte stores.
 __global__ void __launch_bounds__(256) split_operands_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
                                                              int dpad, SplitState* st, __half* __restrict__ W) {
     if (!st->use) return;
@@ -898,9 +898,9 @@ __global__ void __launch_bounds__(256) split_operands_kernel(const float* __rest
             const float2 h = __half22float2(hi[x]);
             lo[x] = __floats2half2_rn(f0 - h.x, f1 - h.y);
         }
-        __half* w = W + r * (2 * (int64_t)dpad) + l;
+        __half* w = W + r * (2 * (int64_t)dpad) + 2 * (l & ~31) + (l & 31);
         *reinterpret_cast<uint2*>(w) = *reinterpret_cast<const uint2*>(hi);
-        *reinterpret_cast<uint2*>(w + dpad) = *reinterpret_cast<const uint2*>(lo);
+        *reinterpret_cast<uint2*>(w + 32) = *reinterpret_cast<const uint2*>(lo);
     }
     low = __reduce_add_sync(0xffffffffu, low);
     if ((threadIdx.x & 31) == 0 && low) atomicAdd(&st->low, (unsigned long long)low);
@@ -994,10 +994,9 @@ cudaError_t launch_tiles(int mode, const void* W, int n, int64_t ldw, int dpad, 
     memset(&mkt, 0, sizeof mkt);
     const CUtensorMapDataType dt = split ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     void* w = const_cast<void*>(W);
-    const int dk = kbuild_dk(mode);
-    const CUtensorMapSwizzle sw = dk == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;   // rows of dk elements
-    if (!make_tensor_map_2d(&mr, dt, w, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, dk, BM, sw) ||
-        !make_tensor_map_2d(&mc, dt, w, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, dk, 2 * BM, sw))
+    const CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B;
+    if (!make_tensor_map_2d(&mr, dt, w, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, kRowElems, BM, sw) ||
+        !make_tensor_map_2d(&mc, dt, w, (uint64_t)ldw, (uint64_t)n, (uint64_t)ldw * 2, kRowElems, 2 * BM, sw))
         return cudaErrorInvalidValue;
     // the full-square stores go through tensor maps; the packed stores are plain bulk copies
     if (out == kOutFull && (!make_tensor_map_2d(&mkd, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, K, (uint64_t)n, (uint64_t)n,
@@ -1009,8 +1008,7 @@ cudaError_t launch_tiles(int mode, const void* W, int n, int64_t ldw, int dpad, 
     a.n = n;
     a.T = (n + BM - 1) / BM;
     a.T2 = (a.T + 1) / 2;
-    a.dpad = dpad;
-    a.nkb = dpad / dk;
+    a.nkb = dpad / kbuild_dk(mode);
     a.full = full;
     a.tiles = tile_count(a.T, a.T2, a.full);
     a.K = K;

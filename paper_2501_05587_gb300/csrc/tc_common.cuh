@@ -228,18 +228,6 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
     return d;
 }
 
-// The same for the 64-byte swizzle: rows of 64 bytes, 8-row core groups 512 bytes apart; swizzle
-// mode 4.
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;
-    return d;
-}
-
 // Instruction descriptor (kind::f16 and kind::f8f6f4): D format at bits 4-5
 // (1 = F32), A format at bits 7-9, B format at bits 10-12 (kind::f16: 1 =
 // BF16; kind::f8f6f4: 0 = E4M3), both operands K-major (bits 15, 16 = 0),
