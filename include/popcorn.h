@@ -407,7 +407,8 @@ POPCORN_API popcorn_status popcorn_kmeanspp(const float* P, int64_t n, int32_t d
  * doing work on the device while the others go on.  Instances of uneven n,
  * d, k and kernel share every launch: work is flattened over (instance,
  * tile / row block).  K is stored as the packed upper triangle and read by
- * block rows; options.k_storage FP16 / BF16 stores it as 32 KB half tiles, which
+ * block rows (an FP32 K of a batch with fewer than about 600 blocks of 128 rows
+ * as squares, row by row); options.k_storage FP16 / BF16 stores it as 32 KB half tiles, which
  * each pass reads on the tensor cores: per 128-row block, MMAs of its tiles
  * (those below the diagonal transposed) against one-hot label operands, the row
  * sums in TMEM.  k_pass and sym_tile do not apply here.

@@ -55,6 +55,7 @@ struct DeviceInfo {
     int smem_optin = 0;
     int reduce_smem = 0;   // dynamic shared memory usable by the reduction kernel
     int recompute_smem = 0;
+    int batched_smem = 0;
     bool coop = false;   // cooperative launches (all CTAs of a grid resident at once)
     cudaMemPool_t pool = nullptr;
     bool ready = false;
@@ -85,6 +86,7 @@ popcorn_status device_info(DeviceInfo** out) {
         POPCORN_CUDA(configure_reduce_smem(d.smem_optin, &d.reduce_smem));
         POPCORN_CUDA(configure_kbuild_tc());
         POPCORN_CUDA(configure_recompute(d.smem_optin, &d.recompute_smem));
+        POPCORN_CUDA(configure_batched(d.smem_optin));
         POPCORN_CUDA(configure_batched_mma(d.smem_optin));
         POPCORN_CUDA(configure_reduce_tiles(d.smem_optin));
         POPCORN_CUDA(configure_reduce_sym(d.smem_optin));
@@ -95,6 +97,7 @@ popcorn_status device_info(DeviceInfo** out) {
         int coop = 0;
         POPCORN_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         d.coop = coop != 0;
+        d.batched_smem = d.smem_optin - 1024;
         d.ready = true;
     }
     *out = &d;
@@ -1301,8 +1304,32 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     // K-stream unit lengths the autotuner may pick (Spart is sized for the shortest)
     static const int kSegCand[] = {2048, 4096, 8192, 16384};
     const int min_seglen = opt.autotune ? kSegCand[0] : kBatchSeg;
-    // FP32 K: column blocks a unit (and a sum) takes
-    auto set_segments = [](BatchInst* b, int seglen) {
+    // FP32 K by block rows, or row by row where there are fewer 128-row blocks than the block rows' stream
+    // has CTAs (or 4 an SM: with few clusters 5 fit, but 600 blocks are enough).  Whole calls of 20 passes,
+    // by block rows and row by row: one instance of n = 2,000 1,877 and 900 us, 8 of n = 300 to 600 1,256 and
+    // 882, 8 of 4,000 to 7,000 (344 blocks for 456 CTAs) 6,252 and 5,636; 256 of 128 to 400 (about 640 for 760)
+    // 4,904 and 5,532, 64 of 1,000 to 4,000 (1,250 for 456) 9,466 and 12,206.
+    bool rows = false;
+    if (!half) {
+        long long blocks = 0;
+        BatchPlan probe{};
+        for (int t = 0; t < count; ++t) {   // (what is not valid is reported below)
+            blocks += inst[t].n > 0 ? (inst[t].n + 127) / 128 : 0;
+            probe.kmax = std::max(probe.kmax, std::min(std::max(inst[t].k, 1), kMaxClusters));
+        }
+        rows = blocks < dev->sms;   // (a CTA an SM at least: no need to ask what fits)
+        if (!rows && !plan_batched_tiles(&probe, dev->sms))
+            return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
+        rows = rows || blocks < std::min(probe.grid, 4 * dev->sms);
+    }
+    bp.rows = rows ? 1 : 0;
+    // FP32 K: columns a unit (and a sum) takes
+    auto set_segments = [rows](BatchInst* b, int seglen) {
+        if (rows) {
+            b->seglen = seglen;
+            b->nseg = (b->n + seglen - 1) / seglen;
+            return;
+        }
         const int blocks = std::min(seglen / 128, b->T);
         b->seglen = 128 * blocks;
         b->nseg = (b->T + blocks - 1) / blocks;
@@ -1329,6 +1356,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.T = (n + 127) / 128;
         b.tile0 = bp.tiles;
         bp.tiles += (long long)b.T * (b.T + 1) / 2;
+        b.ldk = (n + 3) / 4 * 4;
         b.n = n;
         b.k = k;
         if (half) {   // S written once a row
@@ -1339,7 +1367,8 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         }
         b.init_labels = x.init_labels;
         b.labels_out = x.labels_out;
-        bp.units += b.T * b.nseg;
+        b.unit0 = bp.units;
+        bp.units += (rows ? n : b.T) * b.nseg;
         b.zblock0 = bp.zblocks;
         bp.zblocks += (n + kZReduceRows - 1) / kZReduceRows;
         b.ablock0 = bp.ablocks;
@@ -1348,9 +1377,9 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         bp.lblocks += (n + kBatchLabelThreads - 1) / kBatchLabelThreads;
         if (k > bp.kmax) bp.kmax = k;
         const int zb = (n + kZReduceRows - 1) / kZReduceRows;
-        // the packed triangle the K stream reads, FP32 or half tiles
+        // the packed triangle the K stream reads, FP32 or half tiles, or the square by rows
         const size_t tiles = (size_t)b.T * (b.T + 1) / 2;
-        o[t].K = !half ? take(tiles * 65536) : 0;
+        o[t].K = half ? 0 : rows ? take((size_t)n * b.ldk * 4) : take(tiles * 65536);
         if (half) {
             b.N = (k + 15) / 16 * 16;
             bp.nunits += b.T;
@@ -1359,13 +1388,13 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         }
         b.vblock0 = bp.vblocks;
         bp.vblocks += b.T;
-        o_v[t] = take(half ? (size_t)b.T * b.N * 256 : tiles_record_bytes(n));
+        o_v[t] = rows ? 0 : take(half ? (size_t)b.T * b.N * 256 : tiles_record_bytes(n));
         o[t].kdiag = take((size_t)n * 4);
         o[t].lab32 = take((size_t)n * 4);
         o[t].lab8 = take(((size_t)n + 15) & ~(size_t)15);
         o[t].counts = take(2 * (size_t)k * 4);
         o[t].Spart = take((size_t)n * b.nseg * k * 4);
-        o[t].Srun = half ? 0 : take((size_t)n * b.nseg * k * 8);
+        o[t].Srun = half || rows ? 0 : take((size_t)n * b.nseg * k * 8);
         o[t].zpart = take((size_t)zb * k * 8);
         o[t].zsum = take((size_t)k * 8);
         o[t].cnorm = take((size_t)k * 8);
@@ -1389,10 +1418,13 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h[x].T > h[y].T; });
     auto list_units = [&]() {
         hunits.clear();
+        if (rows) return;   // (the kernel finds a row's instance by itself)
         for (int t : order)
             for (int r = 0; r < h[t].T * (half ? 1 : h[t].nseg); ++r) hunits.push_back(make_int2(t, r));
     };
-    if (half ? !plan_batched_mma(&bp, dev->sms, dev->smem_optin) : !plan_batched_tiles(&bp, dev->sms))
+    if (rows)
+        plan_batched_reduce(&bp, dev->sms, dev->batched_smem);
+    else if (half ? !plan_batched_mma(&bp, dev->sms, dev->smem_optin) : !plan_batched_tiles(&bp, dev->sms))
         return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
     list_units();
     const size_t units_off = take(sizeof(int2) * hunits.size());   // (the most units of any schedule)
@@ -1411,7 +1443,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.lab8 = base + o[t].lab8;
         b.counts = reinterpret_cast<int32_t*>(base + o[t].counts);
         b.Spart = reinterpret_cast<float*>(base + o[t].Spart);
-        b.Srun = half ? nullptr : reinterpret_cast<float2*>(base + o[t].Srun);
+        b.Srun = half || rows ? nullptr : reinterpret_cast<float2*>(base + o[t].Srun);
         b.zpart = reinterpret_cast<double*>(base + o[t].zpart);
         b.zsum = reinterpret_cast<double*>(base + o[t].zsum);
         b.cnorm = reinterpret_cast<double*>(base + o[t].cnorm);
@@ -1420,7 +1452,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         b.J_hist = reinterpret_cast<double*>(base + o[t].J);
         b.changed_hist = reinterpret_cast<int32_t*>(base + o[t].ch);
         if (half) b.Kh = base + o_kh[t];
-        b.V = base + o_v[t];
+        b.V = rows ? nullptr : base + o_v[t];
     }
     const int2* dunits = reinterpret_cast<const int2*>(base + units_off);
     auto upload_units = [&]() {
@@ -1440,7 +1472,8 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         bp.units = 0;
         for (int t = 0; t < count; ++t) {
             set_segments(&h[t], seglen);
-            bp.units += h[t].T * h[t].nseg;
+            h[t].unit0 = bp.units;
+            bp.units += (rows ? h[t].n : h[t].T) * h[t].nseg;
         }
         list_units();
     };
@@ -1453,8 +1486,7 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
             sum_n2 += (double)h[t].n * h[t].n;
             max_n = h[t].n > max_n ? h[t].n : max_n;
         }
-        // (4: the block-row stream; files may hold schedules of the row-by-row stream under 1)
-        const TuneKey key{4, opt.precision, count, bp.kmax, log2_bucket(sum_n2), log2_bucket(max_n),
+        const TuneKey key{rows ? 1 : 4, opt.precision, count, bp.kmax, log2_bucket(sum_n2), log2_bucket(max_n),
                           opt.k_storage, dev->sms};
         TuneValue best{};
         if (tune_lookup(key, &best)) {
@@ -1469,46 +1501,56 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
             } else {
                 for (int t = 0; t < count; ++t)
                     POPCORN_CUDA(launch_kbuild_tc(h[t].P, h[t].n, h[t].d, h[t].ldp, h[t].kp, opt.precision, h[t].K,
-                                                  0, h[t].kdiag, base + tc_off, err, dev->sms, s, nullptr,
-                                                  kPackedSw4));
+                                                  rows ? h[t].ldk : 0, h[t].kdiag, base + tc_off, err, dev->sms, s, nullptr,
+                                                  rows ? 0 : kPackedSw4));
             }
             cudaEvent_t t0, t1;
             g_events.used = 0;
             POPCORN_TRY(g_events.get(&t0));
             POPCORN_TRY(g_events.get(&t1));
             best.ms = 3.0e38f;
+            const std::vector<int> warp_cand = rows ? std::vector<int>{4, 8, 16} : std::vector<int>{4};
+            auto stream = [&](const BatchPlan& p) {
+                return rows ? launch_batched_reduce(dI, p, 0, s) : launch_batched_tiles(dI, dunits, p, err, 0, s);
+            };
             for (int seglen : kSegCand)
-                for (int ps : {1, 2}) {
-                    BatchPlan cand = bp;
-                    set_seglen(seglen);
-                    cand.units = bp.units;
-                    if (!plan_batched_tiles(&cand, dev->sms, ps == 2 ? 0 : ps) || cand.per_sm < ps) continue;   // does not fit
-                    POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count,
-                                                 cudaMemcpyHostToDevice, s));
-                    POPCORN_CUDA(upload_units());
-                    POPCORN_CUDA(launch_batched_tiles(dI, dunits, cand, err, 0, s));   // warm-up
-                    float ms = 3.0e38f;
-                    for (int rep = 0; rep < 2; ++rep) {
-                        POPCORN_CUDA(cudaEventRecord(t0, s));
-                        POPCORN_CUDA(launch_batched_tiles(dI, dunits, cand, err, 0, s));
-                        POPCORN_CUDA(cudaEventRecord(t1, s));
-                        POPCORN_CUDA(cudaEventSynchronize(t1));
-                        float e = 0.f;
-                        POPCORN_CUDA(cudaEventElapsedTime(&e, t0, t1));
-                        ms = e < ms ? e : ms;
+                for (int w : warp_cand)
+                    for (int ps : {1, 2}) {
+                        BatchPlan cand = bp;
+                        set_seglen(seglen);
+                        cand.units = bp.units;
+                        if (rows) {
+                            plan_batched_reduce(&cand, dev->sms, dev->batched_smem, w, ps);
+                            if (cand.warps != w || cand.per_sm != ps) continue;   // does not fit
+                        } else if (!plan_batched_tiles(&cand, dev->sms, ps == 2 ? 0 : ps) || cand.per_sm < ps) {
+                            continue;
+                        }
+                        POPCORN_CUDA(cudaMemcpyAsync(dI, h.data(), sizeof(BatchInst) * (size_t)count,
+                                                     cudaMemcpyHostToDevice, s));
+                        if (!rows) POPCORN_CUDA(upload_units());
+                        POPCORN_CUDA(stream(cand));   // warm-up
+                        float ms = 3.0e38f;
+                        for (int rep = 0; rep < 2; ++rep) {
+                            POPCORN_CUDA(cudaEventRecord(t0, s));
+                            POPCORN_CUDA(stream(cand));
+                            POPCORN_CUDA(cudaEventRecord(t1, s));
+                            POPCORN_CUDA(cudaEventSynchronize(t1));
+                            float e = 0.f;
+                            POPCORN_CUDA(cudaEventElapsedTime(&e, t0, t1));
+                            ms = e < ms ? e : ms;
+                        }
+                        // the argmin and the z reduction read every segment's slot, at about 1 TB/s (shorter
+                        // units alone stream up to a tenth faster, and lost more than that there)
+                        for (int t = 0; t < count; ++t) ms += (float)(4.0 * h[t].nseg * h[t].k * h[t].n / 1e9);
+                        ++tune_cands;
+                        if (ms < best.ms) {
+                            best.ms = ms;
+                            best.p[0] = seglen;
+                            best.p[1] = cand.warps;
+                            best.p[2] = ps;
+                            best.p[3] = 0;
+                        }
                     }
-                    // the argmin and the z reduction read every segment's slot, at about 1 TB/s (shorter
-                    // units alone stream up to a tenth faster, and lost more than that there)
-                    for (int t = 0; t < count; ++t) ms += (float)(4.0 * h[t].nseg * h[t].k * h[t].n / 1e9);
-                    ++tune_cands;
-                    if (ms < best.ms) {
-                        best.ms = ms;
-                        best.p[0] = seglen;
-                        best.p[1] = cand.warps;
-                        best.p[2] = ps;
-                        best.p[3] = 0;
-                    }
-                }
             int herr = 0;
             POPCORN_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
             POPCORN_CUDA(cudaStreamSynchronize(s));
@@ -1523,10 +1565,14 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
     }
     if (!half) {
         set_seglen(sched[0]);
-        POPCORN_CUDA(upload_units());
         const bool tuned = sched[2] != 0;
-        if (!plan_batched_tiles(&bp, dev->sms, sched[2] == 1 ? 1 : 0))
-            return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
+        if (rows) {
+            plan_batched_reduce(&bp, dev->sms, dev->batched_smem, sched[1], sched[2]);
+        } else {
+            POPCORN_CUDA(upload_units());
+            if (!plan_batched_tiles(&bp, dev->sms, sched[2] == 1 ? 1 : 0))
+                return fail(POPCORN_ERR_UNSUPPORTED, "the batched K stream does not fit this device");
+        }
         sched[1] = bp.warps;
         sched[2] = tuned ? std::min(bp.per_sm, 2) : bp.per_sm;
     } else {
@@ -1562,8 +1608,8 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         for (int t = 0; t < count && cap == POPCORN_OK; ++t) {
             const BatchInst& b = h[t];
             step(launch_kbuild_tc(b.P, b.n, b.d, b.ldp, b.kp, opt.precision,
-                                  half ? reinterpret_cast<float*>(b.Kh) : b.K, 0, b.kdiag, base + tc_off, err,
-                                  dev->sms, cs, &launches, half ? kPackedSw128H : kPackedSw4, 0, half),
+                                  half ? reinterpret_cast<float*>(b.Kh) : b.K, rows ? b.ldk : 0, b.kdiag, base + tc_off, err,
+                                  dev->sms, cs, &launches, half ? kPackedSw128H : rows ? 0 : kPackedSw4, 0, half),
                  "tensor-core K build");
         }
     }
@@ -1579,18 +1625,19 @@ popcorn_status popcorn_fit_batched(int32_t count, const popcorn_instance* inst, 
         if (stall_ms < 0 || stall_ms > 10000) stall_ms = 0;
     }
     auto pass = [&](int eval) -> cudaError_t {
-        const cudaError_t e = half ? launch_batched_mma_stream(dI, dunits, bp, err, eval, cs, stall_ms)
-                                   : launch_batched_tiles(dI, dunits, bp, err, eval, cs, stall_ms);
+        const cudaError_t e = half   ? launch_batched_mma_stream(dI, dunits, bp, err, eval, cs, stall_ms)
+                              : rows ? launch_batched_reduce(dI, bp, eval, cs)
+                                     : launch_batched_tiles(dI, dunits, bp, err, eval, cs, stall_ms);
         stall_ms = 0;
         return e != cudaSuccess ? e : launch_batched_finish(dI, bp, eval, cs);
     };
     for (int it = 0; it < max_iter && cap == POPCORN_OK; ++it) {
         step(pass(0), "batched pass");
-        launches += 4;
+        launches += rows ? 3 : 4;
     }
     step(pass(1), "batched objective pass");
     step(launch_batched_copy_labels(dI, bp, cs), "batched label copy");
-    launches += 4;
+    launches += rows ? 3 : 4;
     cudaGraph_t graph = nullptr;
     cudaError_t ec = cudaStreamEndCapture(cs, &graph);
     if (cap != POPCORN_OK) {

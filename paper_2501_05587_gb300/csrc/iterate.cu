@@ -969,7 +969,164 @@ __global__ void __launch_bounds__(kAssignThreads) batched_assign_kernel(const Ba
     assign_body(a, blockIdx.x - b.ablock0, (b.n + kAssignThreads - 1) / kAssignThreads);
 }
 
+// FP32 K row by row (BatchPlan.rows: batches with fewer 128-row blocks than reduce_tiles.cu has CTAs for,
+// which would leave SMs idle): K stream over the units (instance, row, segment) of every instance still
+// running: lane-private shared-memory cluster columns as in reduce_kernel,
+// labels read through L1, the next batch in flight while the current one is
+// scattered (across unit boundaries too), and per unit a butterfly reduction
+// for k <= 8 or the rotated walk for larger k.  z and J come from the batched
+// z kernel that follows.
+// U float4 a lane a batch: 4 with two blocks an SM (64 registers); 8 with one block an SM,
+// which keeps twice the bytes in flight where the per-warp cluster columns (kmax x 128 bytes)
+// leave room for only 16 warps an SM.
+template <int U>
+__global__ void __launch_bounds__(kReduceMaxWarps * 32, U == 4 ? 2 : 1)
+    batched_reduce_kernel(const BatchInst* I, int count, int units, int kmax, int eval) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int W = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* accw = reinterpret_cast<float*>(smem) + (size_t)warp * kmax * 32;
+    float* accl = accw + lane;
+    for (int t = lane; t < kmax * 32; t += 32) accw[t] = 0.f;
+    __syncwarp();
+    const int GW = (int)gridDim.x * W;
+
+    // next unit at or after u that belongs to an instance still running
+    struct Geo {
+        const BatchInst* b;
+        int u, i, sg, c1, qb, q1;
+        const float4* row4;
+        const uint32_t* lab4;
+    };
+    auto geom = [&](int u, Geo& g) -> bool {
+        for (; u < units; u += GW) {
+            const int t = find_inst(I, count, u, [](const BatchInst& x) { return (long long)x.unit0; });
+            const BatchInst* b = I + t;
+            if (pass_skip(b->st, eval)) continue;
+            const int lu = u - b->unit0;
+            g.b = b;
+            g.u = u;
+            g.i = lu / b->nseg;
+            g.sg = lu - g.i * b->nseg;
+            const int c0 = g.sg * b->seglen;
+            g.c1 = min(b->n, c0 + b->seglen);
+            g.qb = c0 >> 2;
+            g.q1 = g.c1 >> 2;
+            g.row4 = reinterpret_cast<const float4*>(b->K + (int64_t)g.i * b->ldk);
+            g.lab4 = reinterpret_cast<const uint32_t*>(b->lab8);
+            return true;
+        }
+        return false;
+    };
+    Geo cur;
+    if (!geom((int)blockIdx.x * W + warp, cur)) return;
+    float4 v[U];
+    uint32_t L[U];
+    load_batch<U, false>(cur.row4, cur.lab4, cur.qb + lane, cur.q1, v, L);
+    while (true) {
+        const bool last = cur.qb + 32 * U >= cur.q1;
+        Geo nxt = cur;
+        bool more = true;
+        if (last) {
+            more = geom(cur.u + GW, nxt);
+        } else {
+            nxt.qb = cur.qb + 32 * U;
+        }
+        float4 vn[U];
+        uint32_t Ln[U];
+        if (more) load_batch<U, false>(nxt.row4, nxt.lab4, nxt.qb + lane, nxt.q1, vn, Ln);
+#pragma unroll
+        for (int x = 0; x < U; ++x) {
+            accl[(L[x] & 0xffu) * 32] += v[x].x;
+            accl[((L[x] >> 8) & 0xffu) * 32] += v[x].y;
+            accl[((L[x] >> 16) & 0xffu) * 32] += v[x].z;
+            accl[(L[x] >> 24) * 32] += v[x].w;
+        }
+        if (last) {
+            const BatchInst& b = *cur.b;
+            {
+                const int j = (cur.q1 << 2) + lane;
+                if (j < cur.c1) accl[(int)b.lab8[j] * 32] += b.K[(int64_t)cur.i * b.ldk + j];
+            }
+            __syncwarp();
+            float* out = b.Spart + (size_t)cur.sg * b.k * b.n + cur.i;   // [s][c][i]
+            if (b.k <= 8) {
+                float part[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    part[c] = c < b.k ? accl[c * 32] : 0.f;
+                    if (c < b.k) accl[c * 32] = 0.f;
+                }
+                const float tot = butterfly<8>(part, lane);
+                const int c = bfly_cluster<8>(lane);
+                if ((lane & 3) == 0 && c < b.k) out[(size_t)c * b.n] = tot;
+            } else {
+                for (int cb = 0; cb < b.k; cb += 32) {
+                    const int c = cb + lane;
+                    if (c < b.k) {
+                        float tot = 0.f;
+                        float* rowp = accw + (size_t)c * 32;
+#pragma unroll 8
+                        for (int j = 0; j < 32; ++j) {
+                            const int idx = (j + lane) & 31;
+                            tot += rowp[idx];
+                            rowp[idx] = 0.f;
+                        }
+                        out[(size_t)c * b.n] = tot;
+                    }
+                }
+            }
+            __syncwarp();
+            if (!more) break;
+            cur = nxt;
+        } else {
+            cur.qb = nxt.qb;
+        }
+#pragma unroll
+        for (int x = 0; x < U; ++x) {
+            v[x] = vn[x];
+            L[x] = Ln[x];
+        }
+    }
+}
+
 }  // namespace
+
+void plan_batched_reduce(BatchPlan* bp, int num_sms, int smem_budget, int warps, int per_sm_req) {
+    const size_t per_warp = (size_t)bp->kmax * 32 * sizeof(float);
+    int w = (int)((size_t)smem_budget / per_warp);
+    if (w > kReduceMaxWarps) w = kReduceMaxWarps;
+    if (warps > 0 && warps < w) w = warps;
+    if (w < 1) w = 1;
+    bp->warps = w;
+    bp->smem = per_warp * w;
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_reduce_kernel<4>, 32 * w, bp->smem);
+    cudaGetLastError();
+    if (per_sm_req > 0 && per_sm_req < per_sm) per_sm = per_sm_req;
+    if (per_sm < 1) per_sm = 1;
+    bp->per_sm = per_sm;
+    bp->grid = num_sms * per_sm;
+}
+
+cudaError_t launch_batched_reduce(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s) {
+    if (bp.per_sm == 1)
+        batched_reduce_kernel<8><<<bp.grid, bp.warps * 32, bp.smem, s>>>(dI, bp.count, bp.units, bp.kmax, eval);
+    else
+        batched_reduce_kernel<4><<<bp.grid, bp.warps * 32, bp.smem, s>>>(dI, bp.count, bp.units, bp.kmax, eval);
+    return cudaGetLastError();
+}
+
+cudaError_t configure_batched(int smem_optin) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, batched_reduce_kernel<4>);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(batched_reduce_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             optin_minus_static(smem_optin, fa.sharedSizeBytes));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(batched_reduce_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                optin_minus_static(smem_optin, fa.sharedSizeBytes));
+}
 
 cudaError_t launch_batched_init(const BatchInst* dI, const BatchPlan& bp, int max_iter, int check_conv, double tol,
                                 cudaStream_t s) {

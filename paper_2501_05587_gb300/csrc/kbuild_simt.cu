@@ -553,9 +553,9 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
 
 // All instances of a batch: flattened tile b belongs to the instance whose
 // tile0 is the largest one <= b.
-// TK float: each instance's FP32 block-packed triangle (K, kPackedSw4); TK __half / __nv_bfloat16:
+// TK float: each instance's FP32 block-packed triangle (K, PK = kPackedSw4) or its row-major square (0); TK __half / __nv_bfloat16:
 // its triangle of half tiles (Kh, kPackedSw128H), for the tensor-core batched stream.
-template <typename TK>
+template <typename TK, int PK>
 __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst* I, int count) {
     const long long b = blockIdx.x;
     int lo = 0, hi = count - 1;
@@ -567,17 +567,16 @@ __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst*
     const BatchInst& x = I[lo];
     const long long t = b - x.tile0;
     __shared__ __align__(16) TileSmem sm;   // one copy for the three kernel functions
-    constexpr int PK = sizeof(TK) == 2 ? kPackedSw128H : kPackedSw4;
     TK* K = sizeof(TK) == 2 ? reinterpret_cast<TK*>(x.Kh) : reinterpret_cast<TK*>(x.K);
     switch (x.kp.kind) {
         case POPCORN_LINEAR:
-            kbuild_tile<POPCORN_LINEAR, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, 0, x.kdiag, x.T, t, sm);
+            kbuild_tile<POPCORN_LINEAR, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, x.ldk, x.kdiag, x.T, t, sm);
             break;
         case POPCORN_POLYNOMIAL:
-            kbuild_tile<POPCORN_POLYNOMIAL, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, 0, x.kdiag, x.T, t, sm);
+            kbuild_tile<POPCORN_POLYNOMIAL, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, x.ldk, x.kdiag, x.T, t, sm);
             break;
         default:
-            kbuild_tile<POPCORN_GAUSSIAN, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, 0, x.kdiag, x.T, t, sm);
+            kbuild_tile<POPCORN_GAUSSIAN, TK, false, PK>(x.P, x.n, x.d, x.ldp, x.kp, K, x.ldk, x.kdiag, x.T, t, sm);
             break;
     }
 }
@@ -587,11 +586,13 @@ __global__ void __launch_bounds__(256, 2) batched_kbuild_kernel(const BatchInst*
 cudaError_t launch_batched_kbuild_simt(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s) {
     if (bp.tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     if (bp.half == POPCORN_K_FP16)
-        batched_kbuild_kernel<__half><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
+        batched_kbuild_kernel<__half, kPackedSw128H><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
     else if (bp.half == POPCORN_K_BF16)
-        batched_kbuild_kernel<__nv_bfloat16><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
+        batched_kbuild_kernel<__nv_bfloat16, kPackedSw128H><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
+    else if (bp.rows)
+        batched_kbuild_kernel<float, 0><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
     else
-        batched_kbuild_kernel<float><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
+        batched_kbuild_kernel<float, kPackedSw4><<<(unsigned)bp.tiles, 256, 0, s>>>(dI, bp.count);
     return cudaGetLastError();
 }
 

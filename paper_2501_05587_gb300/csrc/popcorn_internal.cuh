@@ -407,7 +407,8 @@ struct BatchInst {
     KernParams kp;
     int T;                    // 128-row tiles of K
     long long tile0;          // first flattened upper-triangle tile
-    float* K;                 // FP32 K: the packed triangle
+    float* K;                 // FP32 K: the packed triangle, or row-major with pitch ldk (BatchPlan.rows)
+    int64_t ldk;
     float* kdiag;
     int n, k, nseg, seglen;
     uint8_t* lab8;
@@ -424,7 +425,7 @@ struct BatchInst {
     int32_t* changed_hist;
     const int32_t* init_labels;
     int32_t* labels_out;
-    int zblock0, ablock0, lblock0;
+    int unit0, zblock0, ablock0, lblock0;
     // FP16 / BF16 K (batched_mma.cu): the packed triangle in kPackedSw128H; the per-pass one-hot
     // operands of the T blocks, N rows each
     unsigned char* Kh;
@@ -438,6 +439,7 @@ struct BatchPlan {
     long long tiles;          // K tiles of all instances
     int units, zblocks, ablocks, lblocks;
     int kmax;
+    int rows;                 // 1: FP32 K row by row (iterate.cu), units (instance, row, segment)
     int warps, grid, per_sm;  // batched K-stream launch (FP32 K)
     size_t smem;
     // FP16 / BF16 K: the tensor-core stream over (instance, row block) units
@@ -465,6 +467,11 @@ bool plan_batched_tiles(BatchPlan* bp, int num_sms, int per_sm_req = 0);
 // stall_ms as launch_reduce_sym.
 cudaError_t launch_batched_tiles(const BatchInst* dI, const int2* units, const BatchPlan& bp, int* err, int eval,
                                  cudaStream_t s, int stall_ms = 0);
+// FP32 K row by row: warps / grid / shared memory for clusters up to kmax (0: the most warps that fit,
+// the occupancy's blocks an SM), and the K stream of a pass.
+void plan_batched_reduce(BatchPlan* bp, int num_sms, int smem_budget, int warps = 0, int per_sm = 0);
+cudaError_t configure_batched(int smem_optin);
+cudaError_t launch_batched_reduce(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
 // the rest of a pass after its K stream: z (with per-instance finalization) and the argmin
 cudaError_t launch_batched_finish(const BatchInst* dI, const BatchPlan& bp, int eval, cudaStream_t s);
 cudaError_t launch_batched_copy_labels(const BatchInst* dI, const BatchPlan& bp, cudaStream_t s);
@@ -481,7 +488,8 @@ cudaError_t launch_batched_mma_stream(const BatchInst* dI, const int2* units, co
 
 // ---- autotune cache (autotune.cu) ---------------------------------------------
 struct TuneKey {
-    int32_t target;       // 2: recompute pass, 3: K-build schedule, 4: batched K stream
+    int32_t target;       // 1: batched K stream by rows, 2: recompute pass, 3: K-build schedule, 4: batched K
+                          // stream by block rows
     int32_t precision;
     int32_t a, b, c, d, e;   // target-specific size buckets
     int32_t sms;

@@ -45,7 +45,8 @@ def test_block_row_stream(pc, monkeypatch, check):
 
 
 def test_batched_block_row_stream(pc, monkeypatch):
-    wls = synth.batched_instances(6, seed=5, n_lo=300, n_hi=1500)
+    # (1,000 blocks of 128 rows and more: batches of few are read row by row)
+    wls = synth.batched_instances(160, seed=5, n_lo=600, n_hi=1500)
     inst = [{"P": torch.from_numpy(w.P).cuda(), "k": w.k, "kernel": w.kernel,
              "init_labels": torch.from_numpy(w.init_labels).cuda()} for w in wls]
     call = lambda: pc.popcorn_fit_batched(inst, max_iter=4, check_convergence=False)  # noqa: E731

@@ -104,6 +104,7 @@ def test_batched_sums_of_large_clusters(order):
         P, lab = _points(n, g), _labels(order, n, k, g)
         inst.append({"P": P, "init_labels": lab, "k": k, "kernel": LINEAR})
         want.append(_exact(P, lab, k)[1])
+    inst, want = inst * 4, want * 4      # (blocks for every CTA: batches of few are read row by row)
     r = pc.popcorn_fit_batched(inst, max_iter=0, check_convergence=False)
     for x, got, J in zip(inst, r["objectives"], want):
         assert abs(got - J) <= 1e-6 * J, (x["P"].shape, x["k"])
