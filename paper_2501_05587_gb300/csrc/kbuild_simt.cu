@@ -411,6 +411,7 @@ __global__ void __launch_bounds__(256) kbuild_simt_kernel(const float* __restric
                                                           const float* __restrict__ rn, const unsigned* maxr,
                                                           float expand_coef, int dot_expands) {
     __shared__ __align__(16) TileSmem sm;
+    grid_dependency_wait();
     const bool expand = KIND == POPCORN_GAUSSIAN && expansion_applies(rn, maxr, expand_coef);
     if (expand && dot_expands) return;
     if (expand)
@@ -432,6 +433,7 @@ __global__ void __launch_bounds__(128, 2) kbuild_dot_kernel(const float* __restr
                                                             float expand_coef, const SplitState* __restrict__ split,
                                                             long long tiles, int each) {
     __shared__ __align__(16) TileSmem sm;
+    grid_dependency_wait();
     if (split && split_taken(split)) return;   // the tensor-core build has written K
     if (KIND == kGaussExpand && !expansion_applies(rn, maxr, expand_coef)) return;
     const long long t0 = (long long)blockIdx.x * each;
@@ -514,24 +516,21 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
         const dim3 wgrid((unsigned)((tiles + each - 1) / each));
         switch (kp.kind) {
             case POPCORN_LINEAR:
-                kbuild_dot_kernel<POPCORN_LINEAR, PACKED><<<wgrid, dblock, 0, s>>>(
-                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles, (int)each);
-                return cudaGetLastError();
+                return launch_pdl(kbuild_dot_kernel<POPCORN_LINEAR, PACKED>, wgrid, dblock, 0, s, P, n, d, ldp, kp, K, ldk, kdiag,
+                                  T, full, rn, (const unsigned*)maxr, expand_coef, split, tiles, (int)each);
             case POPCORN_POLYNOMIAL:
-                kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED><<<wgrid, dblock, 0, s>>>(
-                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles, (int)each);
-                return cudaGetLastError();
+                return launch_pdl(kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED>, wgrid, dblock, 0, s, P, n, d, ldp, kp, K, ldk, kdiag,
+                                  T, full, rn, (const unsigned*)maxr, expand_coef, split, tiles, (int)each);
             default:
                 if (rn) {
-                    kbuild_dot_kernel<kGaussExpand, PACKED><<<wgrid, dblock, 0, s>>>(
-                        P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, split, tiles, (int)each);
-                    cudaError_t e = cudaGetLastError();
+                    const cudaError_t e = launch_pdl(kbuild_dot_kernel<kGaussExpand, PACKED>, wgrid, dblock, 0, s, P, n, d, ldp, kp,
+                                                     K, ldk, kdiag, T, full, rn, (const unsigned*)maxr, expand_coef, split,
+                                                     tiles, (int)each);
                     if (e != cudaSuccess) return e;
                     if (launches) ++*launches;
                 }
-                kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED><<<grid, block, 0, s>>>(
-                    P, n, d, ldp, kp, K, ldk, kdiag, T, full, rn, maxr, expand_coef, 1);
-                return cudaGetLastError();
+                return launch_pdl(kbuild_simt_kernel<POPCORN_GAUSSIAN, TK, PACKED>, grid, block, 0, s, P, n, d, ldp, kp, K, ldk,
+                                  kdiag, T, full, rn, (const unsigned*)maxr, expand_coef, 1);
         }
     }
     switch (kp.kind) {

@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                      const __grid_constant__ CUtensorMap map_kd, const __grid_constant__ CUtensorMap map_kt,
                      TcArgs a) {
     constexpr bool SPLIT = MODE == kModeSplit, X3 = MODE != kModeBf16;
+    grid_dependency_wait();                       // the operands come from the kernel before
     if (SPLIT && !split_taken(a.split)) return;   // the CUDA-core build takes this matrix
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -807,6 +808,8 @@ __global__ void __launch_bounds__(256) split_scan_kernel(const float* __restrict
                                                          const unsigned* maxr, float expand_coef, SplitState* st) {
     __shared__ unsigned cm[8][kScanCols];
     __shared__ int am_last;
+    // a Gaussian whose norm expansion does not apply: the state stays as it was cleared, not taken
+    if (!rowmax && !(__uint_as_float(*maxr) * expand_coef <= 1e-6f)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t r0 = (int64_t)blockIdx.x * rows, r1 = r0 + rows < n ? r0 + rows : n;
     const bool vec = (ldp & 3) == 0 && ((uintptr_t)P & 15) == 0;
@@ -871,6 +874,7 @@ __global__ void __launch_bounds__(256) split_scan_kernel(const float* __restrict
 // a row (float4 loads when rows are 16-byte aligned), 8-byte stores.
 __global__ void __launch_bounds__(256) split_operands_kernel(const float* __restrict__ P, int n, int d, int64_t ldp,
                                                              int dpad, SplitState* st, __half* __restrict__ W) {
+    grid_dependency_wait();
     if (!st->use) return;
     const float s = st->scale;
     unsigned low = 0u;
@@ -1026,8 +1030,7 @@ cudaError_t launch_tiles(int mode, const void* W, int n, int64_t ldw, int dpad, 
     a.stall = stall_ms > 0 && stall_ms <= 10000 ? 1 : 0;
     a.wait_ns = a.stall ? (unsigned long long)stall_ms * 1000000ull : kWaitLimitNs;
     const int grid = (int)(a.tiles < num_sms ? a.tiles : num_sms);
-    tc_fn(mode, out, kp.kind)<<<grid, NTHREADS, kSmemBytes, s>>>(mr, mc, mkd, mkt, a);
-    return cudaGetLastError();
+    return launch_pdl(tc_fn(mode, out, kp.kind), dim3(grid), dim3(NTHREADS), kSmemBytes, s, mr, mc, mkd, mkt, a);
 }
 
 int packed_out(int packed) { return packed == kPackedSw4 ? kOutSw4 : packed == kPackedSw16 ? kOutSw16 : kOutFull; }
@@ -1060,7 +1063,7 @@ cudaError_t launch_kbuild_tc(const float* P, int n, int d, int64_t ldp, KernPara
 }
 
 // Where the split build is the faster one.  The CUDA-core build takes its tiles in waves, each
-// as long as d; the split build costs four more launches (20 to 25 us, also where it refuses the
+// as long as d; the split build costs four more launches (15 to 20 us, also where it refuses the
 // points) and then a small fraction of that.  Measured (a whole call, us, CUDA cores / split): n = 2,000: d = 400 78 / 77,
 // 512 89 / 78, 784 109 / 91; n = 4,000: d = 128 91 / 88, 256 140 / 95; n = 6,000: d = 48 90 / 101,
 // 96 127 / 103; n = 8,000: d = 64 154 / 134, 784 953 / 266; n = 20,000: d = 48 609 / 441,
@@ -1103,9 +1106,9 @@ cudaError_t launch_kbuild_split(const float* P, int n, int d, int64_t ldp, KernP
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int64_t work = (int64_t)n * (dpad / 4);
     const int64_t blocks = (work + 255) / 256;
-    split_operands_kernel<<<(unsigned)(blocks < 16 * num_sms ? blocks : 16 * num_sms), 256, 0, s>>>(P, n, d, ldp, dpad,
-                                                                                                st, W);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_pdl(split_operands_kernel, dim3((unsigned)(blocks < 16 * num_sms ? blocks : 16 * num_sms)), dim3(256), 0, s,
+                   P, n, d, ldp, dpad, st, W);
+    if (e != cudaSuccess) return e;
     e = launch_tiles(kModeSplit, W, n, 2 * (int64_t)dpad, dpad, st, kp, rn, K, ldk, kdiag, err, num_sms, s,
                      packed_out(packed), full && !packed ? 1 : 0);
     if (launches) *launches += 3;
