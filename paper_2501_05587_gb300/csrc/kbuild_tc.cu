@@ -69,7 +69,7 @@
 //           (uniform: 0.6 to 1.3 here, 1.3 to 7.4 there).
 //           lo.lo is below an ulp, but on the diagonal it is a sum of squares: left out, J =
 //           trace K - ... of tight clusters is off by ten times that.
-//           Images, n = 70,000, d = 784: 10.9 ms (64.7 on CUDA cores); the operand loads allow
+//           Images, n = 70,000, d = 784: 10.5 ms (64.7 on CUDA cores); the operand loads allow
 //           8.4 (36 bytes a clock an SM), the MMAs 6.7, and the epilogue's stores (about 2 ms)
 //           are not overlapped: the next tile's MMAs run two chunks ahead.  n = 20,001,
 //           d = 1,000: 6.87 -> 1.33 ms a call.
@@ -187,7 +187,7 @@ long long tile_count(int T, int T2, int full) {
 // 128 elements a thread ran one after the other (about 300 clocks each, no overlap between
 // their chains), and it, not the MMAs, bounded every Gaussian build (images: 18.2 ms for
 // BF16 and BF16X3 alike; 4.9 and 7.9 ms with the kind a parameter and two epilogue
-// warpgroups, 4.2 and 7.8 now).
+// warpgroups, 3.9 and 7.1 now).
 template <int KIND>
 __device__ __forceinline__ float kappa(float b, float ri, float rj, const KernParams& kp) {
     if constexpr (KIND == POPCORN_LINEAR) return b;

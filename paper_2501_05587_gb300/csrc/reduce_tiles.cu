@@ -19,15 +19,15 @@
 //
 // What bounds it: the chain of a warp's shared-memory additions, with k x 512 bytes of sums a CTA
 // (2 CTAs an SM at k = 100, 3 at 64) to hide it behind; without the additions the stream takes
-// 0.49 ms where it takes 0.73 (k = 100, n = 30,011; HBM delivers 2.05 GB of the 3.6 GB square).
+// 0.49 ms where it takes 0.71 (k = 100, n = 30,011; HBM delivers 2.05 GB of the 3.6 GB square).
 // Two warps a row group, half a piece's columns each with sums of their own (16 consumer warps an
 // SM in place of 12 at k = 64, 8 in one CTA at 100), were slower: 142 -> 153 ms for the batch below
 // (30 passes), 27.0 -> 32.2 ms for 30 passes here.
 // So the labels come as byte offsets with the piece (the record below: no label arithmetic, no
 // global load) and four columns of different labels are added together.  The row-major stream it
 // replaces (iterate.cu: a lane every 32nd float4, k x 32 sums to add up a row, 15 instructions an
-// element) took 1.09 ms there, 0.81 at k = 64 (now 0.66), 0.79 at 40 (0.52) and 1.75 at 200
-// (1.36).  Batch of 256 instances, n 500 to 8,000, k up to 64: 4.7 -> 3.6 ms a pass.  A first form
+// element) took 1.09 ms there, 0.81 at k = 64 (now 0.63), 0.79 at 40 (0.51) and 1.75 at 200
+// (1.31).  Batch of 256 instances, n 500 to 8,000, k up to 64: 4.7 -> 3.6 ms a pass.  A first form
 // with 32 x 32 pieces of row-major rows (128 bytes at a 120 KB stride) stayed at 3.2 TB/s.
 //
 // Every so many column blocks a cluster's sums join the segment's, a pair of floats (Srun) until the
