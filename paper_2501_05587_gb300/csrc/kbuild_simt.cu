@@ -430,15 +430,13 @@ __global__ void __launch_bounds__(128, 2) kbuild_dot_kernel(const float* __restr
                                                             KernParams kp, float* __restrict__ K, int64_t ldk,
                                                             float* __restrict__ kdiag, int T, int full,
                                                             const float* __restrict__ rn, const unsigned* maxr,
-                                                            float expand_coef, const SplitState* __restrict__ split,
-                                                            long long tiles, int each) {
+                                                            float expand_coef, const SplitState* __restrict__ split) {
     __shared__ __align__(16) TileSmem sm;
     grid_dependency_wait();
     if (split && split_taken(split)) return;   // the tensor-core build has written K
     if (KIND == kGaussExpand && !expansion_applies(rn, maxr, expand_coef)) return;
-    const long long t0 = (long long)blockIdx.x * each;
-    for (long long t = t0; t < min(tiles, t0 + each); ++t)
-        kbuild_tile<KIND, float, false, PACKED, 16>(P, n, d, ldp, kp, K, ldk, kdiag, T, t, sm, full, rn);
+    kbuild_tile<KIND, float, false, PACKED, 16>(P, n, d, ldp, kp, K, ldk, kdiag, T, (long long)blockIdx.x, sm, full,
+                                                rn);
 }
 
 // d <= KC: the depth loop is one slice, so no next slice is held in registers;
@@ -506,26 +504,21 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
                                                       err, num_sms, s, launches, PACKED, full, &split);
             if (e != cudaSuccess) return e;
         }
-        // A dot-product launch that another kernel may have taken the work of has at most 512 blocks an
-        // SM, several consecutive tiles each from there (images: 150,000 empty blocks took 0.23 ms).
-        // Points the split refuses pay for it where a block's tiles are more than a few in 100 of what an
-        // SM's slots take in turn: linear, n = 30,000, d = 128, 2.68 ms without the split build, 2.70 so,
-        // 2.75 with at most 128 blocks an SM and 2.78 with 8; n = 20,000, d = 784 5.45, 5.45 and (8) 5.62.
-        const long long most = 512ll * num_sms;
-        const long long each = (split || rn) && num_sms > 0 && tiles > most ? (tiles + most - 1) / most : 1;
-        const dim3 wgrid((unsigned)((tiles + each - 1) / each));
+        // A tile a block, also where the split build may have taken the matrix (150,000 blocks that return at
+        // once: 0.23 ms of a 101 ms fit).  Blocks that loop over several tiles save that, and cost matrices
+        // that the split refuses 2 to 7%: a longer last wave, and 249 registers for 216 in the same loop
+        // (polynomial, 80% zeros, n = 30,000, d = 500 8.60 -> 8.99 ms, n = 12,000, d = 300 1.05 -> 1.13).
         switch (kp.kind) {
             case POPCORN_LINEAR:
-                return launch_pdl(kbuild_dot_kernel<POPCORN_LINEAR, PACKED>, wgrid, dblock, 0, s, P, n, d, ldp, kp, K, ldk, kdiag,
-                                  T, full, rn, (const unsigned*)maxr, expand_coef, split, tiles, (int)each);
+                return launch_pdl(kbuild_dot_kernel<POPCORN_LINEAR, PACKED>, grid, dblock, 0, s, P, n, d, ldp, kp, K, ldk, kdiag,
+                                  T, full, rn, (const unsigned*)maxr, expand_coef, split);
             case POPCORN_POLYNOMIAL:
-                return launch_pdl(kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED>, wgrid, dblock, 0, s, P, n, d, ldp, kp, K, ldk, kdiag,
-                                  T, full, rn, (const unsigned*)maxr, expand_coef, split, tiles, (int)each);
+                return launch_pdl(kbuild_dot_kernel<POPCORN_POLYNOMIAL, PACKED>, grid, dblock, 0, s, P, n, d, ldp, kp, K, ldk, kdiag,
+                                  T, full, rn, (const unsigned*)maxr, expand_coef, split);
             default:
                 if (rn) {
-                    const cudaError_t e = launch_pdl(kbuild_dot_kernel<kGaussExpand, PACKED>, wgrid, dblock, 0, s, P, n, d, ldp, kp,
-                                                     K, ldk, kdiag, T, full, rn, (const unsigned*)maxr, expand_coef, split,
-                                                     tiles, (int)each);
+                    const cudaError_t e = launch_pdl(kbuild_dot_kernel<kGaussExpand, PACKED>, grid, dblock, 0, s, P, n, d, ldp, kp,
+                                                     K, ldk, kdiag, T, full, rn, (const unsigned*)maxr, expand_coef, split);
                     if (e != cudaSuccess) return e;
                     if (launches) ++*launches;
                 }
