@@ -505,7 +505,7 @@ cudaError_t launch_simt_typed(const float* P, int n, int d, int64_t ldp, KernPar
             if (e != cudaSuccess) return e;
         }
         // A tile a block, also where the split build may have taken the matrix (150,000 blocks that return at
-        // once: 0.23 ms of a 101 ms fit).  Blocks that loop over several tiles save that, and cost matrices
+        // once: 0.13 ms of a 101 ms fit).  Blocks that loop over several tiles save that, and cost matrices
         // that the split refuses 2 to 7%: a longer last wave, and 249 registers for 216 in the same loop
         // (polynomial, 80% zeros, n = 30,000, d = 500 8.60 -> 8.99 ms, n = 12,000, d = 300 1.05 -> 1.13).
         switch (kp.kind) {
